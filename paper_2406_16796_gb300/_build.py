@@ -28,6 +28,7 @@ COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler",
 UNITS = {
     "api.cu": [],
     "kernels_general.cu": ["--fmad=false"],
+    "kernels_staged.cu": ["--fmad=false"],
     "kernels_diag.cu": [],
     "kernels_init.cu": [],
     "kernels_fused.cu": [],

@@ -618,7 +618,11 @@ static axp_status run_steps(axp_grid *g, int64_t nsteps)
     }
     if (!handled) {
         e = ensure_integer(g);
-        if (e == cudaSuccess) e = is_fp32(g) ? general_step<float>(g, nsteps) : general_step<double>(g, nsteps);
+        // AUTO: the folded multi-pass kernels; forced GENERAL: the literal ones.  (An
+        // attached but empty particle set keeps the literal kernels' bits.)
+        const bool staged = g->kernel_choice == AXP_KERNEL_AUTO && staged_supported(g) && !(g->parts && g->parts->count == 0);
+        if (e == cudaSuccess && staged) e = is_fp32(g) ? staged_step<float>(g, nsteps) : staged_step<double>(g, nsteps);
+        else if (e == cudaSuccess) e = is_fp32(g) ? general_step<float>(g, nsteps) : general_step<double>(g, nsteps);
     } else {
         e = cudaSuccess;
     }

@@ -202,6 +202,10 @@ View<T> make_view_eset(axp_grid *g, int eset);
 // launchers implemented in the .cu files (return cudaGetLastError())
 template <typename T>
 cudaError_t general_step(axp_grid *g, int64_t nsteps);
+// the folded multi-pass step on the state as it stands (integer time or staggered)
+template <typename T>
+cudaError_t staged_step(axp_grid *g, int64_t nsteps);
+bool staged_supported(const axp_grid *g);
 template <typename T>
 cudaError_t general_current(axp_grid *g);  // J^n of the present state
 template <typename T>

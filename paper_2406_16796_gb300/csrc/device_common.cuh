@@ -213,6 +213,55 @@ __device__ __forceinline__ T source_at(const View<T> &v, int64_t i, int64_t j, i
     return v.g * s;
 }
 
+// P_a = (D_t phi) Bbar0_a - (Ebar0 x grad_c phi)_a at one cell centre, (a, b, c) cyclic.
+template <typename T, bool INCR>
+__device__ T p_comp(const View<T> &v, const PhiPair<T, INCR> &q, int a, int64_t i, int64_t j, int64_t k)
+{
+    const int b = (a + 1) % 3, c = (a + 2) % 3;
+    int64_t ub[3], uc[3];
+    unit(b, ub);
+    unit(c, uc);
+    T mid, Dt;
+    phi_mid_dt<T, INCR>(v, q, i, j, k, &mid, &Dt);
+    const T dphi_c = over_2d(v,
+                             phi_mid<T, INCR>(v, q, i + uc[0], j + uc[1], k + uc[2]) -
+                                 phi_mid<T, INCR>(v, q, i - uc[0], j - uc[1], k - uc[2]),
+                             c);
+    const T dphi_b = over_2d(v,
+                             phi_mid<T, INCR>(v, q, i + ub[0], j + ub[1], k + ub[2]) -
+                                 phi_mid<T, INCR>(v, q, i - ub[0], j - ub[1], k - ub[2]),
+                             b);
+    const T cross = e0_bar(v, b, i, j, k) * dphi_c - e0_bar(v, c, i, j, k) * dphi_b;
+    return Dt * b0_bar(v, a, i, j, k) - cross;
+}
+
+// Outflow ghost t of one face at the new level (Sec. 2.4 item 3): solve the
+// one-way wave equation and the wave equation at the ghost for
+// V = phi^{cur}_{-3/2} and U = phi^{new}_{-1/2}.  Both equations involve only the
+// fields at n+1/2 and the levels before the update.
+template <typename T>
+__device__ __forceinline__ void outflow_ghost_at(const View<T> &v, int ax, int side, int64_t t, const T *g_cur,
+                                                 const T *g_old, T *g_new)
+{
+    const int b = (ax + 1) % 3, cc = (ax + 2) % 3;
+    const int64_t nb = v.n[b];
+    const T r = v.dt / v.d[ax];
+    const T r2 = (v.dt * v.dt) / (v.d[ax] * v.d[ax]);
+    int64_t ca[3];
+    ca[b] = t % nb;
+    ca[cc] = t / nb;
+    ca[ax] = side ? v.n[ax] : -1;
+    const int64_t pi = ax == 0 ? ca[1] + v.n[1] * ca[2] : (ax == 1 ? ca[0] + v.n[0] * ca[2] : ca[0] + v.n[0] * ca[1]);
+    const T Sg = source_at(v, ca[0], ca[1], ca[2]);
+    int64_t ci[3] = {ca[0], ca[1], ca[2]};
+    ci[ax] = side ? v.n[ax] - 1 : 0;
+    const T p0 = v.phi_cur[lin3(v.n, ci[0], ci[1], ci[2])];
+    const T gc = g_cur[pi], go = g_old[pi];
+    const T rhs = T(-2) * gc + T(2) * go - (v.dt * v.dt) * (Sg - v.m2 * gc) + r * p0 - r2 * (p0 - T(2) * gc);
+    const T V = rhs / (r + r2);
+    g_new[pi] = go + r * (p0 - V);
+}
+
 template <typename T>
 __device__ __forceinline__ T sigma_of(const T *const tab[3], int64_t i, int64_t j, int64_t k)
 {

@@ -843,6 +843,8 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     const int set = pick_set(g);
     cudaError_t e = enter_staggered<T>(g);
     if (e != cudaSuccess) return e;
+    if (path == AXP_KERNEL_FUSED && g->kernel_choice == AXP_KERNEL_AUTO && mode >= 2 && staged_supported(g))
+        return staged_step<T>(g, nsteps);
     int tm_tx = tm2d::TX;  // tile width of the 2D kernel (chosen below)
     // FP32 split on an even-width grid without a soft source: the two-column form
     const bool x2 = tm && tm2d_x2_eligible<T>(g);

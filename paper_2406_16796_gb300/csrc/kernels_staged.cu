@@ -1,0 +1,680 @@
+// kernels_staged.cu -- the multi-pass step with folded arithmetic (arXiv 2406.16796
+// Sec. 2.3-2.4), for the grids that no specialised single-pass kernel takes:
+// outflow sides, a uniform E, FP64 3D, macroparticles, lasers outside the TM set.
+//
+// What bounds it: on GB300 an FP64 step is bound by the FP64 pipe (2 operations
+// per cycle per SM), so each quantity is formed once and every constant is folded;
+// an FP32 step by memory and launch latency.  The literal kernels
+// (kernels_general.cu) take 8 launches and about 400 FP64 operations per 3D cell
+// (their divisions included); these take 4 launches and 143:
+//   B      B^{n+1} of both orders; B0^{n+1/2} is kept in scratch
+//   phi    S and phi^{n+3/2}; E0^{n+1} (to scratch) and E0^{n+3/2}
+//   P      the axion current's P at the cell centres
+//   J      J, E1^{n+1} and E1^{n+3/2}
+// With macroparticles the B pass is two half passes around the push and the E0
+// update a pass of its own.  One thread per cell, neighbours through L1/L2 by
+// offsets that already hold the wrap, the closure of non-periodic sides as
+// predicated loads: no branch over cells but the absorbing layer's.
+//
+// Only active axes and order-0 components that can be non-zero are computed (template
+// arguments).  Field sets alternate: the step reads one and writes the other.
+//
+// The E half-steps of one step and of the next read the same X = curl B - g J, so
+// both are taken at once, but as two updates by the same increment: a run cut into
+// several calls then gives the bits of the uncut one.  Multiply-adds are written
+// out and the unit is compiled without contraction, for the same reason.
+//
+// Measured on one GB300, against the literal kernels (us per step):
+//   2D TM laser, outflow axion sides, FP64, 1024 x 512:  STAGED_OUTFLOW
+//   3D laser, absorbing x sides, FP64, 160 x 96 x 96:    STAGED_LASER3D
+#include <algorithm>
+
+#include "device_common.cuh"
+
+namespace axp {
+namespace {
+
+constexpr int kThreads = 256;
+
+template <typename T>
+struct Stage {
+    const T *Ein[6], *Bin[6];  // E^{n+1/2}, B^n (order 0 xyz, order 1 xyz)
+    T *Eout[6], *Bout[6];
+    T *Bh[3];  // scratch: B0^{n+1/2}
+    T *Eh[3];  // scratch: E0^{n+1}
+    T *P[3], *J[3];
+    const T *phi, *phib;  // phi^{n+1/2}; phi^{n-1/2} (FP64) or the increment (FP32 split)
+    T *phi_out, *phib_out;
+    const T *jp[2][3];                  // macroparticle currents (null without)
+    const T *gh[3][2], *gh_hi[3][2];    // outflow ghosts of phi^{n+1/2} and phi^{n+3/2}
+    const T *tab[3];                    // layer coefficients per axis (null: no layer)
+    const T *sig_ax[3];
+    int n[3], per[3], axbc[3][2];
+    int N;
+    T hd[3];              // h/d
+    T inv_h, h;
+    T hg2;                // h g / 2: J is used as the sum of two P
+    T lap_c[3], lap_0, dt2g, dt, inv_dt, q4d[3];
+    T Bext[3], Eext[3];
+    int src_x;            // x index of the soft source's E cells (-1: none)
+    const T *src_w[2];
+    T src_e, src_b;       // h tau of the electric and of the magnetic sheet
+    int last;             // the step ends at integer time (only the first E half-step)
+};
+
+// A cell's index, its neighbours' (wrapped along periodic axes) and whether they exist.
+struct Cell {
+    int c, x[3];
+    int up[3], dn[3];
+    bool hu[3], hd[3];
+};
+
+template <int MASK, typename T>
+__device__ __forceinline__ bool cell_at(const Stage<T> &s, Cell &q)
+{
+    const unsigned c = blockIdx.x * (unsigned)kThreads + threadIdx.x;
+    if (c >= (unsigned)s.N) return false;
+    const unsigned n0 = s.n[0], n1 = s.n[1];
+    const unsigned r = c / n0;
+    q.c = (int)c;
+    q.x[0] = (int)(c - r * n0);
+    q.x[1] = (MASK & 4) ? (int)(r % n1) : (int)r;
+    q.x[2] = (MASK & 4) ? (int)(r / n1) : 0;
+    const int stride[3] = {1, s.n[0], s.n[0] * s.n[1]};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        q.up[a] = q.dn[a] = q.c;
+        q.hu[a] = q.hd[a] = true;
+        if (!(MASK >> a & 1)) continue;
+        const int wrap = (s.n[a] - 1) * stride[a];
+        if (q.x[a] + 1 < s.n[a]) q.up[a] = q.c + stride[a];
+        else { q.up[a] = q.c - wrap; q.hu[a] = s.per[a]; }
+        if (q.x[a] > 0) q.dn[a] = q.c - stride[a];
+        else { q.dn[a] = q.c + wrap; q.hd[a] = s.per[a]; }
+    }
+    return true;
+}
+
+template <typename T>
+__device__ __forceinline__ T ldz(const T *__restrict__ F, int c, bool ok)
+{
+    return ok ? F[c] : T(0);
+}
+
+// h (curl F)_a with differences towards `up` (forward) or from `dn` (backward):
+// hb (dF_c along b) - hc (dF_b along c), without the terms of inactive axes and
+// of components that are zero (CM: mask of the components present).
+template <int MASK, int CM, bool FWD, typename T>
+__device__ __forceinline__ T curl_h(const Stage<T> &s, const T *const F[3], int a, const Cell &q)
+{
+    const int b = (a + 1) % 3, c = (a + 2) % 3;
+    const bool t1 = (MASK >> b & 1) && (CM >> c & 1), t2 = (MASK >> c & 1) && (CM >> b & 1);
+    T d1 = T(0), d2 = T(0);
+    if (t1) d1 = FWD ? ldz(F[c], q.up[b], q.hu[b]) - F[c][q.c] : F[c][q.c] - ldz(F[c], q.dn[b], q.hd[b]);
+    if (t2) d2 = FWD ? ldz(F[b], q.up[c], q.hu[c]) - F[b][q.c] : F[b][q.c] - ldz(F[b], q.dn[c], q.hd[c]);
+    if (t1 && t2) return fma(s.hd[b], d1, -(s.hd[c] * d2));
+    if (t1) return s.hd[b] * d1;
+    if (t2) return -(s.hd[c] * d2);
+    return T(0);
+}
+
+// The absorbing layer at a cell: a half-step is F <- a F + r (h X), a = 1 and r = 1
+// outside the layers; both decrease with sigma, so a corner takes the smallest.
+template <typename T>
+struct Layer {
+    T a, r;
+    bool in;
+};
+template <int MASK, typename T>
+__device__ __forceinline__ Layer<T> layer_at(const Stage<T> &s, const Cell &q)
+{
+    Layer<T> L{T(1), T(1), false};
+    T b = s.h;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (!(MASK >> a & 1) || !s.tab[a]) continue;
+        const T ta = s.tab[a][q.x[a]];
+        if (ta < L.a) {
+            L.a = ta;
+            b = s.tab[a][s.n[a] + q.x[a]];
+            L.in = true;
+        }
+    }
+    if (L.in) L.r = b * s.inv_h;
+    return L;
+}
+template <typename T>
+__device__ __forceinline__ T half_step(const Layer<T> &L, T F, T hX)
+{
+    return L.in ? fma(L.a, F, L.r * hX) : F + hX;
+}
+
+// MODE 0: the full B step (B0^{n+1/2} to scratch); 1 and 2: one half-step from Bin
+// to Bout (with macroparticles; the second in place).
+template <typename T, int MASK, int EM, int BM, int MODE>
+__global__ void __launch_bounds__(kThreads) k_stage_b(Stage<T> s)
+{
+    Cell q;
+    if (!cell_at<MASK>(s, q)) return;
+    const Layer<T> L = layer_at<MASK>(s, q);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (!(BM >> a & 1)) continue;
+        T hX = -curl_h<MASK, EM, true>(s, s.Ein, a, q);
+        if (a > 0 && q.x[0] == s.src_x - 1) {
+            const int jk = q.x[1] + s.n[1] * q.x[2];
+            hX = a == 1 ? fma(-s.src_w[1][jk], s.src_b, hX) : fma(s.src_w[0][jk], s.src_b, hX);
+        }
+        const T Bh = half_step(L, s.Bin[a][q.c], hX);
+        if (MODE == 0) {
+            s.Bh[a][q.c] = Bh;
+            s.Bout[a][q.c] = half_step(L, Bh, hX);
+        } else {
+            s.Bout[a][q.c] = Bh;
+        }
+    }
+    const T *const E1[3] = {s.Ein[3], s.Ein[4], s.Ein[5]};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const T hX = -curl_h<MASK, 7, true>(s, E1, a, q), B = s.Bin[3 + a][q.c];
+        T r = half_step(L, B, hX);
+        if (MODE == 0) r = L.in ? half_step(L, r, hX) : fma(T(2), hX, B);
+        s.Bout[3 + a][q.c] = r;
+    }
+}
+
+// 2-point average of E0_a at the cell centre plus the background
+template <int MASK, int EM, typename T>
+__device__ __forceinline__ T ebar(const Stage<T> &s, const T *const E[3], int a, const Cell &q)
+{
+    if (!(EM >> a & 1)) return s.Eext[a];
+    const T f = E[a][q.c];
+    if (!(MASK >> a & 1)) return f + s.Eext[a];
+    return fma(T(0.5), f + ldz(E[a], q.dn[a], q.hd[a]), s.Eext[a]);
+}
+
+// 4-point average of B0_a at the cell centre plus the background
+template <int MASK, int BM, typename T>
+__device__ __forceinline__ T bbar(const Stage<T> &s, const T *const B[3], int a, const Cell &q)
+{
+    if (!(BM >> a & 1)) return s.Bext[a];
+    const int b = (a + 1) % 3, c = (a + 2) % 3;
+    const bool mb = MASK >> b & 1, mc = MASK >> c & 1;
+    T f = B[a][q.c], w = T(1);
+    if (mb) {
+        f = f + ldz(B[a], q.dn[b], q.hd[b]);
+        w = T(0.5);
+    }
+    if (mc) {
+        T g = ldz(B[a], q.dn[c], q.hd[c]);
+        if (mb) g = g + ldz(B[a], q.dn[b] + (q.dn[c] - q.c), q.hd[b] && q.hd[c]);
+        f = f + g;
+        w = w * T(0.5);
+    }
+    return fma(w, f, s.Bext[a]);
+}
+
+// Neighbour of an axion level along axis a: inside the grid, by the boundary beyond it
+// (periodic wrap, reflect: the cell itself, outflow: the ghost plane, PML: 0).
+template <typename T>
+__device__ __forceinline__ T phi_nb(const Stage<T> &s, const T *__restrict__ F, const T *const gh[3][2], int a, int side,
+                                    const Cell &q)
+{
+    if (side ? q.hu[a] : q.hd[a]) return F[side ? q.up[a] : q.dn[a]];
+    const int bc = s.axbc[a][side];
+    if (bc == AXP_BC_REFLECT) return F[q.c];
+    if (bc != AXP_BC_OUTFLOW) return T(0);
+    const int pi = a == 0 ? q.x[1] + s.n[1] * q.x[2] : (a == 1 ? q.x[0] + s.n[0] * q.x[2] : q.x[0] + s.n[0] * q.x[1]);
+    return gh[a][side][pi];
+}
+
+// E0 from E0^{n+1/2}: E0^{n+1} to scratch and, unless the step ends at integer time,
+// E0^{n+3/2} to the output set.
+template <typename T, int MASK, int EM, int BM>
+__device__ __forceinline__ void e0_update(const Stage<T> &s, const Cell &q, const Layer<T> &L)
+{
+    const T *const B0[3] = {s.Bout[0], s.Bout[1], s.Bout[2]};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (!(EM >> a & 1)) continue;
+        T hX = curl_h<MASK, BM, false>(s, B0, a, q);
+        if (a > 0 && q.x[0] == s.src_x) hX = fma(s.src_w[a - 1][q.x[1] + s.n[1] * q.x[2]], s.src_e, hX);
+        if (s.jp[0][a]) hX = fma(-s.h, s.jp[0][a][q.c], hX);
+        const T E = half_step(L, s.Ein[a][q.c], hX);
+        s.Eh[a][q.c] = E;
+        s.Eout[a][q.c] = s.last ? E : half_step(L, E, hX);
+    }
+}
+
+// PHI: the axion leapfrog with its source; E0: the order-0 E update.  Bs: where
+// B0^{n+1/2} lies (the B pass's scratch, or Bout between the half passes).
+template <typename T, int MASK, int EM, int BM, bool PHI, bool E0>
+__global__ void __launch_bounds__(kThreads) k_stage_phi(Stage<T> s, const T *bs0, const T *bs1, const T *bs2)
+{
+    constexpr bool INCR = sizeof(T) == 4;
+    Cell q;
+    if (!cell_at<MASK>(s, q)) return;
+    if (PHI) {
+        const T *const Bs[3] = {bs0, bs1, bs2};
+        T S = T(0);
+#pragma unroll
+        for (int a = 0; a < 3; a++) S = fma(ebar<MASK, EM>(s, s.Ein, a, q), bbar<MASK, BM>(s, Bs, a, q), S);
+        const T ph = s.phi[q.c], old = s.phib[q.c];
+        T lap = s.dt2g * S;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            if (!(MASK >> a & 1)) continue;
+            const T up = phi_nb(s, s.phi, s.gh, a, 1, q), dn = phi_nb(s, s.phi, s.gh, a, 0, q);
+            // FP32 split: from neighbour differences, which do not round against 2 phi
+            lap = fma(s.lap_c[a], INCR ? (up - ph) + (dn - ph) : up + dn, lap);
+        }
+        lap = fma(s.lap_0, ph, lap);  // FP64: lap_0 holds the 2 phi of the leapfrog too
+        T sig = T(0);
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+            if ((MASK >> a & 1) && s.tab[a]) {
+                const T t = s.sig_ax[a][q.x[a]];
+                if (t > sig) sig = t;
+            }
+        if (INCR) {
+            T nin = lap + old;
+            if (sig != T(0)) {
+                const T sd = sig * s.dt;
+                nin = (fma(-(sd * sd), ph, lap) + (T(1) - sd) * old) / (T(1) + sd);
+            }
+            s.phib_out[q.c] = nin;
+            s.phi_out[q.c] = ph + nin;
+        } else {
+            T nw = lap - old;
+            if (sig != T(0)) {
+                const T sd = sig * s.dt;
+                nw = (fma(-(sd * sd), ph, lap) - (T(1) - sd) * old) / (T(1) + sd);
+            }
+            s.phi_out[q.c] = nw;
+        }
+    }
+    if (E0) e0_update<T, MASK, EM, BM>(s, q, layer_at<MASK>(s, q));
+}
+
+// P = (D_t phi) Bbar0 - Ebar0 x grad_c phi^{n+1} at the cell centres, from E0^{n+1}
+// (e0..e2) and B0^{n+1} (b0..b2); hi/lo: the axion levels around n+1 (lo the
+// increment in FP32 split).
+template <typename T, int MASK, int EM, int BM>
+__global__ void __launch_bounds__(kThreads) k_stage_p(Stage<T> s, const T *e0, const T *e1, const T *e2, const T *b0,
+                                                      const T *b1, const T *b2, const T *hi, const T *lo)
+{
+    constexpr bool INCR = sizeof(T) == 4;
+    Cell q;
+    if (!cell_at<MASK>(s, q)) return;
+    const T *const E[3] = {e0, e1, e2};
+    const T *const B[3] = {b0, b1, b2};
+    T g[3], e[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        g[a] = T(0);
+        e[a] = ebar<MASK, EM>(s, E, a, q);
+        if (!(MASK >> a & 1)) continue;
+        // 2 phi^{n+1} at the two neighbours: the sum of the levels (ghost planes hold
+        // levels, also in FP32 split, where the arrays hold phi and its increment)
+        T two[2];
+#pragma unroll
+        for (int side = 0; side < 2; side++) {
+            const bool in = side ? q.hu[a] : q.hd[a];
+            const T h = phi_nb(s, hi, s.gh_hi, a, side, q), l = phi_nb(s, lo, s.gh, a, side, q);
+            const bool incr = INCR && (in || s.axbc[a][side] == AXP_BC_REFLECT);
+            two[side] = incr ? fma(T(2), h, -l) : h + l;
+        }
+        g[a] = s.q4d[a] * (two[1] - two[0]);
+    }
+    const T l = lo[q.c];
+    const T Dt = (INCR ? l : hi[q.c] - l) * s.inv_dt;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const int b = (a + 1) % 3, c = (a + 2) % 3;
+        T p = Dt * bbar<MASK, BM>(s, B, a, q);
+        if (MASK >> c & 1) p = fma(-e[b], g[c], p);
+        if (MASK >> b & 1) p = fma(e[c], g[b], p);
+        s.P[a][q.c] = p;
+    }
+}
+
+// J = (P(c) + P(c + a)) / 2 and the order-1 E update; CURRENT: only J.  Beyond the
+// last cell of a non-periodic axis P follows the ghost rules: 0 at a PML side without
+// a uniform E, else evaluated in place (one cell per row or plane).
+template <typename T, int MASK, bool CURRENT>
+__global__ void __launch_bounds__(kThreads) k_stage_j(Stage<T> s, View<T> v, PhiPair<T, sizeof(T) == 4> pq)
+{
+    Cell q;
+    if (!cell_at<MASK>(s, q)) return;
+    const bool ext = s.Eext[0] != T(0) || s.Eext[1] != T(0) || s.Eext[2] != T(0);
+    T J2[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const T p0 = s.P[a][q.c];
+        T p1 = p0;
+        if (MASK >> a & 1) {
+            if (q.hu[a]) p1 = s.P[a][q.up[a]];
+            else if (s.axbc[a][1] == AXP_BC_PML && !ext) p1 = T(0);
+            else
+                p1 = p_comp<T, sizeof(T) == 4>(v, pq, a, q.x[0] + (a == 0), q.x[1] + (a == 1), q.x[2] + (a == 2));
+        }
+        J2[a] = p0 + p1;
+        if (CURRENT || s.last) s.J[a][q.c] = T(0.5) * J2[a];
+    }
+    if (CURRENT) return;
+    const Layer<T> L = layer_at<MASK>(s, q);
+    const T *const B1[3] = {s.Bout[3], s.Bout[4], s.Bout[5]};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        T hX = fma(-s.hg2, J2[a], curl_h<MASK, 7, false>(s, B1, a, q));
+        if (s.jp[1][a]) hX = fma(-s.h, s.jp[1][a][q.c], hX);
+        T E = half_step(L, s.Ein[3 + a][q.c], hX);
+        if (!s.last) E = half_step(L, E, hX);
+        s.Eout[3 + a][q.c] = E;
+    }
+}
+
+// The first E half-step of a run that starts at integer time, in place, with the J
+// of the present state (the same increments as the step's own half-steps).
+template <typename T, int MASK, int EM, int BM>
+__global__ void __launch_bounds__(kThreads) k_stage_e_half(Stage<T> s)
+{
+    Cell q;
+    if (!cell_at<MASK>(s, q)) return;
+    const Layer<T> L = layer_at<MASK>(s, q);
+    const T *const B1[3] = {s.Bin[3], s.Bin[4], s.Bin[5]};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (EM >> a & 1) {
+            T hX = curl_h<MASK, BM, false>(s, s.Bin, a, q);
+            if (a > 0 && q.x[0] == s.src_x) hX = fma(s.src_w[a - 1][q.x[1] + s.n[1] * q.x[2]], s.src_e, hX);
+            if (s.jp[0][a]) hX = fma(-s.h, s.jp[0][a][q.c], hX);
+            T *E = const_cast<T *>(s.Ein[a]);
+            E[q.c] = half_step(L, E[q.c], hX);
+        }
+        T hX = fma(-s.hg2, T(2) * s.J[a][q.c], curl_h<MASK, 7, false>(s, B1, a, q));
+        if (s.jp[1][a]) hX = fma(-s.h, s.jp[1][a][q.c], hX);
+        T *E = const_cast<T *>(s.Ein[3 + a]);
+        E[q.c] = half_step(L, E[q.c], hX);
+    }
+}
+
+// every outflow face's ghosts in one launch (blockIdx.y: the face)
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_stage_outflow(View<T> v)
+{
+    int f = (int)blockIdx.y, ax = 0, side = 0;
+    for (int a = 0; a < 3; a++)
+        for (int e = 0; e < 2; e++)
+            if (v.axbc[a][e] == AXP_BC_OUTFLOW && f-- == 0) {
+                ax = a;
+                side = e;
+            }
+    const int64_t plane = v.n[(ax + 1) % 3] * v.n[(ax + 2) % 3];
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < plane; t += (int64_t)gridDim.x * blockDim.x)
+        outflow_ghost_at(v, ax, side, t, v.gh[ax][side][0], v.gh[ax][side][1], v.gh[ax][side][2]);
+}
+
+template <typename T>
+Stage<T> make_stage(axp_grid *g)
+{
+    Stage<T> s;
+    const axp_grid_desc &d = g->desc;
+    const Workspace &w = g->layout;
+    const int in = g->fset, out = 1 - g->fset;
+    auto at = [&](size_t off) { return (T *)(g->ws + off); };
+    for (int q = 0; q < 6; q++) {
+        const int fe = q < 3 ? kE0 + q : kE1 + (q - 3), fb = q < 3 ? kB0 + q : kB1 + (q - 3);
+        s.Ein[q] = at(w.off_fields[in][fe]);
+        s.Bin[q] = at(w.off_fields[in][fb]);
+        s.Eout[q] = at(w.off_fields[out][fe]);
+        s.Bout[q] = at(w.off_fields[out][fb]);
+    }
+    s.phi = at(w.off_phi[g->phi_cur_slot]);
+    s.phib = at(w.off_phi[g->phi_b_slot]);
+    s.phi_out = at(w.off_phi[g->phi_next_slot]);
+    s.phib_out = sizeof(T) == 4 ? at(w.off_phi[g->phi_next_b_slot]) : nullptr;
+    const double h = d.dt / 2.0;
+    double idd = 0.0;
+    for (int a = 0; a < 3; a++) {
+        s.Bh[a] = s.P[a] = at(w.off_P[a]);
+        s.Eh[a] = s.J[a] = at(w.off_J[a]);
+        for (int o = 0; o < 2; o++)
+            s.jp[o][a] = g->parts && sizeof(T) == sizeof(double) ? (const T *)g->parts->j[o][a] : nullptr;
+        bool layer = false;
+        for (int e = 0; e < 2; e++) {
+            const size_t cur = w.off_ghost[a][e][g->ghost_level_slot[0]], nxt = w.off_ghost[a][e][g->ghost_level_slot[2]];
+            s.gh[a][e] = cur ? at(cur) : nullptr;
+            s.gh_hi[a][e] = nxt ? at(nxt) : nullptr;
+            s.axbc[a][e] = d.axion_bc[a][e];
+            if (d.em_bc[a][e] == AXP_BC_PML || d.axion_bc[a][e] == AXP_BC_PML) layer = true;
+        }
+        s.tab[a] = layer && d.pml_cells > 0 && d.pml_sigma_max_dt > 0 ? at(w.off_pml_tab[a]) : nullptr;
+        s.sig_ax[a] = at(w.off_sig_ax[a]);
+        s.n[a] = (int)d.n[a];
+        s.per[a] = d.em_bc[a][0] == AXP_BC_PERIODIC;
+        s.hd[a] = (T)(h / d.d[a]);
+        s.lap_c[a] = d.n[a] > 1 ? (T)(d.dt * d.dt / (d.d[a] * d.d[a])) : T(0);
+        s.q4d[a] = (T)(0.25 / d.d[a]);
+        if (d.n[a] > 1) idd += 1.0 / (d.d[a] * d.d[a]);
+        s.Bext[a] = (T)g->B_ext[a];
+        s.Eext[a] = (T)g->E_ext[a];
+    }
+    s.N = (int)(d.n[0] * d.n[1] * d.n[2]);
+    s.h = (T)h;
+    s.inv_h = (T)(1.0 / h);
+    s.hg2 = (T)(0.5 * h * d.g);
+    s.lap_0 = (T)(sizeof(T) == 4 ? -d.dt * d.dt * d.m * d.m : 2.0 - d.dt * d.dt * (d.m * d.m + 2.0 * idd));
+    s.dt2g = (T)(d.dt * d.dt * d.g);
+    s.dt = (T)d.dt;
+    s.inv_dt = (T)(1.0 / d.dt);
+    s.src_x = -1;
+    s.src_w[0] = at(w.off_src[0]);
+    s.src_w[1] = at(w.off_src[1]);
+    s.src_e = s.src_b = T(0);
+    if (g->src_on) s.src_x = (int)g->src.plane;
+    s.last = 0;
+    return s;
+}
+
+// Launches of one configuration: active axes MASK, order-0 components EM and BM.
+template <typename T, int MASK, int EM, int BM>
+struct Passes {
+    static int blocks(const Stage<T> &s) { return (s.N + kThreads - 1) / kThreads; }
+    static void b(const Stage<T> &s, int mode, cudaStream_t st)
+    {
+        if (mode == 0) k_stage_b<T, MASK, EM, BM, 0><<<blocks(s), kThreads, 0, st>>>(s);
+        else if (mode == 1) k_stage_b<T, MASK, EM, BM, 1><<<blocks(s), kThreads, 0, st>>>(s);
+        else k_stage_b<T, MASK, EM, BM, 2><<<blocks(s), kThreads, 0, st>>>(s);
+    }
+    static void phi(const Stage<T> &s, T *const bs[3], int part, cudaStream_t st)
+    {
+        if (part == 3) k_stage_phi<T, MASK, EM, BM, true, true><<<blocks(s), kThreads, 0, st>>>(s, bs[0], bs[1], bs[2]);
+        else if (part == 1)
+            k_stage_phi<T, MASK, EM, BM, true, false><<<blocks(s), kThreads, 0, st>>>(s, bs[0], bs[1], bs[2]);
+        else
+            k_stage_phi<T, MASK, EM, BM, false, true><<<blocks(s), kThreads, 0, st>>>(s, bs[0], bs[1], bs[2]);
+    }
+    static void p(const Stage<T> &s, const T *const e[3], const T *const b[3], const T *hi, const T *lo, cudaStream_t st)
+    {
+        k_stage_p<T, MASK, EM, BM><<<blocks(s), kThreads, 0, st>>>(s, e[0], e[1], e[2], b[0], b[1], b[2], hi, lo);
+    }
+    static void j(const Stage<T> &s, const View<T> &v, const PhiPair<T, sizeof(T) == 4> &pq, bool current, cudaStream_t st)
+    {
+        if (current) k_stage_j<T, MASK, true><<<blocks(s), kThreads, 0, st>>>(s, v, pq);
+        else k_stage_j<T, MASK, false><<<blocks(s), kThreads, 0, st>>>(s, v, pq);
+    }
+    static void e_half(const Stage<T> &s, cudaStream_t st)
+    {
+        k_stage_e_half<T, MASK, EM, BM><<<blocks(s), kThreads, 0, st>>>(s);
+    }
+};
+
+// Ghost planes of an axion level as the boundary-aware accessors take them.
+template <typename T>
+Ghosts<T> ghost_planes(axp_grid *g, int level)
+{
+    Ghosts<T> G;
+    for (int a = 0; a < 3; a++)
+        for (int e = 0; e < 2; e++) {
+            const size_t off = g->layout.off_ghost[a][e][g->ghost_level_slot[level]];
+            G.p[a][e] = off ? (T *)(g->ws + off) : nullptr;
+        }
+    return G;
+}
+
+template <typename T, typename Q, int EM, int BM>
+cudaError_t run_staged(axp_grid *g, int64_t nsteps)
+{
+    const axp_grid_desc &d = g->desc;
+    const bool stag = g->staggered;  // the single-pass kernels' state: E stays half a step ahead
+    int faces = 0;  // outflow faces
+    int64_t plane = 0;
+    for (int a = 0; a < 3; a++)
+        for (int e = 0; e < 2; e++)
+            if (d.axion_bc[a][e] == AXP_BC_OUTFLOW) {
+                faces++;
+                plane = std::max<int64_t>(plane, d.n[(a + 1) % 3] * d.n[(a + 2) % 3]);
+            }
+    const bool parts = g->parts != nullptr;
+    bool ahead = stag;  // E at n+1/2
+    cudaError_t e = cudaSuccess;
+    for (int64_t it = 0; it < nsteps; it++) {
+        const bool record = d.diag_every > 0 && (g->step + 1) % d.diag_every == 0;
+        if (!ahead) {
+            if (!g->J_valid) {
+                // the P pass reads ghosts of n+1/2 and n-1/2 here
+                const int s0 = g->ghost_level_slot[0], s1 = g->ghost_level_slot[1], s2 = g->ghost_level_slot[2];
+                g->ghost_level_slot[2] = s0;
+                g->ghost_level_slot[0] = s1;
+                const Stage<T> s = make_stage<T>(g);
+                g->ghost_level_slot[0] = s0;
+                g->ghost_level_slot[2] = s2;
+                View<T> v = make_view<T>(g);
+                const T *const b[3] = {s.Bin[0], s.Bin[1], s.Bin[2]};
+                Q::p(s, s.Ein, b, s.phi, s.phib, g->stream);
+                PhiPair<T, sizeof(T) == 4> pq{s.phi, s.phib, ghost_planes<T>(g, 0), ghost_planes<T>(g, 1)};
+                Q::j(s, v, pq, true, g->stream);
+                g->launches += 2;
+            }
+            Stage<T> s = make_stage<T>(g);
+            if (g->src_on) s.src_e = (T)(d.dt / 2.0 * source_wave(g, source_x_b(g), time_n(g, g->step)));
+            Q::e_half(s, g->stream);
+            g->launches++;
+            ahead = true;
+        }
+        Stage<T> s = make_stage<T>(g);
+        s.last = !stag && (it + 1 == nsteps || record);
+        if (g->src_on) {
+            s.src_b = (T)(d.dt / 2.0 * source_wave(g, source_x_e(g), time_half(g, g->step)));
+            s.src_e = (T)(d.dt / 2.0 * source_wave(g, source_x_b(g), time_n(g, g->step + 1)));
+        }
+        // outflow ghosts at the new level, from the fields at n+1/2 (bh: where B0^{n+1/2} lies)
+        auto outflow_ghosts = [&](T *const bh[3]) {
+            if (faces == 0) return;
+            View<T> v = make_view<T>(g);
+            for (int a = 0; a < 3; a++) v.f[kB0 + a] = (BM >> a & 1) ? bh[a] : s.Bout[a];
+            const dim3 grid((unsigned)std::min<int64_t>((plane + kThreads - 1) / kThreads, 1024), (unsigned)faces);
+            k_stage_outflow<T><<<grid, kThreads, 0, g->stream>>>(v);
+            g->launches++;
+        };
+        if constexpr (sizeof(T) == sizeof(double)) {
+            if (parts) {
+                Q::b(s, 1, g->stream);
+                outflow_ghosts(s.Bout);
+                View<double> v = make_view<double>(g);
+                for (int a = 0; a < 3; a++) {
+                    v.f[kB0 + a] = s.Bout[a];
+                    v.f[kB1 + a] = s.Bout[3 + a];
+                }
+                if ((e = particles_push(g, v)) != cudaSuccess) return e;
+                Q::phi(s, s.Bout, 1, g->stream);
+                Stage<double> s2 = s;
+                for (int f = 0; f < 6; f++) s2.Bin[f] = s.Bout[f];
+                Q::b(s2, 2, g->stream);
+                Q::phi(s, s.Bh, 2, g->stream);
+                g->launches += 4;
+            }
+        }
+        if (!parts) {
+            Q::b(s, 0, g->stream);
+            outflow_ghosts(s.Bh);
+            Q::phi(s, s.Bh, 3, g->stream);
+            g->launches += 2;
+        }
+        const T *hi = s.phi_out, *lo = sizeof(T) == 4 ? s.phib_out : s.phi;
+        const T *const b[3] = {s.Bout[0], s.Bout[1], s.Bout[2]};
+        const T *eh[3];
+        View<T> v = make_view<T>(g);
+        for (int a = 0; a < 3; a++) {
+            eh[a] = (EM >> a & 1) ? s.Eh[a] : s.Eout[a];  // (an inactive array is zero in both sets)
+            v.f[kE0 + a] = const_cast<T *>(eh[a]);
+            v.f[kB0 + a] = s.Bout[a];
+        }
+        if (s.last) {  // E0^{n+1} lies in the output set too, and J takes the scratch
+            for (int a = 0; a < 3; a++) {
+                eh[a] = s.Eout[a];
+                v.f[kE0 + a] = s.Eout[a];
+            }
+        }
+        Q::p(s, eh, b, hi, lo, g->stream);
+        PhiPair<T, sizeof(T) == 4> pq{hi, lo, ghost_planes<T>(g, 2), ghost_planes<T>(g, 0)};
+        Q::j(s, v, pq, false, g->stream);
+        g->launches += 2;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        rotate_roles(g);
+        const int s0 = g->ghost_level_slot[0], s1 = g->ghost_level_slot[1], s2 = g->ghost_level_slot[2];
+        g->ghost_level_slot[0] = s2;
+        g->ghost_level_slot[1] = s0;
+        g->ghost_level_slot[2] = s1;
+        g->step++;
+        g->J_valid = s.last != 0;
+        ahead = !s.last;
+        if (stag) {
+            g->half_prev = true;  // the other set holds the last step's E^{n-1/2}
+            g->half_prev_cfg = g->cfg_version;
+        }
+        if (record) {
+            if ((e = diag_compute<T>(g, ring_slot(g, g->ring_written))) != cudaSuccess) return e;
+            g->ring_written++;
+        }
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// 32-bit cell indexes, and at least one active axis (a single cell keeps the general kernels)
+bool staged_supported(const axp_grid *g)
+{
+    const int64_t *n = g->desc.n;
+    return n[0] * n[1] * n[2] < ((int64_t)1 << 30) && n[0] > 1;
+}
+
+template <typename T>
+cudaError_t staged_step(axp_grid *g, int64_t nsteps)
+{
+    const int64_t *n = g->desc.n;
+    const uint32_t m = order0_closure(g);
+    auto in = [&](uint32_t set) { return (m & ~set) == 0; };
+    const uint32_t tm = 4u | (3u << 3), te = 3u | (4u << 3);  // (E0z; B0x, B0y) and (E0x, E0y; B0z)
+    if (n[1] == 1 && n[2] == 1) {
+        if (m == 0) return run_staged<T, Passes<T, 1, 0, 0>, 0, 0>(g, nsteps);
+        if (in(tm)) return run_staged<T, Passes<T, 1, 4, 3>, 4, 3>(g, nsteps);
+        if (in(te)) return run_staged<T, Passes<T, 1, 3, 4>, 3, 4>(g, nsteps);
+        return run_staged<T, Passes<T, 1, 7, 7>, 7, 7>(g, nsteps);
+    }
+    if (n[2] == 1) {
+        if (m == 0) return run_staged<T, Passes<T, 3, 0, 0>, 0, 0>(g, nsteps);
+        if (in(tm)) return run_staged<T, Passes<T, 3, 4, 3>, 4, 3>(g, nsteps);
+        if (in(te)) return run_staged<T, Passes<T, 3, 3, 4>, 3, 4>(g, nsteps);
+        return run_staged<T, Passes<T, 3, 7, 7>, 7, 7>(g, nsteps);
+    }
+    if (m == 0) return run_staged<T, Passes<T, 7, 0, 0>, 0, 0>(g, nsteps);
+    return run_staged<T, Passes<T, 7, 7, 7>, 7, 7>(g, nsteps);
+}
+
+template cudaError_t staged_step<double>(axp_grid *, int64_t);
+template cudaError_t staged_step<float>(axp_grid *, int64_t);
+
+}  // namespace axp
