@@ -3,7 +3,9 @@
 Each translation unit is compiled in parallel and linked into
 paper_2406_16796_gb300/_lib/libaxp.so.  The general-path unit is compiled
 without multiply-add contraction (its FP64 results follow a literal
-double-precision evaluation of the scheme); the others use the default.
+double-precision evaluation of the scheme), and so is the folded multi-pass unit
+(its multiply-adds are written out, so a run's bits do not depend on how it is
+cut into calls); the others use the default.
 """
 from __future__ import annotations
 

@@ -235,33 +235,6 @@ __device__ T p_comp(const View<T> &v, const PhiPair<T, INCR> &q, int a, int64_t 
     return Dt * b0_bar(v, a, i, j, k) - cross;
 }
 
-// Outflow ghost t of one face at the new level (Sec. 2.4 item 3): solve the
-// one-way wave equation and the wave equation at the ghost for
-// V = phi^{cur}_{-3/2} and U = phi^{new}_{-1/2}.  Both equations involve only the
-// fields at n+1/2 and the levels before the update.
-template <typename T>
-__device__ __forceinline__ void outflow_ghost_at(const View<T> &v, int ax, int side, int64_t t, const T *g_cur,
-                                                 const T *g_old, T *g_new)
-{
-    const int b = (ax + 1) % 3, cc = (ax + 2) % 3;
-    const int64_t nb = v.n[b];
-    const T r = v.dt / v.d[ax];
-    const T r2 = (v.dt * v.dt) / (v.d[ax] * v.d[ax]);
-    int64_t ca[3];
-    ca[b] = t % nb;
-    ca[cc] = t / nb;
-    ca[ax] = side ? v.n[ax] : -1;
-    const int64_t pi = ax == 0 ? ca[1] + v.n[1] * ca[2] : (ax == 1 ? ca[0] + v.n[0] * ca[2] : ca[0] + v.n[0] * ca[1]);
-    const T Sg = source_at(v, ca[0], ca[1], ca[2]);
-    int64_t ci[3] = {ca[0], ca[1], ca[2]};
-    ci[ax] = side ? v.n[ax] - 1 : 0;
-    const T p0 = v.phi_cur[lin3(v.n, ci[0], ci[1], ci[2])];
-    const T gc = g_cur[pi], go = g_old[pi];
-    const T rhs = T(-2) * gc + T(2) * go - (v.dt * v.dt) * (Sg - v.m2 * gc) + r * p0 - r2 * (p0 - T(2) * gc);
-    const T V = rhs / (r + r2);
-    g_new[pi] = go + r * (p0 - V);
-}
-
 template <typename T>
 __device__ __forceinline__ T sigma_of(const T *const tab[3], int64_t i, int64_t j, int64_t k)
 {

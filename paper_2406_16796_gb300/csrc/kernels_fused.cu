@@ -827,6 +827,12 @@ cudaError_t step_graph(axp_grid *g, Launch &&launch_one, cudaGraphExec_t *out)
     return cudaSuccess;
 }
 
+// FP64 grids of the 2D kernel up to this many cells take the folded passes: a block of
+// the 2D kernel marches at least 14 planes through one SM's FP64 units, which leaves a
+// small grid's step a serial chain.  us per step, passes / 2D kernel: 96 x 64 15 / 47,
+// 400 x 400 44 / 107, 1024 x 512 109 / 142, 800 x 800 131 / 142, 1024 x 768 157 / 142.
+constexpr int64_t kSmallTm = 700000;
+
 template <typename T>
 cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
 {
@@ -843,7 +849,10 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     const int set = pick_set(g);
     cudaError_t e = enter_staggered<T>(g);
     if (e != cudaSuccess) return e;
-    if (path == AXP_KERNEL_FUSED && g->kernel_choice == AXP_KERNEL_AUTO && mode >= 2 && staged_supported(g))
+    // AUTO runs the folded passes on the same staggered state where they are faster: in
+    // place of the generic kernel in 2D and 3D, and on small FP64 grids of the 2D kernel
+    const bool small_tm = tm && sizeof(T) == 8 && g->desc.n[0] * g->desc.n[1] <= kSmallTm;
+    if (g->kernel_choice == AXP_KERNEL_AUTO && (small_tm || (path == AXP_KERNEL_FUSED && mode >= 2)) && staged_supported(g))
         return staged_step<T>(g, nsteps);
     int tm_tx = tm2d::TX;  // tile width of the 2D kernel (chosen below)
     // FP32 split on an even-width grid without a soft source: the two-column form

@@ -339,13 +339,31 @@ __global__ void __launch_bounds__(kThreads) k_axion(View<T> v, Ghosts<T> gcur)
     }
 }
 
-// Outflow ghosts at the new level for one face (outflow_ghost_at).
+// Outflow ghosts at the new level for one face (Sec. 2.4 item 3): solve the
+// one-way wave equation and the wave equation at the ghost for
+// V = phi^{cur}_{-3/2} and U = phi^{new}_{-1/2}.
 template <typename T>
 __global__ void k_outflow(View<T> v, int ax, int side, const T *g_cur, const T *g_old, T *g_new)
 {
-    const int64_t plane = v.n[(ax + 1) % 3] * v.n[(ax + 2) % 3];
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < plane; t += (int64_t)gridDim.x * blockDim.x)
-        outflow_ghost_at(v, ax, side, t, g_cur, g_old, g_new);
+    const int b = (ax + 1) % 3, cc = (ax + 2) % 3;
+    const int64_t nb = v.n[b], nc = v.n[cc];
+    const T r = v.dt / v.d[ax];
+    const T r2 = (v.dt * v.dt) / (v.d[ax] * v.d[ax]);
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < nb * nc; t += (int64_t)gridDim.x * blockDim.x) {
+        int64_t ca[3];
+        ca[b] = t % nb;
+        ca[cc] = t / nb;
+        ca[ax] = side ? v.n[ax] : -1;
+        const int64_t pi = ax == 0 ? ca[1] + v.n[1] * ca[2] : (ax == 1 ? ca[0] + v.n[0] * ca[2] : ca[0] + v.n[0] * ca[1]);
+        const T Sg = source_at(v, ca[0], ca[1], ca[2]);
+        int64_t ci[3] = {ca[0], ca[1], ca[2]};
+        ci[ax] = side ? v.n[ax] - 1 : 0;
+        const T p0 = v.phi_cur[lin3(v.n, ci[0], ci[1], ci[2])];
+        const T gc = g_cur[pi], go = g_old[pi];
+        const T rhs = T(-2) * gc + T(2) * go - (v.dt * v.dt) * (Sg - v.m2 * gc) + r * p0 - r2 * (p0 - T(2) * gc);
+        const T V = rhs / (r + r2);
+        g_new[pi] = go + r * (p0 - V);
+    }
 }
 
 // Inverse of half_update: the field a half-step h earlier, given X.

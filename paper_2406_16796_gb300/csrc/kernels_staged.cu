@@ -5,8 +5,8 @@
 // What bounds it: on GB300 an FP64 step is bound by the FP64 pipe (2 operations
 // per cycle per SM), so each quantity is formed once and every constant is folded;
 // an FP32 step by memory and launch latency.  The literal kernels
-// (kernels_general.cu) take 8 launches and about 400 FP64 operations per 3D cell
-// (their divisions included); these take 4 launches and 143:
+// (kernels_general.cu) take 8 launches and several hundred FP64 operations per 3D cell
+// (their divisions included); these take 4 launches and about 170:
 //   B      B^{n+1} of both orders; B0^{n+1/2} is kept in scratch
 //   phi    S and phi^{n+3/2}; E0^{n+1} (to scratch) and E0^{n+3/2}
 //   P      the axion current's P at the cell centres
@@ -24,9 +24,12 @@
 // several calls then gives the bits of the uncut one.  Multiply-adds are written
 // out and the unit is compiled without contraction, for the same reason.
 //
-// Measured on one GB300, against the literal kernels (us per step):
-//   2D TM laser, outflow axion sides, FP64, 1024 x 512:  STAGED_OUTFLOW
-//   3D laser, absorbing x sides, FP64, 160 x 96 x 96:    STAGED_LASER3D
+// Measured on one GB300 (us per step, before: the literal or the generic kernel):
+//   2D TM laser, outflow axion sides, FP64, 1024 x 512       686 -> 120
+//   3D laser, absorbing x sides, FP64, 160 x 96 x 96        1922 -> 535
+//   2D laser polarised in the plane, FP32 split, 1024 x 512  130 -> 33
+//   2D TM laser, absorbing sides, FP64, 400 x 400            160 -> 44 (the 2D kernel)
+// ncu: the FP64 passes keep the FP64 pipe 76-84% busy while an SM is active.
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -34,7 +37,7 @@
 namespace axp {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;  // (256: 3% slower on 1024 x 512, 8% on 400 x 400)
 
 template <typename T>
 struct Stage {
@@ -46,21 +49,50 @@ struct Stage {
     const T *phi, *phib;  // phi^{n+1/2}; phi^{n-1/2} (FP64) or the increment (FP32 split)
     T *phi_out, *phib_out;
     const T *jp[2][3];                  // macroparticle currents (null without)
-    const T *gh[3][2], *gh_hi[3][2];    // outflow ghosts of phi^{n+1/2} and phi^{n+3/2}
+    // outflow ghosts: phi^{n+1/2}, phi^{n-1/2}, phi^{n+3/2} written, and (gh_hi) the later
+    // level the P pass reads
+    const T *gh[3][2], *gh_old[3][2], *gh_hi[3][2];
+    T *gh_new[3][2];
     const T *tab[3];                    // layer coefficients per axis (null: no layer)
     const T *sig_ax[3];
     int n[3], per[3], axbc[3][2];
+    int lay[3][2];  // cells of absorbing layer at each side
     int N;
+    int uniform_e;
     T hd[3];              // h/d
     T inv_h, h;
     T hg2;                // h g / 2: J is used as the sum of two P
-    T lap_c[3], lap_0, dt2g, dt, inv_dt, q4d[3];
+    T lap_c[3], lap_0, dt2g, m2dt2, dt, dt2, inv_dt2, inv_dt, q4d[3], of_r[3];
     T Bext[3], Eext[3];
     int src_x;            // x index of the soft source's E cells (-1: none)
     const T *src_w[2];
     T src_e, src_b;       // h tau of the electric and of the magnetic sheet
     int last;             // the step ends at integer time (only the first E half-step)
 };
+
+// Programmatic dependent launch: a pass is set up while the one before it ends, and
+// waits here before its first access to memory another pass writes.  No earlier
+// trigger is given: blocks of the next pass that come in while this one still runs
+// land on the SMs that are free first and leave them unevenly loaded (256 x 128 FP64:
+// 41 us per step with a trigger at the start, 18 without).
+__device__ __forceinline__ void wait_for_previous_pass()
+{
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+}
+template <typename... KArgs, typename... Args>
+void launch_pass(void (*kern)(KArgs...), int blocks, cudaStream_t st, const Args &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);  // (errors: the caller's cudaGetLastError)
+}
 
 // A cell's index, its neighbours' (wrapped along periodic axes) and whether they exist.
 struct Cell {
@@ -118,45 +150,56 @@ __device__ __forceinline__ T curl_h(const Stage<T> &s, const T *const F[3], int 
     return T(0);
 }
 
-// The absorbing layer at a cell: a half-step is F <- a F + r (h X), a = 1 and r = 1
-// outside the layers; both decrease with sigma, so a corner takes the smallest.
-template <typename T>
+// The absorbing layer at a cell: a half-step is F <- a F + r (h X) (a = r = 1 outside
+// the layers); both decrease with sigma, so a corner takes the smallest.  Whether a
+// cell lies in a layer is decided on integers (a comparison of doubles takes the FP64
+// pipe), and a warp with any layer cell takes the IN body for all its cells: with
+// a = r = 1 it rounds as the plain one, and two bodies run in turn by a divided warp
+// cost more (3D laser 160 x 96 x 96: 658 against 538 us per step).
+template <typename T, bool IN>
 struct Layer {
     T a, r;
     bool in;
+    __device__ __forceinline__ T half_step(T F, T hX) const { return IN ? fma(a, F, r * hX) : F + hX; }
 };
 template <int MASK, typename T>
-__device__ __forceinline__ Layer<T> layer_at(const Stage<T> &s, const Cell &q)
+__device__ __forceinline__ bool in_layer(const Stage<T> &s, const Cell &q)
 {
-    Layer<T> L{T(1), T(1), false};
+    bool in = false;
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+        if (MASK >> a & 1) in = in || q.x[a] < s.lay[a][0] || q.x[a] >= s.n[a] - s.lay[a][1];
+    return in;
+}
+// whether any of the warp's cells (those of an incomplete last warp) lies in a layer
+template <int MASK, typename T>
+__device__ __forceinline__ bool warp_in_layer(const Stage<T> &s, const Cell &q)
+{
+    return __any_sync(__activemask(), in_layer<MASK>(s, q));
+}
+template <int MASK, bool IN, typename T>
+__device__ __forceinline__ Layer<T, IN> layer_at(const Stage<T> &s, const Cell &q)
+{
+    Layer<T, IN> L{T(1), T(1), false};
+    if (!IN || !in_layer<MASK>(s, q)) return L;
+    L.in = true;
     T b = s.h;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         if (!(MASK >> a & 1) || !s.tab[a]) continue;
-        const T ta = s.tab[a][q.x[a]];
-        if (ta < L.a) {
-            L.a = ta;
-            b = s.tab[a][s.n[a] + q.x[a]];
-            L.in = true;
-        }
+        L.a = min(L.a, s.tab[a][q.x[a]]);
+        b = min(b, s.tab[a][s.n[a] + q.x[a]]);
     }
-    if (L.in) L.r = b * s.inv_h;
+    L.r = b * s.inv_h;
     return L;
-}
-template <typename T>
-__device__ __forceinline__ T half_step(const Layer<T> &L, T F, T hX)
-{
-    return L.in ? fma(L.a, F, L.r * hX) : F + hX;
 }
 
 // MODE 0: the full B step (B0^{n+1/2} to scratch); 1 and 2: one half-step from Bin
 // to Bout (with macroparticles; the second in place).
-template <typename T, int MASK, int EM, int BM, int MODE>
-__global__ void __launch_bounds__(kThreads) k_stage_b(Stage<T> s)
+template <typename T, int MASK, int EM, int BM, int MODE, bool IN>
+__device__ __forceinline__ void b_pass(const Stage<T> &s, const Cell &q)
 {
-    Cell q;
-    if (!cell_at<MASK>(s, q)) return;
-    const Layer<T> L = layer_at<MASK>(s, q);
+    const Layer<T, IN> L = layer_at<MASK, IN>(s, q);
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         if (!(BM >> a & 1)) continue;
@@ -165,10 +208,10 @@ __global__ void __launch_bounds__(kThreads) k_stage_b(Stage<T> s)
             const int jk = q.x[1] + s.n[1] * q.x[2];
             hX = a == 1 ? fma(-s.src_w[1][jk], s.src_b, hX) : fma(s.src_w[0][jk], s.src_b, hX);
         }
-        const T Bh = half_step(L, s.Bin[a][q.c], hX);
+        const T Bh = L.half_step(s.Bin[a][q.c], hX);
         if (MODE == 0) {
             s.Bh[a][q.c] = Bh;
-            s.Bout[a][q.c] = half_step(L, Bh, hX);
+            s.Bout[a][q.c] = L.half_step(Bh, hX);
         } else {
             s.Bout[a][q.c] = Bh;
         }
@@ -177,10 +220,22 @@ __global__ void __launch_bounds__(kThreads) k_stage_b(Stage<T> s)
 #pragma unroll
     for (int a = 0; a < 3; a++) {
         const T hX = -curl_h<MASK, 7, true>(s, E1, a, q), B = s.Bin[3 + a][q.c];
-        T r = half_step(L, B, hX);
-        if (MODE == 0) r = L.in ? half_step(L, r, hX) : fma(T(2), hX, B);
+        T r;
+        if (MODE > 0) r = L.half_step(B, hX);
+        else if (IN && L.in) r = L.half_step(L.half_step(B, hX), hX);
+        else r = fma(T(2), hX, B);
         s.Bout[3 + a][q.c] = r;
     }
+}
+template <typename T, int MASK, int EM, int BM, int MODE>
+__global__ void __launch_bounds__(kThreads) k_stage_b(Stage<T> s)
+{
+    Cell q;
+    const bool mine = cell_at<MASK>(s, q);
+    wait_for_previous_pass();
+    if (!mine) return;
+    if (warp_in_layer<MASK>(s, q)) b_pass<T, MASK, EM, BM, MODE, true>(s, q);
+    else b_pass<T, MASK, EM, BM, MODE, false>(s, q);
 }
 
 // 2-point average of E0_a at the cell centre plus the background
@@ -228,11 +283,40 @@ __device__ __forceinline__ T phi_nb(const Stage<T> &s, const T *__restrict__ F, 
     return gh[a][side][pi];
 }
 
+// The outflow ghost next to cell q on one face, at the new level (Sec. 2.4 item 3): the
+// one-way wave equation and the wave equation at the ghost, solved for phi^{cur} half
+// a cell further out (V) and phi^{new} at the ghost.  The source at the ghost cell, which
+// sees zero fields outside the grid plus the background: along the face normal E0 of
+// the last cell (high side) meets B_ext, across it E_ext meets B0 averaged with zeros.
+template <typename T, int MASK, int EM, int BM>
+__device__ void outflow_ghost(const Stage<T> &s, const T *const Bs[3], int ax, int side, T p0, const Cell &q)
+{
+    T S = T(0);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        T e = s.Eext[a], b = s.Bext[a];
+        if (a == ax) {
+            if (side && (EM >> a & 1)) e = fma(T(0.5), s.Ein[a][q.c], e);
+        } else if (side && (BM >> a & 1)) {
+            const int o = 3 - a - ax;  // the third axis
+            b = fma(T(0.25), Bs[a][q.c] + ldz(Bs[a], q.dn[o], q.hd[o]), b);
+        }
+        S = fma(e, b, S);
+    }
+    const int pi = ax == 0 ? q.x[1] + s.n[1] * q.x[2] : (ax == 1 ? q.x[0] + s.n[0] * q.x[2] : q.x[0] + s.n[0] * q.x[1]);
+    const T gc = s.gh[ax][side][pi], go = s.gh_old[ax][side][pi], r = s.of_r[ax];
+    T rhs = fma(T(2), go - gc, fma(s.m2dt2, gc, -(s.dt2g * S)));
+    rhs = fma(r, p0, rhs) - r * r * fma(T(-2), gc, p0);
+    const T V = rhs / fma(r, r, r);
+    s.gh_new[ax][side][pi] = fma(r, p0 - V, go);
+}
+
 // E0 from E0^{n+1/2}: E0^{n+1} to scratch and, unless the step ends at integer time,
 // E0^{n+3/2} to the output set.
-template <typename T, int MASK, int EM, int BM>
-__device__ __forceinline__ void e0_update(const Stage<T> &s, const Cell &q, const Layer<T> &L)
+template <typename T, int MASK, int EM, int BM, bool IN>
+__device__ __forceinline__ void e0_update(const Stage<T> &s, const Cell &q)
 {
+    const Layer<T, IN> L = layer_at<MASK, IN>(s, q);
     const T *const B0[3] = {s.Bout[0], s.Bout[1], s.Bout[2]};
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -240,9 +324,9 @@ __device__ __forceinline__ void e0_update(const Stage<T> &s, const Cell &q, cons
         T hX = curl_h<MASK, BM, false>(s, B0, a, q);
         if (a > 0 && q.x[0] == s.src_x) hX = fma(s.src_w[a - 1][q.x[1] + s.n[1] * q.x[2]], s.src_e, hX);
         if (s.jp[0][a]) hX = fma(-s.h, s.jp[0][a][q.c], hX);
-        const T E = half_step(L, s.Ein[a][q.c], hX);
+        const T E = L.half_step(s.Ein[a][q.c], hX);
         s.Eh[a][q.c] = E;
-        s.Eout[a][q.c] = s.last ? E : half_step(L, E, hX);
+        s.Eout[a][q.c] = s.last ? E : L.half_step(E, hX);
     }
 }
 
@@ -253,7 +337,9 @@ __global__ void __launch_bounds__(kThreads) k_stage_phi(Stage<T> s, const T *bs0
 {
     constexpr bool INCR = sizeof(T) == 4;
     Cell q;
-    if (!cell_at<MASK>(s, q)) return;
+    const bool mine = cell_at<MASK>(s, q);
+    wait_for_previous_pass();
+    if (!mine) return;
     if (PHI) {
         const T *const Bs[3] = {bs0, bs1, bs2};
         T S = T(0);
@@ -269,31 +355,38 @@ __global__ void __launch_bounds__(kThreads) k_stage_phi(Stage<T> s, const T *bs0
             lap = fma(s.lap_c[a], INCR ? (up - ph) + (dn - ph) : up + dn, lap);
         }
         lap = fma(s.lap_0, ph, lap);  // FP64: lap_0 holds the 2 phi of the leapfrog too
-        T sig = T(0);
+        T nw;  // phi^{n+3/2}, or its increment in FP32 split
+        if (in_layer<MASK>(s, q)) {
+            // (lap - (sigma dt)^2 phi -+ (1 - sigma dt) old) / (1 + sigma dt) from the tables
+            // c1 = dt^2 / (1 + sigma dt) and c2 = (1 - sigma dt) / (1 + sigma dt)
+            T sd = T(0), c1 = s.dt2, c2 = T(1);
 #pragma unroll
-        for (int a = 0; a < 3; a++)
-            if ((MASK >> a & 1) && s.tab[a]) {
-                const T t = s.sig_ax[a][q.x[a]];
-                if (t > sig) sig = t;
+            for (int a = 0; a < 3; a++) {
+                if (!(MASK >> a & 1) || !s.tab[a]) continue;
+                sd = max(sd, s.sig_ax[a][q.x[a]]);
+                c1 = min(c1, s.tab[a][4 * s.n[a] + q.x[a]]);
+                c2 = min(c2, s.tab[a][5 * s.n[a] + q.x[a]]);
             }
-        if (INCR) {
-            T nin = lap + old;
-            if (sig != T(0)) {
-                const T sd = sig * s.dt;
-                nin = (fma(-(sd * sd), ph, lap) + (T(1) - sd) * old) / (T(1) + sd);
-            }
-            s.phib_out[q.c] = nin;
-            s.phi_out[q.c] = ph + nin;
+            sd = sd * s.dt;
+            lap = fma(-(sd * sd), ph, lap);
+            nw = fma(INCR ? c2 : -c2, old, c1 * s.inv_dt2 * lap);
         } else {
-            T nw = lap - old;
-            if (sig != T(0)) {
-                const T sd = sig * s.dt;
-                nw = (fma(-(sd * sd), ph, lap) - (T(1) - sd) * old) / (T(1) + sd);
-            }
-            s.phi_out[q.c] = nw;
+            nw = INCR ? lap + old : lap - old;
+        }
+        s.phi_out[q.c] = INCR ? ph + nw : nw;
+        if (INCR) s.phib_out[q.c] = nw;
+        // the ghosts beyond outflow faces belong to the cells next to them
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            if (!(MASK >> a & 1)) continue;
+            if (!q.hd[a] && s.axbc[a][0] == AXP_BC_OUTFLOW) outflow_ghost<T, MASK, EM, BM>(s, Bs, a, 0, ph, q);
+            if (!q.hu[a] && s.axbc[a][1] == AXP_BC_OUTFLOW) outflow_ghost<T, MASK, EM, BM>(s, Bs, a, 1, ph, q);
         }
     }
-    if (E0) e0_update<T, MASK, EM, BM>(s, q, layer_at<MASK>(s, q));
+    if (E0) {
+        if (warp_in_layer<MASK>(s, q)) e0_update<T, MASK, EM, BM, true>(s, q);
+        else e0_update<T, MASK, EM, BM, false>(s, q);
+    }
 }
 
 // P = (D_t phi) Bbar0 - Ebar0 x grad_c phi^{n+1} at the cell centres, from E0^{n+1}
@@ -305,7 +398,9 @@ __global__ void __launch_bounds__(kThreads) k_stage_p(Stage<T> s, const T *e0, c
 {
     constexpr bool INCR = sizeof(T) == 4;
     Cell q;
-    if (!cell_at<MASK>(s, q)) return;
+    const bool mine = cell_at<MASK>(s, q);
+    wait_for_previous_pass();
+    if (!mine) return;
     const T *const E[3] = {e0, e1, e2};
     const T *const B[3] = {b0, b1, b2};
     T g[3], e[3];
@@ -341,12 +436,27 @@ __global__ void __launch_bounds__(kThreads) k_stage_p(Stage<T> s, const T *e0, c
 // J = (P(c) + P(c + a)) / 2 and the order-1 E update; CURRENT: only J.  Beyond the
 // last cell of a non-periodic axis P follows the ghost rules: 0 at a PML side without
 // a uniform E, else evaluated in place (one cell per row or plane).
+template <typename T, int MASK, bool IN>
+__device__ __forceinline__ void e1_update(const Stage<T> &s, const T J2[3], const Cell &q)
+{
+    const Layer<T, IN> L = layer_at<MASK, IN>(s, q);
+    const T *const B1[3] = {s.Bout[3], s.Bout[4], s.Bout[5]};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        T hX = fma(-s.hg2, J2[a], curl_h<MASK, 7, false>(s, B1, a, q));
+        if (s.jp[1][a]) hX = fma(-s.h, s.jp[1][a][q.c], hX);
+        T E = L.half_step(s.Ein[3 + a][q.c], hX);
+        if (!s.last) E = L.half_step(E, hX);
+        s.Eout[3 + a][q.c] = E;
+    }
+}
 template <typename T, int MASK, bool CURRENT>
 __global__ void __launch_bounds__(kThreads) k_stage_j(Stage<T> s, View<T> v, PhiPair<T, sizeof(T) == 4> pq)
 {
     Cell q;
-    if (!cell_at<MASK>(s, q)) return;
-    const bool ext = s.Eext[0] != T(0) || s.Eext[1] != T(0) || s.Eext[2] != T(0);
+    const bool mine = cell_at<MASK>(s, q);
+    wait_for_previous_pass();
+    if (!mine) return;
     T J2[3];
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -354,7 +464,7 @@ __global__ void __launch_bounds__(kThreads) k_stage_j(Stage<T> s, View<T> v, Phi
         T p1 = p0;
         if (MASK >> a & 1) {
             if (q.hu[a]) p1 = s.P[a][q.up[a]];
-            else if (s.axbc[a][1] == AXP_BC_PML && !ext) p1 = T(0);
+            else if (s.axbc[a][1] == AXP_BC_PML && !s.uniform_e) p1 = T(0);
             else
                 p1 = p_comp<T, sizeof(T) == 4>(v, pq, a, q.x[0] + (a == 0), q.x[1] + (a == 1), q.x[2] + (a == 2));
         }
@@ -362,26 +472,16 @@ __global__ void __launch_bounds__(kThreads) k_stage_j(Stage<T> s, View<T> v, Phi
         if (CURRENT || s.last) s.J[a][q.c] = T(0.5) * J2[a];
     }
     if (CURRENT) return;
-    const Layer<T> L = layer_at<MASK>(s, q);
-    const T *const B1[3] = {s.Bout[3], s.Bout[4], s.Bout[5]};
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        T hX = fma(-s.hg2, J2[a], curl_h<MASK, 7, false>(s, B1, a, q));
-        if (s.jp[1][a]) hX = fma(-s.h, s.jp[1][a][q.c], hX);
-        T E = half_step(L, s.Ein[3 + a][q.c], hX);
-        if (!s.last) E = half_step(L, E, hX);
-        s.Eout[3 + a][q.c] = E;
-    }
+    if (warp_in_layer<MASK>(s, q)) e1_update<T, MASK, true>(s, J2, q);
+    else e1_update<T, MASK, false>(s, J2, q);
 }
 
 // The first E half-step of a run that starts at integer time, in place, with the J
 // of the present state (the same increments as the step's own half-steps).
-template <typename T, int MASK, int EM, int BM>
-__global__ void __launch_bounds__(kThreads) k_stage_e_half(Stage<T> s)
+template <typename T, int MASK, int EM, int BM, bool IN>
+__device__ __forceinline__ void e_half_pass(const Stage<T> &s, const Cell &q)
 {
-    Cell q;
-    if (!cell_at<MASK>(s, q)) return;
-    const Layer<T> L = layer_at<MASK>(s, q);
+    const Layer<T, IN> L = layer_at<MASK, IN>(s, q);
     const T *const B1[3] = {s.Bin[3], s.Bin[4], s.Bin[5]};
 #pragma unroll
     for (int a = 0; a < 3; a++) {
@@ -390,29 +490,23 @@ __global__ void __launch_bounds__(kThreads) k_stage_e_half(Stage<T> s)
             if (a > 0 && q.x[0] == s.src_x) hX = fma(s.src_w[a - 1][q.x[1] + s.n[1] * q.x[2]], s.src_e, hX);
             if (s.jp[0][a]) hX = fma(-s.h, s.jp[0][a][q.c], hX);
             T *E = const_cast<T *>(s.Ein[a]);
-            E[q.c] = half_step(L, E[q.c], hX);
+            E[q.c] = L.half_step(E[q.c], hX);
         }
         T hX = fma(-s.hg2, T(2) * s.J[a][q.c], curl_h<MASK, 7, false>(s, B1, a, q));
         if (s.jp[1][a]) hX = fma(-s.h, s.jp[1][a][q.c], hX);
         T *E = const_cast<T *>(s.Ein[3 + a]);
-        E[q.c] = half_step(L, E[q.c], hX);
+        E[q.c] = L.half_step(E[q.c], hX);
     }
 }
-
-// every outflow face's ghosts in one launch (blockIdx.y: the face)
-template <typename T>
-__global__ void __launch_bounds__(kThreads) k_stage_outflow(View<T> v)
+template <typename T, int MASK, int EM, int BM>
+__global__ void __launch_bounds__(kThreads) k_stage_e_half(Stage<T> s)
 {
-    int f = (int)blockIdx.y, ax = 0, side = 0;
-    for (int a = 0; a < 3; a++)
-        for (int e = 0; e < 2; e++)
-            if (v.axbc[a][e] == AXP_BC_OUTFLOW && f-- == 0) {
-                ax = a;
-                side = e;
-            }
-    const int64_t plane = v.n[(ax + 1) % 3] * v.n[(ax + 2) % 3];
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < plane; t += (int64_t)gridDim.x * blockDim.x)
-        outflow_ghost_at(v, ax, side, t, v.gh[ax][side][0], v.gh[ax][side][1], v.gh[ax][side][2]);
+    Cell q;
+    const bool mine = cell_at<MASK>(s, q);
+    wait_for_previous_pass();
+    if (!mine) return;
+    if (warp_in_layer<MASK>(s, q)) e_half_pass<T, MASK, EM, BM, true>(s, q);
+    else e_half_pass<T, MASK, EM, BM, false>(s, q);
 }
 
 template <typename T>
@@ -443,13 +537,19 @@ Stage<T> make_stage(axp_grid *g)
             s.jp[o][a] = g->parts && sizeof(T) == sizeof(double) ? (const T *)g->parts->j[o][a] : nullptr;
         bool layer = false;
         for (int e = 0; e < 2; e++) {
-            const size_t cur = w.off_ghost[a][e][g->ghost_level_slot[0]], nxt = w.off_ghost[a][e][g->ghost_level_slot[2]];
-            s.gh[a][e] = cur ? at(cur) : nullptr;
-            s.gh_hi[a][e] = nxt ? at(nxt) : nullptr;
+            const size_t *lev = w.off_ghost[a][e];
+            const bool of = d.axion_bc[a][e] == AXP_BC_OUTFLOW;
+            s.gh[a][e] = of ? at(lev[g->ghost_level_slot[0]]) : nullptr;
+            s.gh_old[a][e] = of ? at(lev[g->ghost_level_slot[1]]) : nullptr;
+            s.gh_new[a][e] = of ? at(lev[g->ghost_level_slot[2]]) : nullptr;
+            s.gh_hi[a][e] = s.gh_new[a][e];
             s.axbc[a][e] = d.axion_bc[a][e];
-            if (d.em_bc[a][e] == AXP_BC_PML || d.axion_bc[a][e] == AXP_BC_PML) layer = true;
+            const bool pml = (d.em_bc[a][e] == AXP_BC_PML || d.axion_bc[a][e] == AXP_BC_PML) && d.pml_sigma_max_dt > 0;
+            s.lay[a][e] = pml ? (int)std::min<int64_t>(d.pml_cells, d.n[a]) : 0;
+            if (s.lay[a][e] > 0) layer = true;
         }
-        s.tab[a] = layer && d.pml_cells > 0 && d.pml_sigma_max_dt > 0 ? at(w.off_pml_tab[a]) : nullptr;
+        s.tab[a] = layer ? at(w.off_pml_tab[a]) : nullptr;
+        s.of_r[a] = (T)(d.dt / d.d[a]);
         s.sig_ax[a] = at(w.off_sig_ax[a]);
         s.n[a] = (int)d.n[a];
         s.per[a] = d.em_bc[a][0] == AXP_BC_PERIODIC;
@@ -466,7 +566,11 @@ Stage<T> make_stage(axp_grid *g)
     s.hg2 = (T)(0.5 * h * d.g);
     s.lap_0 = (T)(sizeof(T) == 4 ? -d.dt * d.dt * d.m * d.m : 2.0 - d.dt * d.dt * (d.m * d.m + 2.0 * idd));
     s.dt2g = (T)(d.dt * d.dt * d.g);
+    s.m2dt2 = (T)(d.dt * d.dt * d.m * d.m);
+    s.uniform_e = g->E_ext[0] != 0.0 || g->E_ext[1] != 0.0 || g->E_ext[2] != 0.0;
     s.dt = (T)d.dt;
+    s.dt2 = (T)(d.dt * d.dt);
+    s.inv_dt2 = (T)(1.0 / (d.dt * d.dt));
     s.inv_dt = (T)(1.0 / d.dt);
     s.src_x = -1;
     s.src_w[0] = at(w.off_src[0]);
@@ -483,30 +587,29 @@ struct Passes {
     static int blocks(const Stage<T> &s) { return (s.N + kThreads - 1) / kThreads; }
     static void b(const Stage<T> &s, int mode, cudaStream_t st)
     {
-        if (mode == 0) k_stage_b<T, MASK, EM, BM, 0><<<blocks(s), kThreads, 0, st>>>(s);
-        else if (mode == 1) k_stage_b<T, MASK, EM, BM, 1><<<blocks(s), kThreads, 0, st>>>(s);
-        else k_stage_b<T, MASK, EM, BM, 2><<<blocks(s), kThreads, 0, st>>>(s);
+        if (mode == 0) launch_pass(k_stage_b<T, MASK, EM, BM, 0>, blocks(s), st, s);
+        else if (mode == 1) launch_pass(k_stage_b<T, MASK, EM, BM, 1>, blocks(s), st, s);
+        else launch_pass(k_stage_b<T, MASK, EM, BM, 2>, blocks(s), st, s);
     }
+    // part 1: the axion, 2: E0, 3: both
     static void phi(const Stage<T> &s, T *const bs[3], int part, cudaStream_t st)
     {
-        if (part == 3) k_stage_phi<T, MASK, EM, BM, true, true><<<blocks(s), kThreads, 0, st>>>(s, bs[0], bs[1], bs[2]);
-        else if (part == 1)
-            k_stage_phi<T, MASK, EM, BM, true, false><<<blocks(s), kThreads, 0, st>>>(s, bs[0], bs[1], bs[2]);
-        else
-            k_stage_phi<T, MASK, EM, BM, false, true><<<blocks(s), kThreads, 0, st>>>(s, bs[0], bs[1], bs[2]);
+        if (part == 3) launch_pass(k_stage_phi<T, MASK, EM, BM, true, true>, blocks(s), st, s, bs[0], bs[1], bs[2]);
+        else if (part == 1) launch_pass(k_stage_phi<T, MASK, EM, BM, true, false>, blocks(s), st, s, bs[0], bs[1], bs[2]);
+        else launch_pass(k_stage_phi<T, MASK, EM, BM, false, true>, blocks(s), st, s, bs[0], bs[1], bs[2]);
     }
     static void p(const Stage<T> &s, const T *const e[3], const T *const b[3], const T *hi, const T *lo, cudaStream_t st)
     {
-        k_stage_p<T, MASK, EM, BM><<<blocks(s), kThreads, 0, st>>>(s, e[0], e[1], e[2], b[0], b[1], b[2], hi, lo);
+        launch_pass(k_stage_p<T, MASK, EM, BM>, blocks(s), st, s, e[0], e[1], e[2], b[0], b[1], b[2], hi, lo);
     }
     static void j(const Stage<T> &s, const View<T> &v, const PhiPair<T, sizeof(T) == 4> &pq, bool current, cudaStream_t st)
     {
-        if (current) k_stage_j<T, MASK, true><<<blocks(s), kThreads, 0, st>>>(s, v, pq);
-        else k_stage_j<T, MASK, false><<<blocks(s), kThreads, 0, st>>>(s, v, pq);
+        if (current) launch_pass(k_stage_j<T, MASK, true>, blocks(s), st, s, v, pq);
+        else launch_pass(k_stage_j<T, MASK, false>, blocks(s), st, s, v, pq);
     }
     static void e_half(const Stage<T> &s, cudaStream_t st)
     {
-        k_stage_e_half<T, MASK, EM, BM><<<blocks(s), kThreads, 0, st>>>(s);
+        launch_pass(k_stage_e_half<T, MASK, EM, BM>, blocks(s), st, s);
     }
 };
 
@@ -528,14 +631,6 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
 {
     const axp_grid_desc &d = g->desc;
     const bool stag = g->staggered;  // the single-pass kernels' state: E stays half a step ahead
-    int faces = 0;  // outflow faces
-    int64_t plane = 0;
-    for (int a = 0; a < 3; a++)
-        for (int e = 0; e < 2; e++)
-            if (d.axion_bc[a][e] == AXP_BC_OUTFLOW) {
-                faces++;
-                plane = std::max<int64_t>(plane, d.n[(a + 1) % 3] * d.n[(a + 2) % 3]);
-            }
     const bool parts = g->parts != nullptr;
     bool ahead = stag;  // E at n+1/2
     cudaError_t e = cudaSuccess;
@@ -543,13 +638,12 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
         const bool record = d.diag_every > 0 && (g->step + 1) % d.diag_every == 0;
         if (!ahead) {
             if (!g->J_valid) {
-                // the P pass reads ghosts of n+1/2 and n-1/2 here
-                const int s0 = g->ghost_level_slot[0], s1 = g->ghost_level_slot[1], s2 = g->ghost_level_slot[2];
-                g->ghost_level_slot[2] = s0;
-                g->ghost_level_slot[0] = s1;
-                const Stage<T> s = make_stage<T>(g);
-                g->ghost_level_slot[0] = s0;
-                g->ghost_level_slot[2] = s2;
+                Stage<T> s = make_stage<T>(g);
+                for (int a = 0; a < 3; a++)  // the levels around n: n+1/2 and n-1/2
+                    for (int f = 0; f < 2; f++) {
+                        s.gh_hi[a][f] = s.gh[a][f];
+                        s.gh[a][f] = s.gh_old[a][f];
+                    }
                 View<T> v = make_view<T>(g);
                 const T *const b[3] = {s.Bin[0], s.Bin[1], s.Bin[2]};
                 Q::p(s, s.Ein, b, s.phi, s.phib, g->stream);
@@ -569,19 +663,9 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
             s.src_b = (T)(d.dt / 2.0 * source_wave(g, source_x_e(g), time_half(g, g->step)));
             s.src_e = (T)(d.dt / 2.0 * source_wave(g, source_x_b(g), time_n(g, g->step + 1)));
         }
-        // outflow ghosts at the new level, from the fields at n+1/2 (bh: where B0^{n+1/2} lies)
-        auto outflow_ghosts = [&](T *const bh[3]) {
-            if (faces == 0) return;
-            View<T> v = make_view<T>(g);
-            for (int a = 0; a < 3; a++) v.f[kB0 + a] = (BM >> a & 1) ? bh[a] : s.Bout[a];
-            const dim3 grid((unsigned)std::min<int64_t>((plane + kThreads - 1) / kThreads, 1024), (unsigned)faces);
-            k_stage_outflow<T><<<grid, kThreads, 0, g->stream>>>(v);
-            g->launches++;
-        };
         if constexpr (sizeof(T) == sizeof(double)) {
             if (parts) {
                 Q::b(s, 1, g->stream);
-                outflow_ghosts(s.Bout);
                 View<double> v = make_view<double>(g);
                 for (int a = 0; a < 3; a++) {
                     v.f[kB0 + a] = s.Bout[a];
@@ -598,7 +682,6 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
         }
         if (!parts) {
             Q::b(s, 0, g->stream);
-            outflow_ghosts(s.Bh);
             Q::phi(s, s.Bh, 3, g->stream);
             g->launches += 2;
         }
