@@ -147,7 +147,8 @@ cudaError_t diag_compute(axp_grid *g, axp_diag *dev_dst)
 // half-step's layer coefficients (a = 1, b = h outside the layers; the smallest
 // a of the axes at a corner).  Hence E^n = (E^{n+1/2} + a E^{n-1/2}) / (1 + a),
 // the mean of the two levels outside the layers.  Written over E^{n-1/2} (the
-// other field set); the active E arrays only (the others are zero in both sets).
+// other field set); only the E arrays that can be non-zero (the others are zero in
+// both sets).
 template <typename T>
 struct ELevels {
     T *lo[6];        // E^{n-1/2}, overwritten with E^n (order 0 xyz, order 1 xyz)
@@ -187,10 +188,11 @@ cudaError_t e_level_from_halves(axp_grid *g)
     const int oset = 1 - g->fset;
     const int fe[6] = {kE0, kE0 + 1, kE0 + 2, kE1, kE1 + 1, kE1 + 2};
     L.mask = 0;
+    const uint32_t closure = order0_closure(g);  // the components a step moves, injected or driven
     for (int f = 0; f < 6; f++) {
         L.lo[f] = (T *)(g->ws + w.off_fields[oset][fe[f]]);
         L.hi[f] = (const T *)(g->ws + w.off_fields[g->fset][fe[f]]);
-        if (f >= 3 || (g->active >> fe[f] & 1u)) L.mask |= 1u << f;
+        if (f >= 3 || (closure >> f & 1u)) L.mask |= 1u << f;
     }
     for (int a = 0; a < 3; a++) {
         const bool lay = g->desc.em_bc[a][0] != AXP_BC_PERIODIC && g->desc.pml_cells > 0 && g->desc.pml_sigma_max_dt > 0;
