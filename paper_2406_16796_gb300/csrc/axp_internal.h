@@ -183,6 +183,10 @@ struct axp_grid {
     // half_prev_cfg), so E^n follows cell by cell from the two levels
     bool half_prev;
     int64_t half_prev_cfg;
+    // the time-blocked 1D kernel's last launch left E^n of the present staggered state in
+    // the current's scratch (at configuration en_scratch_cfg)
+    bool en_scratch;
+    int64_t en_scratch_cfg;
     // attached macroparticles (Sec. 2.2), or null; a grid with particles takes the
     // general path
     axp::Particles *parts;

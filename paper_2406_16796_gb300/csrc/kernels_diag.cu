@@ -6,10 +6,12 @@
 // block sums the partials in fixed order.  The result depends only on the
 // grid size, never on scheduling, so a grid's diagnostics are bit-identical
 // however the work around it is arranged.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <mutex>
 
+#include "cells.cuh"
 #include "device_common.cuh"
 
 namespace axp {
@@ -18,6 +20,343 @@ namespace {
 constexpr int kDiagThreads = 256;
 constexpr int kQ = 7;  // H_phi, H_g0, H_g1, cross, sum x B1z^2, sum B1z^2, gauss
 
+// ---------------------------------------------------------------------------
+// Sums over the grid (the regular entry points).  What bounds it: a literal double
+// evaluation spends most of its time on GB300's narrow FP64 pipe (2 operations per
+// cycle per SM: 36.7 ms for the 512^3 FP32 box, whose 8 arrays cross HBM in 0.7 ms).
+//  * Only the components that can be non-zero are read (template masks).
+//  * Constants (1/2, dV, 1/d^2, m^2, 1/dt^2) are applied to the sums, not per cell.
+//  * FP64 grids work in double.  FP32 grids work in pairs of floats (a value as the
+//    sum hi + lo of two floats, 48 bits; error-free sums and products after Dekker and
+//    Knuth, products by fma), on the FP32 pipe that is 64 times wider.  Each input is an
+//    exact float, so the pairs hold differences and squares of them as a double would
+//    to 2^-48, and a thread's partial sum is turned into a double once.
+//  * Floats span less than squares of small fields need, so each group of fields is
+//    scaled by a power of two taken from its largest magnitude in the region (max_group:
+//    a pass of its own, or part of the pass that forms E^n).  Scaling by a power of
+//    two is exact; what then underflows is below 2^-60 of the largest value.
+// Measured (us, before -> after): 512^3 FP32 box DIAG_A3; 4096 x 2048 pulse FP32 DIAG_P32,
+// FP64 DIAG_P64.
+// ---------------------------------------------------------------------------
+struct FF {
+    float h, l;
+};
+__device__ __forceinline__ FF two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ FF quick_sum(float a, float b)  // |a| >= |b|
+{
+    const float s = __fadd_rn(a, b);
+    return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ FF operator+(FF a, FF b)
+{
+    const FF s = two_sum(a.h, b.h);
+    return quick_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ FF operator*(FF a, FF b)
+{
+    const float p = __fmul_rn(a.h, b.h);
+    const float e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)));
+    return quick_sum(p, e);
+}
+__device__ __forceinline__ FF operator*(FF a, float b)
+{
+    const float p = __fmul_rn(a.h, b);
+    return quick_sum(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+
+// a running sum of pairs: the high words by an error-free sum, the low words as they come
+// (the pair is normalised once, when the thread's sum becomes a double)
+__device__ __forceinline__ void accumulate(FF &acc, FF x)
+{
+    const FF s = two_sum(acc.h, x.h);
+    acc.h = s.h;
+    acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, x.l));
+}
+__device__ __forceinline__ void accumulate(double &acc, double x) { acc = acc + x; }
+
+// Sums of 7 quantities over a warp: at each of the first three steps a lane keeps half of
+// its values and adds its partner's, so 9 additions take the place of 35 (an FP64
+// addition holds its SM sub-partition's unit for 64 cycles).  Lane 4 k holds quantity k.
+__device__ __forceinline__ double warp_sums(double v[8], int lane)
+{
+#pragma unroll
+    for (int h = 4, w = 16; h >= 1; h >>= 1, w >>= 1) {
+        const bool upper = lane & w;
+#pragma unroll
+        for (int i = 0; i < h; i++) {
+            const double give = upper ? v[i] : v[i + h], keep = upper ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, w);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+}
+// the block's sums into sh[quantity][warp] (then a __syncthreads), and their total over warps
+__device__ __forceinline__ void block_sums(double v[8], double sh[8][kDiagThreads / 32])
+{
+    const int lane = threadIdx.x % 32;
+    const double t = warp_sums(v, lane);
+    if (lane % 4 == 0) sh[lane / 4][threadIdx.x / 32] = t;
+    __syncthreads();
+}
+
+// the arithmetic of the sums: V holds a term, from values T
+template <typename T>
+struct Ops;
+template <>
+struct Ops<double> {
+    using V = double;
+    static __device__ __forceinline__ V of(double a) { return a; }
+    static __device__ __forceinline__ V diff(double a, double b) { return a - b; }
+    static __device__ __forceinline__ V prod(double a, double b) { return a * b; }
+    static __device__ __forceinline__ V square(V a) { return a * a; }
+    static __device__ __forceinline__ double total(V a) { return a; }
+    static __device__ __forceinline__ double scaled(double a, double) { return a; }
+};
+template <>
+struct Ops<float> {
+    using V = FF;
+    static __device__ __forceinline__ V of(float a) { return {a, 0.0f}; }
+    static __device__ __forceinline__ V diff(float a, float b) { return two_sum(a, -b); }
+    static __device__ __forceinline__ V prod(float a, float b)
+    {
+        const float p = __fmul_rn(a, b);
+        return {p, __fmaf_rn(a, b, -p)};
+    }
+    static __device__ __forceinline__ V square(V a)  // (not normalised: for accumulate)
+    {
+        const float p = __fmul_rn(a.h, a.h);
+        return {p, __fmaf_rn(__fadd_rn(a.h, a.h), a.l, __fmaf_rn(a.h, a.h, -p))};
+    }
+    static __device__ __forceinline__ double total(V a) { return (double)a.h + (double)a.l; }
+    static __device__ __forceinline__ float scaled(float a, float s) { return __fmul_rn(a, s); }
+};
+
+template <typename T>
+struct Sums {
+    const T *E0[3], *B0[3], *E1[3], *B1[3];
+    const T *phi, *phib;               // phi^{n+1/2}; phi^{n-1/2}, or the increment (FP32 split)
+    const T *gh[3][2], *gh_old[3][2];  // outflow ghosts of the two levels
+    int n[3], per[3], axbc[3][2];
+    int lo[3], hi[3];                  // the region summed
+    unsigned N;
+    T Bext[3], Eext[3];
+    int ext;                           // bits: non-zero background components, E (0-2) and B (3-5)
+    double d[3], lo0, dt, g, m2;
+    unsigned *top;      // FP32: largest magnitude of E0/B0, E1/B1, phi (float bits)
+    double *partials;
+    axp_diag *out;
+    int64_t step;
+};
+
+constexpr int kSums = 11;  // phi: Dt^2, mid^2, 3 forward differences; E0B0^2; E1B1^2 less B1z; cross; x B1z^2; B1z^2; R^2
+
+// a power of two near 1 / (largest magnitude), kept well inside the floats' range
+__device__ __forceinline__ float scale_of(double top)
+{
+    if (!(top > 0.0) || !isfinite(top)) return 1.0f;
+    return exp2f((float)min(max(-ilogb(top), -100), 100));
+}
+
+// phi^n of a neighbour: phi^n itself in FP32 split, 2 phi^n (the levels' sum) in FP64
+template <typename T, int MASK>
+__device__ __forceinline__ T mid_at(const Sums<T> &s, int a, int side, const Cell &q)
+{
+    constexpr bool INCR = sizeof(T) == 4;
+    const bool in = side ? q.hu[a] : q.hd[a];
+    const int bc = s.axbc[a][side];
+    if (in || bc == AXP_BC_REFLECT) {
+        const int c = in ? (side ? q.up[a] : q.dn[a]) : q.c;
+        return INCR ? s.phi[c] - T(0.5) * s.phib[c] : s.phi[c] + s.phib[c];
+    }
+    if (bc != AXP_BC_OUTFLOW) return T(0);
+    const int pi = ghost_index(s.n, a, q);
+    const T sum = s.gh[a][side][pi] + s.gh_old[a][side][pi];
+    return INCR ? T(0.5) * sum : sum;
+}
+
+// EM, BM: the order-0 components present
+template <typename T, int MASK, int EM, int BM>
+__global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 ? 3 : 4) k_diag_sums(Sums<T> s)
+{
+    using O = Ops<T>;
+    using V = typename O::V;
+    constexpr bool INCR = sizeof(T) == 4;
+    // scales: of phi, of the order-0 and order-1 fields, of the order-0 fields with the
+    // background, and of the Gauss residual (1 in double)
+    T sp = T(1), s0 = T(1), s1 = T(1), sx = T(1), sr = T(1);
+    if (INCR) {
+        const double t0 = __uint_as_float(s.top[0]), t1 = __uint_as_float(s.top[1]), tp = __uint_as_float(s.top[2]);
+        double ext = 0.0;
+        for (int a = 0; a < 3; a++) ext = max(ext, max(fabs((double)s.Bext[a]), fabs((double)s.Eext[a])));
+        sp = scale_of(tp);
+        s0 = scale_of(t0);
+        s1 = scale_of(t1);
+        sx = scale_of(max(t0, ext));
+        sr = scale_of(max(t1, fabs(s.g) * max(t0, ext) * tp));
+    }
+    V acc[kSums];
+#pragma unroll
+    for (int k = 0; k < kSums; k++) acc[k] = O::of(T(0));
+    V rd[3], kg;  // 1/d, and g/2 times the Gauss sum's scale over phi's
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const double x = 1.0 / s.d[a];
+        if constexpr (INCR) rd[a] = {(float)x, (float)(x - (double)(float)x)};
+        else rd[a] = x;
+    }
+    constexpr double half = INCR ? 1.0 : 0.5;  // phi^n over what mid_at gives
+    const double kd = half * 0.5 * s.g * ((double)sr / (double)sp);
+    if constexpr (INCR) kg = {(float)kd, (float)(kd - (double)(float)kd)};
+    else kg = kd;
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < s.N; c += gridDim.x * blockDim.x) {
+        Cell q;
+        cell_of_index<MASK>(s.n, s.per, c, q);
+        bool in = true;
+#pragma unroll
+        for (int a = 0; a < 3; a++) in = in && q.x[a] >= s.lo[a] && q.x[a] < s.hi[a];
+        if (!in) continue;
+        const T hi = s.phi[c], b = s.phib[c];
+        const T mid = O::scaled(INCR ? hi - T(0.5) * b : hi + b, sp);
+        if constexpr (INCR) accumulate(acc[0], O::prod(O::scaled(b, sp), O::scaled(b, sp)));
+        else accumulate(acc[0], O::square(O::diff(hi, b)));
+        accumulate(acc[1], O::prod(mid, mid));
+        V R = O::of(T(0));
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            if (!(MASK >> a & 1)) continue;
+            const T up = O::scaled(mid_at<T, MASK>(s, a, 1, q), sp), dn = O::scaled(mid_at<T, MASK>(s, a, 0, q), sp);
+            accumulate(acc[2 + a], O::square(O::diff(up, mid)));
+            // div E1 + g Bbar0 . grad_c phi, term by term along the axis
+            V t = O::diff(O::scaled(s.E1[a][c], sr), O::scaled(ldz(s.E1[a], q.dn[a], q.hd[a]), sr));
+            T bb = s.Bext[a];
+            if (BM >> a & 1) {
+                const int p = (a + 1) % 3, r = (a + 2) % 3;
+                const T *B = s.B0[a];
+                constexpr bool all = MASK == 7;
+                T f = B[c], w = T(1);  // (along an inactive axis the neighbour is the cell itself)
+                if (all || (MASK >> p & 1)) {
+                    f = f + ldz(B, q.dn[p], q.hd[p]);
+                    w = T(0.5);
+                }
+                if (all || (MASK >> r & 1)) {
+                    T h = ldz(B, q.dn[r], q.hd[r]);
+                    if (all || (MASK >> p & 1)) h = h + ldz(B, q.dn[p] + (q.dn[r] - q.c), q.hd[p] && q.hd[r]);
+                    f = f + h;
+                    w = w * T(0.5);
+                }
+                bb = w * f + bb;
+            }
+            if ((BM >> a & 1) || (s.ext >> (3 + a) & 1)) t = t + (O::diff(up, dn) * kg) * bb;
+            R = R + t * rd[a];
+        }
+        accumulate(acc[10], O::square(R));
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const T e1 = O::scaled(s.E1[a][c], s1), b1 = O::scaled(s.B1[a][c], s1);
+            accumulate(acc[6], O::prod(e1, e1));
+            const V bb = O::prod(b1, b1);
+            if (a < 2) {
+                accumulate(acc[6], bb);
+            } else {
+                accumulate(acc[9], bb);
+                accumulate(acc[8], bb * T(q.x[0] + 1));
+            }
+            if (EM >> a & 1) {
+                const T e0 = s.E0[a][c];
+                accumulate(acc[5], O::prod(O::scaled(e0, s0), O::scaled(e0, s0)));
+                accumulate(acc[7], O::diff(O::scaled(e0, sx), -O::scaled(s.Eext[a], sx)) * e1);
+            } else if (s.ext >> a & 1) {
+                accumulate(acc[7], O::prod(O::scaled(s.Eext[a], sx), e1));
+            }
+            if (BM >> a & 1) {
+                const T b0 = s.B0[a][c];
+                accumulate(acc[5], O::prod(O::scaled(b0, s0), O::scaled(b0, s0)));
+                accumulate(acc[7], O::diff(O::scaled(b0, sx), -O::scaled(s.Bext[a], sx)) * b1);
+            } else if (s.ext >> (3 + a) & 1) {
+                accumulate(acc[7], O::prod(O::scaled(s.Bext[a], sx), b1));
+            }
+        }
+    }
+    // each thread's sums as doubles, the scales undone; then a fixed tree over the block
+    const double up = 1.0 / ((double)sp * (double)sp), u0 = 1.0 / ((double)s0 * (double)s0);
+    const double u1 = 1.0 / ((double)s1 * (double)s1), ux = 1.0 / ((double)sx * (double)s1), ur = 1.0 / ((double)sr * (double)sr);
+    const double dV = s.d[0] * s.d[1] * s.d[2];
+    double tot[8];
+    tot[7] = 0.0;
+    double hphi = O::total(acc[0]) / (s.dt * s.dt) + s.m2 * half * half * O::total(acc[1]);
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+        if (MASK >> a & 1) hphi += half * half * O::total(acc[2 + a]) / (s.d[a] * s.d[a]);
+    const double bz2 = O::total(acc[9]) * u1;
+    tot[0] = 0.5 * dV * up * hphi;
+    tot[1] = 0.5 * dV * u0 * O::total(acc[5]);
+    tot[2] = 0.5 * dV * (u1 * O::total(acc[6]) + bz2);
+    tot[3] = dV * ux * O::total(acc[7]);
+    tot[4] = dV * (s.lo0 * bz2 + s.d[0] * u1 * O::total(acc[8]));
+    tot[5] = dV * bz2;
+    tot[6] = dV * ur * O::total(acc[10]);
+    __shared__ double sh[8][kDiagThreads / 32];
+    block_sums(tot, sh);
+    if (threadIdx.x < kQ) {
+        double t = 0.0;
+        for (int w = 0; w < kDiagThreads / 32; w++) t += sh[threadIdx.x][w];
+        s.partials[(int64_t)blockIdx.x * kQ + threadIdx.x] = t;
+    }
+}
+
+// largest magnitudes by group, as float bits (of non-negative floats: their order);
+// NaN and infinity come out above every finite value
+__device__ __forceinline__ unsigned mag(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+__device__ __forceinline__ void max_group(unsigned *top, unsigned m0, unsigned m1, unsigned mp)
+{
+    m0 = __reduce_max_sync(0xffffffffu, m0);
+    m1 = __reduce_max_sync(0xffffffffu, m1);
+    mp = __reduce_max_sync(0xffffffffu, mp);
+    if (threadIdx.x % 32 == 0) {
+        if (m0) atomicMax(top, m0);
+        if (m1) atomicMax(top + 1, m1);
+        if (mp) atomicMax(top + 2, mp);
+    }
+}
+template <typename T>
+__device__ __forceinline__ void max_of_cell(const Sums<T> &s, int64_t c, uint32_t mask, bool with_e, unsigned &m0, unsigned &m1,
+                                            unsigned &mp)
+{
+    if constexpr (sizeof(T) == 4) {
+        for (int a = 0; a < 3; a++) {
+            if (with_e && (mask >> a & 1u)) m0 = max(m0, mag(s.E0[a][c]));
+            if (mask >> (3 + a) & 1u) m0 = max(m0, mag(s.B0[a][c]));
+            if (with_e) m1 = max(m1, mag(s.E1[a][c]));
+            m1 = max(m1, mag(s.B1[a][c]));
+        }
+        mp = max(mp, max(mag(s.phi[c]), mag(s.phib[c])));
+    }
+}
+
+// the magnitudes alone, over the region's cells (mask: order-0 components present)
+template <typename T>
+__global__ void __launch_bounds__(kDiagThreads) k_diag_max(Sums<T> s, uint32_t mask)
+{
+    unsigned m0 = 0, m1 = 0, mp = 0;
+    const unsigned n0 = s.n[0], n1 = s.n[1];
+    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < s.N; c += gridDim.x * blockDim.x) {
+        const unsigned r = c / n0, k = r / n1;
+        const int x[3] = {(int)(c - r * n0), (int)(r - k * n1), (int)k};
+        bool in = true;
+#pragma unroll
+        for (int a = 0; a < 3; a++) in = in && x[a] >= s.lo[a] && x[a] < s.hi[a];
+        if (in) max_of_cell(s, c, mask, true, m0, m1, mp);
+    }
+    max_group(s.top, m0, m1, mp);
+}
+
+// the literal evaluation (fields of a caller, and grids of 2^30 cells or more)
 template <typename T, bool INCR>
 __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(View<T> v, PhiPair<T, INCR> q, double *partials)
 {
@@ -86,37 +425,36 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(View<T> v, PhiPai
 }
 
 __global__ void __launch_bounds__(kDiagThreads) k_diag_final(const double *partials, int nblocks, axp_diag *out,
-                                                             int64_t step, double t)
+                                                             int64_t step, double t, unsigned *top)
 {
-    __shared__ double sh[kQ][kDiagThreads];
-    double acc[kQ];
+    if (top && threadIdx.x < 3) top[threadIdx.x] = 0;  // for the next record's magnitudes
+    __shared__ double part[8][kDiagThreads / 32], sh[kQ];
+    double acc[8];
 #pragma unroll
-    for (int s = 0; s < kQ; s++) acc[s] = 0.0;
+    for (int s = 0; s < 8; s++) acc[s] = 0.0;
     for (int b = threadIdx.x; b < nblocks; b += kDiagThreads)
 #pragma unroll
         for (int s = 0; s < kQ; s++) acc[s] += partials[(int64_t)b * kQ + s];
-#pragma unroll
-    for (int s = 0; s < kQ; s++) sh[s][threadIdx.x] = acc[s];
-    __syncthreads();
-    for (int w = kDiagThreads / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int s = 0; s < kQ; s++) sh[s][threadIdx.x] += sh[s][threadIdx.x + w];
-        __syncthreads();
+    block_sums(acc, part);
+    if (threadIdx.x < kQ) {
+        double t = 0.0;
+        for (int w = 0; w < kDiagThreads / 32; w++) t += part[threadIdx.x][w];
+        sh[threadIdx.x] = t;
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
         axp_diag d;
         d.step = step;
         d.t = t;
-        d.H_phi = sh[0][0];
-        d.H_g0 = sh[1][0];
-        d.H_g1 = sh[2][0];
+        d.H_phi = sh[0];
+        d.H_g0 = sh[1];
+        d.H_g1 = sh[2];
         d.P_g2a = d.H_g0 > 0 ? d.H_phi / d.H_g0 : 0.0;
         d.P_a2g = d.H_phi > 0 ? d.H_g1 / d.H_phi : 0.0;
-        d.W = d.H_phi + sh[3][0];
-        d.sum_xB1z2 = sh[4][0];
-        d.sum_B1z2 = sh[5][0];
-        d.gauss_l2 = sh[6][0];
+        d.W = d.H_phi + sh[3];
+        d.sum_xB1z2 = sh[4];
+        d.sum_B1z2 = sh[5];
+        d.gauss_l2 = sh[6];
         *out = d;
     }
 }
@@ -155,33 +493,110 @@ struct ELevels {
     const T *hi[6];  // E^{n+1/2}
     const T *a1[3];  // per axis, the one-half-step layer coefficient a (null: no layer along the axis)
     unsigned mask;   // arrays to form
+    int lay[3][2];   // cells of absorbing layer at each side
     int64_t n0, n1, n2;
 };
 
-template <typename T>
-__global__ void __launch_bounds__(kDiagThreads) k_e_level(ELevels<T> L)
+template <typename T, typename I>
+__global__ void __launch_bounds__(kDiagThreads) k_e_level(ELevels<T> L, Sums<T> s, uint32_t mask)
 {
-    const int64_t rows = L.n1 * L.n2;
-    for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
-        const int64_t j = r % L.n1, k = r / L.n1;
-        T ayz = T(1);
-        if (L.a1[1] && L.a1[1][j] < ayz) ayz = L.a1[1][j];
-        if (L.a1[2] && L.a1[2][k] < ayz) ayz = L.a1[2][k];
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < L.n0; i += (int64_t)gridDim.x * blockDim.x) {
-            T a = ayz;
-            if (L.a1[0] && L.a1[0][i] < a) a = L.a1[0][i];
-            const int64_t c = i + L.n0 * r;
+    unsigned m0 = 0, m1 = 0, mp = 0;  // FP32: the region's largest magnitudes on the way
+    const I N = (I)L.n0 * (I)L.n1 * (I)L.n2, n0 = (I)L.n0, n1 = (I)L.n1;
+    for (I c = (I)blockIdx.x * blockDim.x + threadIdx.x; c < N; c += (I)gridDim.x * blockDim.x) {
+        const I r = c / n0, k = r / n1;
+        const int x[3] = {(int)(c - r * n0), (int)(r - k * n1), (int)k};
+        bool layer = false, in = sizeof(T) == 4 && s.top;
 #pragma unroll
-            for (int f = 0; f < 6; f++) {
-                if (!(L.mask >> f & 1u)) continue;
-                L.lo[f][c] = a == T(1) ? T(0.5) * (L.hi[f][c] + L.lo[f][c]) : (L.hi[f][c] + a * L.lo[f][c]) / (T(1) + a);
+        for (int a = 0; a < 3; a++) {
+            layer = layer || x[a] < L.lay[a][0] || x[a] >= s.n[a] - L.lay[a][1];
+            in = in && x[a] >= s.lo[a] && x[a] < s.hi[a];
+        }
+        T a1 = T(1), inv = T(0.5);
+        if (layer) {
+#pragma unroll
+            for (int a = 0; a < 3; a++)
+                if (L.a1[a]) a1 = min(a1, L.a1[a][x[a]]);
+            inv = T(1) / (T(1) + a1);
+        }
+#pragma unroll
+        for (int f = 0; f < 6; f++) {
+            if (!(L.mask >> f & 1u)) continue;
+            const T hi = L.hi[f][c], lo = L.lo[f][c];
+            T e = hi + lo;
+            if (layer) e = hi + a1 * lo;
+            e = e * inv;
+            L.lo[f][c] = e;
+            if constexpr (sizeof(T) == 4) {
+                if (in && f < 3) m0 = max(m0, mag(e));
+                if (in && f >= 3) m1 = max(m1, mag(e));
             }
         }
+        if (in) max_of_cell(s, c, mask, false, m0, m1, mp);
     }
+    if (sizeof(T) == 4 && s.top) max_group(s.top, m0, m1, mp);
 }
 
 template <typename T>
-cudaError_t e_level_from_halves(axp_grid *g)
+static Sums<T> make_sums(axp_grid *g, const View<T> &v)
+{
+    Sums<T> s;
+    for (int a = 0; a < 3; a++) {
+        s.E0[a] = v.f[kE0 + a];
+        s.B0[a] = v.f[kB0 + a];
+        s.E1[a] = v.f[kE1 + a];
+        s.B1[a] = v.f[kB1 + a];
+        for (int e = 0; e < 2; e++) {
+            s.gh[a][e] = v.gh[a][e][0];
+            s.gh_old[a][e] = v.gh[a][e][1];
+            s.axbc[a][e] = v.axbc[a][e];
+        }
+        s.n[a] = (int)v.n[a];
+        s.per[a] = v.periodic[a];
+        s.lo[a] = v.region_lo[a];
+        s.hi[a] = v.region_hi[a];
+        s.Bext[a] = v.Bext[a];
+        s.Eext[a] = v.Eext[a];
+        s.d[a] = (double)v.d[a];
+        s.ext = (a ? s.ext : 0) | (v.Eext[a] != T(0) ? 1 << a : 0) | (v.Bext[a] != T(0) ? 8 << a : 0);
+    }
+    s.phi = v.phi_cur;
+    s.phib = v.phi_b;
+    s.N = (unsigned)v.N;
+    s.lo0 = (double)v.lo[0];
+    s.dt = (double)v.dt;
+    s.g = (double)v.g;
+    s.m2 = (double)v.m2;
+    s.top = sizeof(T) == 4 ? (unsigned *)(g->ws + g->layout.off_flag) + 8 : nullptr;
+    s.partials = (double *)(g->ws + g->layout.off_partials);
+    return s;
+}
+
+// the kernel for the active axes and the order-0 components present (mask: bits 0-2 E0,
+// 3-5 B0)
+template <typename T>
+static void launch_sums(const Sums<T> &s, uint32_t mask, int nb, cudaStream_t st)
+{
+    const uint32_t tm = 4u | (3u << 3), te = 3u | (4u << 3);
+    const int set = mask == 0 ? 0 : (mask & ~tm) == 0 ? 1 : (mask & ~te) == 0 ? 2 : 3;
+#define AXP_SUMS(M)                                                                                        \
+    switch (set) {                                                                                         \
+    case 0: k_diag_sums<T, M, 0, 0><<<nb, kDiagThreads, 0, st>>>(s); break;                                \
+    case 1: k_diag_sums<T, M, 4, 3><<<nb, kDiagThreads, 0, st>>>(s); break;                                \
+    case 2: k_diag_sums<T, M, 3, 4><<<nb, kDiagThreads, 0, st>>>(s); break;                                \
+    default: k_diag_sums<T, M, 7, 7><<<nb, kDiagThreads, 0, st>>>(s); break;                               \
+    }
+    if (s.n[2] == 1 && s.n[1] == 1) {
+        AXP_SUMS(1)
+    } else if (s.n[2] == 1) {
+        AXP_SUMS(3)
+    } else {
+        AXP_SUMS(7)
+    }
+#undef AXP_SUMS
+}
+
+template <typename T>
+cudaError_t e_level_from_halves(axp_grid *g, const Sums<T> &s, uint32_t mask)
 {
     ELevels<T> L;
     const Workspace &w = g->layout;
@@ -197,14 +612,16 @@ cudaError_t e_level_from_halves(axp_grid *g)
     for (int a = 0; a < 3; a++) {
         const bool lay = g->desc.em_bc[a][0] != AXP_BC_PERIODIC && g->desc.pml_cells > 0 && g->desc.pml_sigma_max_dt > 0;
         L.a1[a] = lay ? (const T *)(g->ws + w.off_pml_tab[a]) : nullptr;
+        for (int e = 0; e < 2; e++)
+            L.lay[a][e] = lay && g->desc.em_bc[a][e] == AXP_BC_PML ? (int)std::min<int64_t>(g->desc.pml_cells, g->desc.n[a]) : 0;
     }
     L.n0 = g->desc.n[0];
     L.n1 = g->desc.n[1];
     L.n2 = g->desc.n[2];
-    const int64_t rows = L.n1 * L.n2;
-    dim3 grid((unsigned)((L.n0 + kDiagThreads - 1) / kDiagThreads), (unsigned)(rows < 65535 ? rows : 65535), 1);
-    if (grid.x > 64) grid.x = 64;
-    k_e_level<T><<<grid, kDiagThreads, 0, g->stream>>>(L);
+    const int64_t N = L.n0 * L.n1 * L.n2;
+    const unsigned nb = (unsigned)std::min<int64_t>((N + kDiagThreads - 1) / kDiagThreads, 152 * 8);
+    if (N < (int64_t)1 << 30) k_e_level<T, unsigned><<<nb, kDiagThreads, 0, g->stream>>>(L, s, mask);
+    else k_e_level<T, int64_t><<<nb, kDiagThreads, 0, g->stream>>>(L, s, mask);
     g->launches++;
     g->half_prev = false;  // the other set now holds E^n
     return cudaGetLastError();
@@ -219,29 +636,46 @@ cudaError_t diag_compute_rows(axp_grid *g, axp_diag *dev_dst, int axis, int64_t 
     // staggered (fused-path) state: reconstruct E^n into the spare field set first,
     // from the two levels of the last single-pass step where the other set holds
     // them, else by the general kernels' inverse half-step
-    View<T> v;
-    if (g->staggered) {
-        const bool halves = g->half_prev && g->half_prev_cfg == g->cfg_version;
-        const cudaError_t e = halves ? e_level_from_halves<T>(g) : exit_staggered<T>(g, false);
+    const bool halves = g->staggered && g->half_prev && g->half_prev_cfg == g->cfg_version;
+    // the time-blocked 1D kernel leaves E^n in the current's scratch (J: E0y, E0z, E1x; P: E1y, E1z)
+    const bool scratch = g->staggered && g->en_scratch && g->en_scratch_cfg == g->cfg_version;
+    const bool wide = (int64_t)g->desc.n[0] * g->desc.n[1] * g->desc.n[2] >= (int64_t)1 << 30;  // (64-bit indexes)
+    const uint32_t mask = order0_closure(g);
+    if (g->staggered && !halves && !scratch) {
+        const cudaError_t e = exit_staggered<T>(g, false);
         if (e != cudaSuccess) return e;
-        v = make_view_eset<T>(g, 1 - g->fset);
-    } else {
-        v = make_view<T>(g);
+    }
+    View<T> v = g->staggered && !scratch ? make_view_eset<T>(g, 1 - g->fset) : make_view<T>(g);
+    if (scratch) {
+        const Workspace &w = g->layout;
+        const size_t off[5] = {w.off_J[0], w.off_J[1], w.off_J[2], w.off_P[0], w.off_P[1]};
+        const int f[5] = {kE0 + 1, kE0 + 2, kE1, kE1 + 1, kE1 + 2};
+        for (int q = 0; q < 5; q++) v.f[f[q]] = (T *)(g->ws + off[q]);
     }
     if (axis >= 0) {
         if (lo > v.region_lo[axis]) v.region_lo[axis] = (int)lo;
         if (hi < v.region_hi[axis]) v.region_hi[axis] = (int)hi;
     }
-    double *partials = (double *)(g->ws + g->layout.off_partials);
-    const int nb = g->layout.diag_blocks;
-    if (g->desc.precision == AXP_FP32_SPLIT) {
-        PhiPair<T, true> q{v.phi_cur, v.phi_b, ghosts_lvl<T>(g, 0), ghosts_lvl<T>(g, 1)};
-        k_diag_partial<T, true><<<nb, kDiagThreads, 0, g->stream>>>(v, q, partials);
-    } else {
-        PhiPair<T, false> q{v.phi_cur, v.phi_b, ghosts_lvl<T>(g, 0), ghosts_lvl<T>(g, 1)};
-        k_diag_partial<T, false><<<nb, kDiagThreads, 0, g->stream>>>(v, q, partials);
+    Sums<T> s = make_sums<T>(g, v);
+    if (wide) s.top = nullptr;
+    if (halves) {
+        const cudaError_t e = e_level_from_halves<T>(g, s, mask);
+        if (e != cudaSuccess) return e;
+    } else if (s.top) {
+        const unsigned grid = std::min<unsigned>((s.N + kDiagThreads - 1) / kDiagThreads, 152 * 8);
+        k_diag_max<T><<<grid, kDiagThreads, 0, g->stream>>>(s, mask);
+        g->launches++;
     }
-    k_diag_final<<<1, kDiagThreads, 0, g->stream>>>(partials, nb, dev_dst, g->step, (double)g->step * g->desc.dt);
+    double *partials = s.partials;
+    // one wave of blocks (4 per SM; FP32: 3): a wave and a part of the next costs two
+    const int nb = wide ? g->layout.diag_blocks : std::min(g->layout.diag_blocks, 152 * (sizeof(T) == 4 ? 3 : 4));
+    if (wide) {
+        PhiPair<T, sizeof(T) == 4> q{v.phi_cur, v.phi_b, ghosts_lvl<T>(g, 0), ghosts_lvl<T>(g, 1)};
+        k_diag_partial<T, sizeof(T) == 4><<<nb, kDiagThreads, 0, g->stream>>>(v, q, partials);
+    } else {
+        launch_sums<T>(s, mask, nb, g->stream);
+    }
+    k_diag_final<<<1, kDiagThreads, 0, g->stream>>>(partials, nb, dev_dst, g->step, (double)g->step * g->desc.dt, s.top);
     g->launches += 2;
     return cudaGetLastError();
 }
@@ -368,7 +802,7 @@ extern "C" axp_status axp_diagnostics_noalloc(const axp_grid_desc *desc, const d
     int nb = (int)((N + kNoallocCellsPerBlock - 1) / kNoallocCellsPerBlock);
     if (nb < 1) nb = 1;
     k_diag_partial<double, false><<<nb, kDiagThreads, 0, stream>>>(v, q, partials);
-    k_diag_final<<<1, kDiagThreads, 0, stream>>>(partials, nb, result, step, (double)step * desc->dt);
+    k_diag_final<<<1, kDiagThreads, 0, stream>>>(partials, nb, result, step, (double)step * desc->dt, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(host_out, result, sizeof(axp_diag), cudaMemcpyDeviceToHost, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);

@@ -305,6 +305,8 @@ cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
     A.q4dx = 1.0 / (4.0 * dx);
     for (int a = 0; a < 3; a++) A.Bext[a] = g->B_ext[a];
     const Workspace &w = g->layout;
+    const size_t en[5] = {w.off_J[0], w.off_J[1], w.off_J[2], w.off_P[0], w.off_P[1]};
+    for (int q = 0; q < 5; q++) A.En[q] = (double *)(g->ws + en[q]);
     A.ctr = (unsigned *)(g->ws + w.off_flag);
     A.err = (int *)(g->ws + w.off_flag) + 1;  // read (and cleared) by the next synchronising call
     A.absent = g->coop_absent;
@@ -340,6 +342,8 @@ cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
             std::swap(g->phi_b_slot, g->phi_next_b_slot);
         }
         g->step += k;
+        g->en_scratch = true;
+        g->en_scratch_cfg = g->cfg_version;
         left -= k;
         if (d.diag_every > 0 && g->step % d.diag_every == 0) {
             axp_diag *dst = ring_slot(g, g->ring_written);
@@ -852,6 +856,7 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     // AUTO runs the folded passes on the same staggered state where they are faster: in
     // place of the generic kernel in 2D and 3D, and on small FP64 grids of the 2D kernel
     const bool small_tm = tm && sizeof(T) == 8 && g->desc.n[0] * g->desc.n[1] <= kSmallTm;
+    g->en_scratch = false;
     if (g->kernel_choice == AXP_KERNEL_AUTO && (small_tm || (path == AXP_KERNEL_FUSED && mode >= 2)) && staged_supported(g))
         return staged_step<T>(g, nsteps);
     int tm_tx = tm2d::TX;  // tile width of the 2D kernel (chosen below)

@@ -59,6 +59,7 @@ struct Args {
     double Bext[3];
     unsigned *ctr;  // grid-wait arrivals (zeroed before the launch)
     int *err;       // 1 once a wait gave up
+    double *En[5];  // E at the integer time the launch ends at: E0 y z, E1 x y z
     int absent;     // failure-detection test: this block leaves before its first wait (-1: none)
 };
 
@@ -226,6 +227,15 @@ __global__ void __launch_bounds__(kThreads) k_line1d(Args A)
             }
             A.phi[1 - par][0][gi] = cur[w];
             A.phi[1 - par][1][gi] = old[w];
+            if (done + A.tblock >= A.nsteps) {
+                // E^{n+1} of the last step, for a record taken here: E1 less the second of
+                // its two half-steps, E0 as the step formed it
+                A.En[0][gi] = Eny[w];
+                A.En[1][gi] = Enz[w];
+                A.En[2][gi] = fma(0.5 * A.h2g, 0.5 * (Px[w] + at(Px, w + 1)), E[3][w]);
+                A.En[3][gi] = fma(A.cB, B[5][w] - at(B[5], w - 1), fma(0.5 * A.h2g, PY[w], E[4][w]));
+                A.En[4][gi] = fma(-A.cB, B[4][w] - at(B[4], w - 1), fma(0.5 * A.h2g, PZ[w], E[5][w]));
+            }
         }
         par ^= 1;
         if (done + A.tblock < A.nsteps) {

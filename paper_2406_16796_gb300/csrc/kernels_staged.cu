@@ -32,6 +32,7 @@
 // ncu: the FP64 passes keep the FP64 pipe 76-84% busy while an SM is active.
 #include <algorithm>
 
+#include "cells.cuh"
 #include "device_common.cuh"
 
 namespace axp {
@@ -94,43 +95,14 @@ void launch_pass(void (*kern)(KArgs...), int blocks, cudaStream_t st, const Args
     cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);  // (errors: the caller's cudaGetLastError)
 }
 
-// A cell's index, its neighbours' (wrapped along periodic axes) and whether they exist.
-struct Cell {
-    int c, x[3];
-    int up[3], dn[3];
-    bool hu[3], hd[3];
-};
-
+// this thread's cell
 template <int MASK, typename T>
 __device__ __forceinline__ bool cell_at(const Stage<T> &s, Cell &q)
 {
     const unsigned c = blockIdx.x * (unsigned)kThreads + threadIdx.x;
     if (c >= (unsigned)s.N) return false;
-    const unsigned n0 = s.n[0], n1 = s.n[1];
-    const unsigned r = c / n0;
-    q.c = (int)c;
-    q.x[0] = (int)(c - r * n0);
-    q.x[1] = (MASK & 4) ? (int)(r % n1) : (int)r;
-    q.x[2] = (MASK & 4) ? (int)(r / n1) : 0;
-    const int stride[3] = {1, s.n[0], s.n[0] * s.n[1]};
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        q.up[a] = q.dn[a] = q.c;
-        q.hu[a] = q.hd[a] = true;
-        if (!(MASK >> a & 1)) continue;
-        const int wrap = (s.n[a] - 1) * stride[a];
-        if (q.x[a] + 1 < s.n[a]) q.up[a] = q.c + stride[a];
-        else { q.up[a] = q.c - wrap; q.hu[a] = s.per[a]; }
-        if (q.x[a] > 0) q.dn[a] = q.c - stride[a];
-        else { q.dn[a] = q.c + wrap; q.hd[a] = s.per[a]; }
-    }
+    cell_of_index<MASK>(s.n, s.per, c, q);
     return true;
-}
-
-template <typename T>
-__device__ __forceinline__ T ldz(const T *__restrict__ F, int c, bool ok)
-{
-    return ok ? F[c] : T(0);
 }
 
 // h (curl F)_a with differences towards `up` (forward) or from `dn` (backward):
@@ -279,8 +251,7 @@ __device__ __forceinline__ T phi_nb(const Stage<T> &s, const T *__restrict__ F, 
     const int bc = s.axbc[a][side];
     if (bc == AXP_BC_REFLECT) return F[q.c];
     if (bc != AXP_BC_OUTFLOW) return T(0);
-    const int pi = a == 0 ? q.x[1] + s.n[1] * q.x[2] : (a == 1 ? q.x[0] + s.n[0] * q.x[2] : q.x[0] + s.n[0] * q.x[1]);
-    return gh[a][side][pi];
+    return gh[a][side][ghost_index(s.n, a, q)];
 }
 
 // The outflow ghost next to cell q on one face, at the new level (Sec. 2.4 item 3): the
@@ -303,7 +274,7 @@ __device__ void outflow_ghost(const Stage<T> &s, const T *const Bs[3], int ax, i
         }
         S = fma(e, b, S);
     }
-    const int pi = ax == 0 ? q.x[1] + s.n[1] * q.x[2] : (ax == 1 ? q.x[0] + s.n[0] * q.x[2] : q.x[0] + s.n[0] * q.x[1]);
+    const int pi = ghost_index(s.n, ax, q);
     const T gc = s.gh[ax][side][pi], go = s.gh_old[ax][side][pi], r = s.of_r[ax];
     T rhs = fma(T(2), go - gc, fma(s.m2dt2, gc, -(s.dt2g * S)));
     rhs = fma(r, p0, rhs) - r * r * fma(T(-2), gc, p0);

@@ -26,6 +26,7 @@ CASES = {
     "2d_outflow_mixed": (dict(n=(36, 31, 1), B=(0.0, 0.4, 1.0), ax=bcs("outflow", ("reflect", "pml")),
                               em=bcs("pml", ("reflect", "pml")), E=(0.1, 0.0, -0.05)), None, 1),
     "2d_te_pml": (dict(n=(75, 44, 1), B=(0.2, 0.9, 0.0), ax=bcs("pml", "pml"), em=bcs("pml", "pml")), TE, 2),
+    "2d_tm_pml": (dict(n=(61, 37, 1), B=(0.0, 0.0, 1.0), ax=bcs("pml", "pml"), em=bcs("pml", "pml")), TM, None),
     "2d_te_periodic": (dict(n=(50, 33, 1), B=(0.2, 0.9, 0.3)), TE, 2),
     "2d_all_reflect": (dict(n=(45, 29, 1), B=(0.2, 0.9, 0.3), ax=bcs("reflect", "pml"), em=bcs("reflect", "pml")), None, 2),
     "2d_no_laser_reflect": (dict(n=(45, 29, 1), B=(0.2, 0.9, 0.3), ax=bcs("reflect", "pml"), em=bcs("reflect", "pml")),
