@@ -405,7 +405,8 @@ axp_status axp_get_window_offset(const axp_grid *grid, int64_t *cells);
  * 1e-12 of the literal ones in FP64; reported as AXP_KERNEL_GENERAL).  The same
  * passes step the staggered state of the generic kernel's 2D and 3D grids and of
  * the 2D TM kernel's small FP64 grids, where they are faster; the path reported
- * is then still that kernel's, whose state it is.
+ * is then still that kernel's, whose state it is.  Likewise 1D grids in FP32 split
+ * or with absorbing ends run on the time-blocked 1D kernel and report the generic one.
  * AXP_KERNEL_GENERAL forces the general kernels (one pass per stage of the
  * time scheme, in the oracle's operation order); AXP_KERNEL_FUSED forces the
  * generic single-pass kernel (1D/2D/3D, periodic, reflect and PML edges);

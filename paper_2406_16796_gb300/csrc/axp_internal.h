@@ -230,9 +230,8 @@ void particles_layout(const axp_grid_desc &d, Particles *P);
 cudaError_t particles_start(axp_grid *g);
 cudaError_t particles_push(axp_grid *g, const View<double> &v);
 cudaError_t particles_now(axp_grid *g);
-// time-blocked 1D kernel (FP64, periodic): eligibility and steps on the integer-time state
+// whether AXP_KERNEL_BLOCK1D (the time-blocked kernel of periodic FP64 1D grids) takes the grid
 bool block1d_supported(const axp_grid *g);
-cudaError_t block1d_step(axp_grid *g, int64_t nsteps);
 template <typename T>
 bool fused_supported(const axp_grid *g);
 // the path axp_step will take under the handle's kernel choice (an axp_kernel value)

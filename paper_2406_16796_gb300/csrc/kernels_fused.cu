@@ -27,6 +27,9 @@ cudaError_t ax3d_dispatch_f32(const fused::Params<float> &P, int nchunks, cudaSt
 
 namespace {
 
+// largest 1D grid that takes the time-blocked kernel in place of the generic one
+constexpr int64_t kLineMost = 1 << 17;
+
 constexpr uint32_t kSets[4] = {0u, (4u) | (3u << 3), (3u) | (4u << 3), 63u};
 
 int grid_mode(const axp_grid *g)
@@ -240,73 +243,110 @@ bool fused_supported(const axp_grid *g)
     return true;
 }
 
-// steps per block of the time-blocked 1D kernel (halo tblock + 3 on each side):
-// with 4096 cells over 152 SMs a window of 27 + 2 x 18 cells fits one pass of
-// the kernel's 64 cells (T = 12, 14, 15 measured 1.80, 1.77, 1.76 us/step; from
-// 16 the window takes two passes)
-#ifndef AXP_LINE_BLOCK
-#define AXP_LINE_BLOCK 15
-#endif
-constexpr int kLineBlock = AXP_LINE_BLOCK;
-// blocks per SM of the time-blocked 1D kernel (each owns n / (SMs x this) cells)
-#ifndef AXP_LINE_BLOCKS_PER_SM
-#define AXP_LINE_BLOCKS_PER_SM 1
-#endif
-constexpr int kLineBlocksPerSM = AXP_LINE_BLOCKS_PER_SM;
+// The time-blocked 1D kernel owns n / SMs cells per block.
+int64_t line_seg(const axp_grid *g)
+{
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess || sms < 1) return -1;
+    return (g->desc.n[0] + sms - 1) / sms;
+}
 
-// Which grids take the time-blocked 1D kernel: FP64, 1D and periodic along x,
-// no soft source and no uniform E (as the other single-pass kernels), a window
-// that fits shared memory, a spare pair of axion buffers and a device that
-// supports cooperative launches.
-bool block1d_supported(const axp_grid *g)
+// Steps per window of the time-blocked 1D kernel (halo: that + 3 cells a side): the
+// longest that fits p passes of the block's lanes over the window, p the one with the
+// least time per step, passes x pass + wait / steps, from pass = 1.6 us (FP64) or 0.45 us
+// (FP32) and 2.5 us for a grid-wide wait.  FP64, 4096 cells over 152 SMs: 15 steps in one
+// pass of 64 cells (12, 14, 15: 1.80, 1.77, 1.76 us per step; 16 takes two passes).  The
+// bits of a run do not depend on it.
+template <typename T>
+int line_block(int64_t seg)
+{
+    const int lanes = line1d::lanes_of<T>(), most = line1d::max_window<T>();
+    const double pass = sizeof(T) == 8 ? 1.6 : 0.45;
+    int best = 0;
+    double best_cost = 0.0;
+    for (int p = 1; p * lanes <= most + lanes; p++) {
+        const int64_t w = std::min<int64_t>((int64_t)p * lanes, most), t = std::min<int64_t>((w - seg) / 2 - 3, 64);
+        if (t < 1) continue;
+        const double cost = p * pass + 2.5 / (double)t;
+        if (best == 0 || cost < best_cost) {
+            best = (int)t;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+// What the kernel computes: 1D grids without a soft source or a uniform E, on a device
+// with cooperative launches.  kind 0: periodic FP64, which AXP_KERNEL_BLOCK1D names; 1:
+// FP32 split, or absorbing layers at both ends (the order-0 x components, which no
+// curl drives, must then be absent: the layer would damp them), which AUTO takes in
+// place of the generic kernel on the same staggered state.
+bool line_takes(const axp_grid *g, int kind)
 {
     const axp_grid_desc &d = g->desc;
-    if (d.precision != AXP_FP64 || d.n[1] != 1 || d.n[2] != 1 || d.n[0] < 256 || g->src_on) return false;
-    if (d.em_bc[0][0] != AXP_BC_PERIODIC || d.axion_bc[0][0] != AXP_BC_PERIODIC) return false;
+    if (d.n[1] != 1 || d.n[2] != 1 || d.n[0] < 256 || g->src_on) return false;
+    const bool per = d.em_bc[0][0] == AXP_BC_PERIODIC && d.axion_bc[0][0] == AXP_BC_PERIODIC;
+    if (kind == 0 && (!per || d.precision != AXP_FP64)) return false;
+    if (!per) {
+        for (int s = 0; s < 2; s++)
+            if (d.em_bc[0][s] != AXP_BC_PML || d.axion_bc[0][s] != AXP_BC_PML) return false;
+        if (order0_closure(g) & (1u | 8u)) return false;
+    }
     for (int a = 0; a < 3; a++)
         if (g->E_ext[a] != 0.0) return false;
     if (g->layout.off_phi[3] == 0) return false;
-    int coop = 0, sms = 0;
+    int coop = 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device) != cudaSuccess || !coop) return false;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess || sms < 1) return false;
-    const int64_t slots = (int64_t)sms * kLineBlocksPerSM, seg = (d.n[0] + slots - 1) / slots;
-    return seg + 2 * (kLineBlock + 3) <= line1d::kMaxWindow;
+    const int64_t seg = line_seg(g);
+    if (seg < 1) return false;
+    // periodic FP64 windows as ever: up to 964 cells a block; the others while a step of theirs
+    // is cheaper than a launch of the generic kernel (kLineMost cells)
+    if (kind == 0) return seg + 2 * 18 <= 1000 && line_block<double>(seg) >= 1;
+    return d.n[0] <= kLineMost && (d.precision == AXP_FP64 ? line_block<double>(seg) : line_block<float>(seg)) >= 1;
 }
+bool block1d_supported(const axp_grid *g) { return line_takes(g, 0); }
 
 // Runs of steps of the time-blocked 1D kernel on the staggered state: one
 // cooperative launch per run, split at diagnostic steps.
+template <typename T>
 cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
 {
     const axp_grid_desc &d = g->desc;
-    int sms = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
     g->coop_used = true;
     g->half_prev = false;  // (its windows double-buffer both field sets)
-    line1d::Args A;
+    line1d::Args<T> A;
     std::memset(&A, 0, sizeof(A));
     A.n = d.n[0];
-    A.tblock = kLineBlock;
-    A.halo = kLineBlock + 3;
-    A.seg = (int)((d.n[0] + (int64_t)sms * kLineBlocksPerSM - 1) / ((int64_t)sms * kLineBlocksPerSM));
+    A.seg = (int)line_seg(g);
+    A.tblock = line_block<T>(A.seg);
+    A.halo = A.tblock + 3;
     const int blocks = (int)((d.n[0] + A.seg - 1) / A.seg);
-    const size_t smem = (size_t)line1d::kArrays * (A.seg + 2 * A.halo) * sizeof(double);
-    e = cudaFuncSetAttribute(line1d::k_line1d, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(line1d::kArrays * line1d::kMaxWindow * sizeof(double)));
+    const bool layer = d.em_bc[0][0] != AXP_BC_PERIODIC;
+    const size_t smem = (size_t)(line1d::kArrays + (layer ? line1d::kLayerArrays : 0)) * (A.seg + 2 * A.halo) * sizeof(T);
+    const void *kern = layer ? (const void *)line1d::k_line1d<T, true> : (const void *)line1d::k_line1d<T, false>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024);
     if (e != cudaSuccess) return e;
     const double dx = d.d[0], dt = d.dt;
-    A.cB = dt / 2.0 / dx;
-    A.c2B = dt / dx;
-    A.h2g = dt * d.g;
-    A.lap_0 = 2.0 - dt * dt * (d.m * d.m + 2.0 / (dx * dx));
-    A.lap_c = dt * dt / (dx * dx);
-    A.dt2g = dt * dt * d.g;
-    A.inv_dt = 1.0 / dt;
-    A.q4dx = 1.0 / (4.0 * dx);
-    for (int a = 0; a < 3; a++) A.Bext[a] = g->B_ext[a];
+    A.cB = (T)(dt / 2.0 / dx);
+    A.c2B = (T)(dt / dx);
+    A.h2g = (T)(dt * d.g);
+    A.lap_0 = (T)(sizeof(T) == 8 ? 2.0 - dt * dt * (d.m * d.m + 2.0 / (dx * dx)) : -dt * dt * d.m * d.m);
+    A.lap_c = (T)(dt * dt / (dx * dx));
+    A.dt2g = (T)(dt * dt * d.g);
+    A.inv_dt = (T)(1.0 / dt);
+    A.q4dx = (T)(1.0 / (4.0 * dx));
+    for (int a = 0; a < 3; a++) A.Bext[a] = (T)g->B_ext[a];
     const Workspace &w = g->layout;
+    for (int s = 0; s < 2; s++)
+        A.lay[s] = layer && d.pml_sigma_max_dt > 0 ? (int)std::min<int64_t>(d.pml_cells, d.n[0]) : 0;
+    A.tab = (const T *)(g->ws + w.off_pml_tab[0]);
+    A.sig = (const T *)(g->ws + w.off_sig_ax[0]);
+    A.inv_h = (T)(2.0 / dt);
+    A.inv_dt2 = (T)(1.0 / (dt * dt));
+    A.dt = (T)dt;
     const size_t en[5] = {w.off_J[0], w.off_J[1], w.off_J[2], w.off_P[0], w.off_P[1]};
-    for (int q = 0; q < 5; q++) A.En[q] = (double *)(g->ws + en[q]);
+    for (int q = 0; q < 5; q++) A.En[q] = (T *)(g->ws + en[q]);
     A.ctr = (unsigned *)(g->ws + w.off_flag);
     A.err = (int *)(g->ws + w.off_flag) + 1;  // read (and cleared) by the next synchronising call
     A.absent = g->coop_absent;
@@ -320,19 +360,18 @@ cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
         for (int p = 0; p < 2; p++) {
             for (int q = 0; q < 6; q++) {
                 const int fe = q < 3 ? kE0 + q : kE1 + (q - 3), fb = q < 3 ? kB0 + q : kB1 + (q - 3);
-                A.Ew[p][q] = (double *)(g->ws + w.off_fields[sets[p]][fe]);
-                A.Bw[p][q] = (double *)(g->ws + w.off_fields[sets[p]][fb]);
+                A.Ew[p][q] = (T *)(g->ws + w.off_fields[sets[p]][fe]);
+                A.Bw[p][q] = (T *)(g->ws + w.off_fields[sets[p]][fb]);
                 A.E[p][q] = A.Ew[p][q];
                 A.B[p][q] = A.Bw[p][q];
             }
-            A.phi[p][0] = (double *)(g->ws + w.off_phi[ph[p][0]]);
-            A.phi[p][1] = (double *)(g->ws + w.off_phi[ph[p][1]]);
+            A.phi[p][0] = (T *)(g->ws + w.off_phi[ph[p][0]]);
+            A.phi[p][1] = (T *)(g->ws + w.off_phi[ph[p][1]]);
         }
         A.nsteps = k;
         if ((e = cudaMemsetAsync(A.ctr, 0, sizeof(unsigned), g->stream)) != cudaSuccess) return e;
         void *args[] = {&A};
-        e = cudaLaunchCooperativeKernel((const void *)line1d::k_line1d, dim3(blocks), dim3(line1d::kThreads), args,
-                                        smem, g->stream);
+        e = cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(line1d::threads_of<T>()), args, smem, g->stream);
         if (e != cudaSuccess) return e;
         g->launches++;
         A.absent = -1;
@@ -347,10 +386,11 @@ cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
         left -= k;
         if (d.diag_every > 0 && g->step % d.diag_every == 0) {
             axp_diag *dst = ring_slot(g, g->ring_written);
-            if ((e = diag_compute<double>(g, dst)) != cudaSuccess) return e;
+            if ((e = diag_compute<T>(g, dst)) != cudaSuccess) return e;
             g->ring_written++;
         }
     }
+    g->J_valid = false;
     return cudaGetLastError();
 }
 
@@ -844,9 +884,11 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     const int32_t path = fused_path<T>(g);
     if (path == AXP_KERNEL_GENERAL) return cudaSuccess;
     *handled = true;
-    if (path == AXP_KERNEL_BLOCK1D) {
+    // the time-blocked 1D kernel: chosen, or AUTO in place of the generic kernel on its state
+    if (path == AXP_KERNEL_BLOCK1D ||
+        (path == AXP_KERNEL_FUSED && g->kernel_choice == AXP_KERNEL_AUTO && line_takes(g, 1))) {
         cudaError_t e = enter_staggered<T>(g);
-        return e != cudaSuccess ? e : block1d_step(g, nsteps);
+        return e != cudaSuccess ? e : block1d_step<T>(g, nsteps);
     }
     const bool tm = path == AXP_KERNEL_TM2D || path == AXP_KERNEL_TM2D_LIST, ax = path == AXP_KERNEL_AX3D;
     const int mode = grid_mode(g);

@@ -1,5 +1,5 @@
-// kernels_line1d.cuh -- time-blocked step for FP64 1D grids periodic along x
-// (arXiv 2406.16796 Sec. 2.3; the 1D conversion workload).
+// kernels_line1d.cuh -- time-blocked step for 1D grids (arXiv 2406.16796 Sec. 2.3; the
+// 1D conversion workload): FP64 and FP32 split, periodic along x or with absorbing layers.
 //
 // A 1D grid of a few thousand cells is far too small to fill the GPU: launched
 // one step at a time its steps cost launch and synchronisation latency, not
@@ -24,6 +24,20 @@
 //      + 2h (curl B1^{n+1} - g J^{n+1}); E0^{n+3/2} = 2 E0^{n+1} - E0^{n+1/2}
 // with the averages of Sec. 2.3 reduced to 1D (a 4-point mean over cells that
 // coincide along y and z is the 2-point mean along x).
+//
+// Absorbing layers (LAYER): windows that reach a layer or the grid's end take a body
+// that asks each cell where it lies; a cell outside the layers takes the plain update's
+// own operations, so its bits do not depend on the window it is computed in.  Cells
+// beyond the grid hold zeros (the closure of E and B and the PML ghost of phi): their
+// coefficients are zero.
+//
+// FP32 split holds phi^{n+1/2} and its increment, and forms the Laplacian from neighbour
+// differences.  Its step is bound by the barriers' latency (about 0.55 us), not by a pipe,
+// so its windows are blocked over more steps (line_block).
+//
+// Measured, us per step (one launch per step before): 2048 cells with absorbing ends
+// FP32 5.2 -> 0.92, FP64 16.8 -> 2.8; 4096 periodic FP32 2.9 -> 0.63;
+// 65536 with absorbing ends FP32 7.0 -> 2.3, FP64 36 -> 11.5; 4096 periodic FP64 1.8 before and now.
 #pragma once
 
 #include "kernels_fused.cuh"
@@ -36,30 +50,43 @@ namespace line1d {
 // FP64 rate.  The window's cells are covered by two warps and each stage's work
 // on a cell is split into two halves of independent outputs: warps 0-1 take one
 // half and warps 2-3 (the other two sub-partitions) the other.
-constexpr int kThreads = 128;
-constexpr int kLanes = 64;               // cells a pass of one half covers
-constexpr int kArrays = 27;              // window arrays (listed in k_line1d)
-constexpr int kMaxWindow = 1000;         // cells: kArrays x 1000 x 8 B = 216 KB of shared memory
+// FP32: eight warps, so that a pass covers 128 cells.
+template <typename T>
+__host__ __device__ constexpr int threads_of() { return sizeof(T) == 8 ? 128 : 256; }
+template <typename T>
+__host__ __device__ constexpr int lanes_of() { return threads_of<T>() / 2; }  // cells a pass of one half covers
+constexpr int kArrays = 28;              // window arrays (listed in k_line1d)
+constexpr int kLayerArrays = 5;          // and the layer's coefficients
+template <typename T>
+__host__ __device__ constexpr int max_window() { return 216 * 1024 / ((kArrays + kLayerArrays) * (int)sizeof(T)); }
 constexpr unsigned kSpinLimit = 1u << 26;        // polls of a grid-wide wait before it gives up ...
 constexpr unsigned long long kWaitNs = 1000000000ull;  // ... or one second, whichever comes first
 
+template <typename T>
 struct Args {
-    const double *E[2][6], *B[2][6];  // buffer sets: order-0 xyz, order-1 xyz (E^{n+1/2}, B^n)
-    double *Ew[2][6], *Bw[2][6];      // the same arrays, written
-    double *phi[2][2];                // per set: phi^{n+1/2}, phi^{n-1/2}
+    const T *E[2][6], *B[2][6];  // buffer sets: order-0 xyz, order-1 xyz (E^{n+1/2}, B^n)
+    T *Ew[2][6], *Bw[2][6];      // the same arrays, written
+    T *phi[2][2];                     // per set: phi^{n+1/2}; phi^{n-1/2} (FP64) or the increment
     int64_t n;                        // cells
     int64_t nsteps;
     int tblock, halo, seg;
     // step constants
-    double cB;      // h/dx: one B or E0 half-step per difference
-    double c2B;     // 2h/dx: the two half-steps of E1 (and of B1) per difference
-    double h2g;     // 2hg: the current's term in E1's two half-steps
-    double lap_0, lap_c, dt2g;  // phi^{n+3/2} = lap_0 phi + lap_c (phi+ + phi-) - phi^{n-1/2} + dt2g S/g
-    double inv_dt, q4dx;        // 1/dt; 1/(4 dx) for the central gradient of 2 phi^{n+1}
-    double Bext[3];
+    T cB;           // h/dx: one B or E0 half-step per difference
+    T c2B;          // 2h/dx: the two half-steps of E1 (and of B1) per difference
+    T h2g;          // 2hg: the current's term in E1's two half-steps
+    // FP64: phi^{n+3/2} = lap_0 phi + lap_c (phi+ + phi-) - phi^{n-1/2} + dt2g S/g;
+    // FP32: the increment grows by lap_0 phi + lap_c (second difference) + dt2g S/g
+    T lap_0, lap_c, dt2g;
+    T inv_dt, q4dx;        // 1/dt; 1/(4 dx) for the central gradient of 2 phi^{n+1}
+    T Bext[3];
+    // absorbing layers: their cells at either end, the coefficient tables of the grid
+    // (a, b, a^2, b (1 + a), c1, c2: n each), sigma of the axion, 1/h, 1/dt^2, dt
+    int lay[2];
+    const T *tab, *sig;
+    T inv_h, inv_dt2, dt;
     unsigned *ctr;  // grid-wait arrivals (zeroed before the launch)
     int *err;       // 1 once a wait gave up
-    double *En[5];  // E at the integer time the launch ends at: E0 y z, E1 x y z
+    T *En[5];  // E at the integer time the launch ends at: E0 y z, E1 x y z
     int absent;     // failure-detection test: this block leaves before its first wait (-1: none)
 };
 
@@ -97,102 +124,169 @@ __device__ __forceinline__ bool grid_wait(unsigned *ctr, unsigned target, int *e
     return ok != 0;
 }
 
-__global__ void __launch_bounds__(kThreads) k_line1d(Args A)
+template <typename T, bool LAYER>
+__global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
 {
-    extern __shared__ __align__(16) double l1_sm[];
+    constexpr bool INCR = sizeof(T) == 4;
+    constexpr int LANES = lanes_of<T>();
+    extern __shared__ __align__(16) unsigned char l1_raw[];
+    T *l1_sm = reinterpret_cast<T *>(l1_raw);
     const int64_t N = A.n;
     const int64_t s0 = (int64_t)blockIdx.x * A.seg;
     const int own = (int)(min(N, s0 + A.seg) - s0);
     const int H = A.halo, W = own + 2 * H, Wm = A.seg + 2 * A.halo;
     const int tid = threadIdx.x, nt = blockDim.x;
-    // window arrays: E (6), B (6), phi^{n+1/2}, phi^{n-1/2}, B0^{n+1/2} y z, E0^{n+1} y z,
-    // 2 phi^{n+1}, dt D_t phi^{n+1}, P (3), Bbar0^{n+1} y z (with B_ext), and two values that
-    // stay fixed over a window's steps: E0x and B0x do not change in 1D (no curl along x),
-    // so Bbar0_x = B0x + B_ext,x and the source's term Ebar0_x Bbar0_x are formed once
-    double *E[6], *B[6];
+    // window arrays: E (6), B (6), phi^{n+1/2}, phi^{n-1/2} (FP32: the next phi), B0^{n+1/2}
+    // y z, E0^{n+1} y z, 2 phi^{n+1}, dt D_t phi^{n+1}, P (3), Bbar0^{n+1} y z (with B_ext),
+    // two values that stay fixed over a window's steps (E0x and B0x do not change in 1D, no
+    // curl along x: Bbar0_x = B0x + B_ext,x and the source's term Ebar0_x Bbar0_x), and
+    // FP32's increment
+    auto arr = [&](int q) { return l1_sm + (size_t)q * Wm; };
+    T *E[6], *B[6];
     for (int q = 0; q < 6; q++) {
-        E[q] = l1_sm + (size_t)q * Wm;
-        B[q] = l1_sm + (size_t)(6 + q) * Wm;
+        E[q] = arr(q);
+        B[q] = arr(6 + q);
     }
-    double *cur = l1_sm + (size_t)12 * Wm, *old = l1_sm + (size_t)13 * Wm;
-    double *Bhy = l1_sm + (size_t)14 * Wm, *Bhz = l1_sm + (size_t)15 * Wm;
-    double *Eny = l1_sm + (size_t)16 * Wm, *Enz = l1_sm + (size_t)17 * Wm;
-    double *SM = l1_sm + (size_t)18 * Wm, *DF = l1_sm + (size_t)19 * Wm;
-    double *Px = l1_sm + (size_t)20 * Wm, *PY = l1_sm + (size_t)21 * Wm, *PZ = l1_sm + (size_t)22 * Wm;
-    double *BY = l1_sm + (size_t)23 * Wm, *BZ = l1_sm + (size_t)24 * Wm;
-    double *BXT = l1_sm + (size_t)25 * Wm, *SX = l1_sm + (size_t)26 * Wm;
-    const int half = tid / kLanes, lane = tid % kLanes;  // (a warp-uniform half)
+    T *cur = arr(12), *old = arr(13), *Bhy = arr(14), *Bhz = arr(15), *Eny = arr(16), *Enz = arr(17);
+    T *SM = arr(18), *DF = arr(19), *Px = arr(20), *PY = arr(21), *PZ = arr(22), *BY = arr(23), *BZ = arr(24);
+    T *BXT = arr(25), *SX = arr(26), *inc = INCR ? arr(27) : arr(13);
+    // the layer's a, r = b/h, and for the axion 1/(1 + sigma dt), (1 - sigma dt)/(1 + sigma dt), (sigma dt)^2
+    T *La = arr(28), *Lr = arr(29), *Lc1 = arr(30), *Lc2 = arr(31), *Lss = arr(32);
+    const int half = tid / LANES, lane = tid % LANES;  // (a warp-uniform half)
     // values beyond the window's ends: the zero closure
-    auto at = [&](const double *a, int w) { return (w >= 0 && w < W) ? a[w] : 0.0; };
-    const double Bx = A.Bext[0], By = A.Bext[1], Bz = A.Bext[2];
+    auto at = [&](const T *a, int w) { return (w >= 0 && w < W) ? a[w] : T(0); };
+    const T Bx = A.Bext[0], By = A.Bext[1], Bz = A.Bext[2];
+    // window cells [wl, wh) lie in the grid outside the layers
+    const int64_t wl = LAYER ? A.lay[0] - (s0 - H) : 0, wh = LAYER ? N - A.lay[1] - (s0 - H) : W;
+    const bool layered = LAYER && (wl > 0 || wh < W);  // this window's body
+    auto in_layer = [&](int w) { return LAYER && layered && (w < wl || w >= wh); };
+    if (LAYER && layered) {
+        for (int w = tid; w < W; w += nt) {
+            const int64_t gi = s0 - H + w;
+            const bool in = gi >= 0 && gi < N;
+            La[w] = in ? A.tab[gi] : T(0);
+            Lr[w] = in ? A.tab[N + gi] * A.inv_h : T(0);
+            Lc1[w] = in ? A.tab[4 * N + gi] * A.inv_dt2 : T(0);
+            Lc2[w] = in ? A.tab[5 * N + gi] : T(0);
+            const T sd = in ? A.sig[gi] * A.dt : T(0);
+            Lss[w] = sd * sd;
+        }
+    }
 
     int par = 0;
     unsigned waits = 0;
     for (int64_t done = 0; done < A.nsteps; done += A.tblock) {
         const int steps = (int)min((int64_t)A.tblock, A.nsteps - done);
         for (int w = tid; w < W; w += nt) {
-            int64_t gi = (s0 - H + w) % N;
-            if (gi < 0) gi += N;
+            int64_t gi = s0 - H + w;
+            const bool in = !LAYER || (gi >= 0 && gi < N);
+            if (!LAYER) {
+                gi %= N;
+                if (gi < 0) gi += N;
+            }
 #pragma unroll
             for (int q = 0; q < 6; q++) {
-                E[q][w] = A.E[par][q][gi];
-                B[q][w] = A.B[par][q][gi];
+                E[q][w] = in ? A.E[par][q][gi] : T(0);
+                B[q][w] = in ? A.B[par][q][gi] : T(0);
             }
-            cur[w] = A.phi[par][0][gi];
-            old[w] = A.phi[par][1][gi];
+            cur[w] = in ? A.phi[par][0][gi] : T(0);
+            inc[w] = in ? A.phi[par][1][gi] : T(0);
         }
         __syncthreads();
         for (int w = tid; w < W; w += nt) {
-            const double ex = 0.5 * (E[0][w] + at(E[0], w - 1));
-            const double bx = B[0][w] + Bx;
+            const T ex = T(0.5) * (E[0][w] + at(E[0], w - 1));
+            const T bx = B[0][w] + Bx;
             BXT[w] = bx;
             SX[w] = ex * bx;
         }
         __syncthreads();
         for (int st = 0; st < steps; st++) {
             // 1. B^{n+1/2} and B^{n+1}: (curl E)_y = -D_x E_z, (curl E)_z = D_x E_y (forward)
-            for (int w = lane; w < W; w += kLanes) {
+            for (int w = lane; w < W; w += LANES) {
                 if (half == 0) {
-                    const double d0z = at(E[2], w + 1) - E[2][w], d1z = at(E[5], w + 1) - E[5][w];
-                    const double hy = fma(A.cB, d0z, B[1][w]);
-                    Bhy[w] = hy;
-                    B[1][w] = fma(A.cB, d0z, hy);
-                    B[4][w] = fma(A.c2B, d1z, B[4][w]);
+                    const T d0z = at(E[2], w + 1) - E[2][w], d1z = at(E[5], w + 1) - E[5][w];
+                    if (in_layer(w)) {
+                        const T a = La[w], x0 = Lr[w] * (A.cB * d0z), x1 = Lr[w] * (A.cB * d1z);
+                        const T hy = fma(a, B[1][w], x0);
+                        Bhy[w] = hy;
+                        B[1][w] = fma(a, hy, x0);
+                        B[4][w] = fma(a, fma(a, B[4][w], x1), x1);
+                        B[3][w] = a * (a * B[3][w]);
+                    } else {
+                        const T hy = fma(A.cB, d0z, B[1][w]);
+                        Bhy[w] = hy;
+                        B[1][w] = fma(A.cB, d0z, hy);
+                        B[4][w] = fma(A.c2B, d1z, B[4][w]);
+                    }
                 } else {
-                    const double d0y = at(E[1], w + 1) - E[1][w], d1y = at(E[4], w + 1) - E[4][w];
-                    const double hz = fma(-A.cB, d0y, B[2][w]);
-                    Bhz[w] = hz;
-                    B[2][w] = fma(-A.cB, d0y, hz);
-                    B[5][w] = fma(-A.c2B, d1y, B[5][w]);
+                    const T d0y = at(E[1], w + 1) - E[1][w], d1y = at(E[4], w + 1) - E[4][w];
+                    if (in_layer(w)) {
+                        const T a = La[w], x0 = Lr[w] * (-A.cB * d0y), x1 = Lr[w] * (-A.cB * d1y);
+                        const T hz = fma(a, B[2][w], x0);
+                        Bhz[w] = hz;
+                        B[2][w] = fma(a, hz, x0);
+                        B[5][w] = fma(a, fma(a, B[5][w], x1), x1);
+                    } else {
+                        const T hz = fma(-A.cB, d0y, B[2][w]);
+                        Bhz[w] = hz;
+                        B[2][w] = fma(-A.cB, d0y, hz);
+                        B[5][w] = fma(-A.c2B, d1y, B[5][w]);
+                    }
                 }
             }
             __syncthreads();
             // 2. source, phi^{n+3/2}, 2 phi^{n+1}, dt D_t phi^{n+1} | E0^{n+1}, Bbar0^{n+1} y z
-            for (int w = lane; w < W; w += kLanes) {
+            for (int w = lane; w < W; w += LANES) {
                 if (half == 0) {
-                    const double by = fma(0.5, Bhy[w] + at(Bhy, w - 1), By);
-                    const double bz = fma(0.5, Bhz[w] + at(Bhz, w - 1), Bz);
-                    const double S = fma(E[2][w], bz, fma(E[1][w], by, SX[w]));  // S/g
-                    const double ph = cur[w];
-                    double nw = fma(A.lap_0, ph, -old[w]);
-                    nw = fma(A.lap_c, at(cur, w + 1) + at(cur, w - 1), nw);
-                    nw = fma(A.dt2g, S, nw);
-                    old[w] = nw;  // phi^{n+3/2} over phi^{n-1/2} (read by this cell only)
-                    SM[w] = nw + ph;
-                    DF[w] = nw - ph;
+                    const T by = fma(T(0.5), Bhy[w] + at(Bhy, w - 1), By);
+                    const T bz = fma(T(0.5), Bhz[w] + at(Bhz, w - 1), Bz);
+                    const T S = fma(E[2][w], bz, fma(E[1][w], by, SX[w]));  // S/g
+                    const T ph = cur[w];
+                    if (INCR) {
+                        const T d2 = (at(cur, w + 1) - ph) + (at(cur, w - 1) - ph);
+                        T di = fma(A.lap_0, ph, fma(A.lap_c, d2, A.dt2g * S));
+                        if (in_layer(w)) di = fma(Lc2[w], inc[w], Lc1[w] * fma(-Lss[w], ph, di));
+                        else di = inc[w] + di;
+                        const T nw = ph + di;
+                        inc[w] = di;
+                        old[w] = nw;
+                        SM[w] = fma(T(2), nw, -di);
+                        DF[w] = di;
+                    } else {
+                        T nw;
+                        if (in_layer(w)) {
+                            nw = A.lap_0 * ph;
+                            nw = fma(A.lap_c, at(cur, w + 1) + at(cur, w - 1), nw);
+                            nw = fma(A.dt2g, S, nw);
+                            nw = fma(-Lc2[w], old[w], Lc1[w] * fma(-Lss[w], ph, nw));
+                        } else {
+                            nw = fma(A.lap_0, ph, -old[w]);
+                            nw = fma(A.lap_c, at(cur, w + 1) + at(cur, w - 1), nw);
+                            nw = fma(A.dt2g, S, nw);
+                        }
+                        old[w] = nw;  // phi^{n+3/2} over phi^{n-1/2} (read by this cell only)
+                        SM[w] = nw + ph;
+                        DF[w] = nw - ph;
+                    }
                 } else {
                     // (curl B0)_y = -D_x B0z, (curl B0)_z = D_x B0y (backward)
-                    Eny[w] = fma(-A.cB, B[2][w] - at(B[2], w - 1), E[1][w]);
-                    Enz[w] = fma(A.cB, B[1][w] - at(B[1], w - 1), E[2][w]);
-                    BY[w] = fma(0.5, B[1][w] + at(B[1], w - 1), By);
-                    BZ[w] = fma(0.5, B[2][w] + at(B[2], w - 1), Bz);
+                    const T dz = B[2][w] - at(B[2], w - 1), dy = B[1][w] - at(B[1], w - 1);
+                    if (in_layer(w)) {
+                        Eny[w] = fma(La[w], E[1][w], Lr[w] * (-A.cB * dz));
+                        Enz[w] = fma(La[w], E[2][w], Lr[w] * (A.cB * dy));
+                    } else {
+                        Eny[w] = fma(-A.cB, dz, E[1][w]);
+                        Enz[w] = fma(A.cB, dy, E[2][w]);
+                    }
+                    BY[w] = fma(T(0.5), B[1][w] + at(B[1], w - 1), By);
+                    BZ[w] = fma(T(0.5), B[2][w] + at(B[2], w - 1), Bz);
                 }
             }
             __syncthreads();
             // 3. P^{n+1} at the cell centres
-            for (int w = lane; w < W; w += kLanes) {
-                const double Dt = DF[w] * A.inv_dt;
-                const double dphi = (at(SM, w + 1) - at(SM, w - 1)) * A.q4dx;
+            for (int w = lane; w < W; w += LANES) {
+                const T Dt = DF[w] * A.inv_dt;
+                const T dphi = (at(SM, w + 1) - at(SM, w - 1)) * A.q4dx;
                 if (half == 0) {
                     PY[w] = fma(-Enz[w], dphi, Dt * BY[w]);
                 } else {
@@ -202,20 +296,37 @@ __global__ void __launch_bounds__(kThreads) k_line1d(Args A)
             }
             __syncthreads();
             // 4. J^{n+1}; E1^{n+3/2}; E0^{n+3/2}
-            for (int w = lane; w < W; w += kLanes) {
+            for (int w = lane; w < W; w += LANES) {
                 if (half == 0) {
-                    const double Jx = 0.5 * (Px[w] + at(Px, w + 1));
-                    E[3][w] = fma(-A.h2g, Jx, E[3][w]);
-                    E[4][w] = fma(-A.c2B, B[5][w] - at(B[5], w - 1), fma(-A.h2g, PY[w], E[4][w]));
+                    const T Jx = T(0.5) * (Px[w] + at(Px, w + 1)), dz = B[5][w] - at(B[5], w - 1);
+                    if (in_layer(w)) {
+                        // two half-steps: a^2 E + (1 + a) r h X
+                        const T a = La[w], r2 = T(0.5) * Lr[w];
+                        const T xx = r2 * (-A.h2g * Jx), xy = r2 * fma(-A.c2B, dz, -A.h2g * PY[w]);
+                        E[3][w] = fma(a, fma(a, E[3][w], xx), xx);
+                        E[4][w] = fma(a, fma(a, E[4][w], xy), xy);
+                    } else {
+                        E[3][w] = fma(-A.h2g, Jx, E[3][w]);
+                        E[4][w] = fma(-A.c2B, dz, fma(-A.h2g, PY[w], E[4][w]));
+                    }
                 } else {
-                    E[5][w] = fma(A.c2B, B[4][w] - at(B[4], w - 1), fma(-A.h2g, PZ[w], E[5][w]));
-                    E[1][w] = fma(2.0, Eny[w], -E[1][w]);
-                    E[2][w] = fma(2.0, Enz[w], -E[2][w]);
+                    const T dy = B[4][w] - at(B[4], w - 1);
+                    if (in_layer(w)) {
+                        const T a = La[w], xz = T(0.5) * Lr[w] * fma(A.c2B, dy, -A.h2g * PZ[w]);
+                        E[5][w] = fma(a, fma(a, E[5][w], xz), xz);
+                        E[1][w] = fma(T(1) + a, Eny[w], -a * E[1][w]);
+                        E[2][w] = fma(T(1) + a, Enz[w], -a * E[2][w]);
+                    } else {
+                        E[5][w] = fma(A.c2B, dy, fma(-A.h2g, PZ[w], E[5][w]));
+                        E[1][w] = fma(T(2), Eny[w], -E[1][w]);
+                        E[2][w] = fma(T(2), Enz[w], -E[2][w]);
+                    }
                 }
             }
-            double *t = cur;
+            T *t = cur;
             cur = old;
             old = t;
+            if (!INCR) inc = old;
             __syncthreads();
         }
         for (int w = H + tid; w < H + own; w += nt) {
@@ -226,15 +337,20 @@ __global__ void __launch_bounds__(kThreads) k_line1d(Args A)
                 A.Bw[1 - par][q][gi] = B[q][w];
             }
             A.phi[1 - par][0][gi] = cur[w];
-            A.phi[1 - par][1][gi] = old[w];
+            A.phi[1 - par][1][gi] = inc[w];
             if (done + A.tblock >= A.nsteps) {
                 // E^{n+1} of the last step, for a record taken here: E1 less the second of
                 // its two half-steps, E0 as the step formed it
+                const T Jx = T(0.5) * (Px[w] + at(Px, w + 1));
+                const T hx = T(-0.5) * A.h2g * Jx, hy = fma(-A.cB, B[5][w] - at(B[5], w - 1), T(-0.5) * A.h2g * PY[w]);
+                const T hz = fma(A.cB, B[4][w] - at(B[4], w - 1), T(-0.5) * A.h2g * PZ[w]);
+                const bool lay = in_layer(w);
+                const T r = lay ? Lr[w] : T(1), ia = lay ? T(1) / La[w] : T(1);
                 A.En[0][gi] = Eny[w];
                 A.En[1][gi] = Enz[w];
-                A.En[2][gi] = fma(0.5 * A.h2g, 0.5 * (Px[w] + at(Px, w + 1)), E[3][w]);
-                A.En[3][gi] = fma(A.cB, B[5][w] - at(B[5], w - 1), fma(0.5 * A.h2g, PY[w], E[4][w]));
-                A.En[4][gi] = fma(-A.cB, B[4][w] - at(B[4], w - 1), fma(0.5 * A.h2g, PZ[w], E[5][w]));
+                A.En[2][gi] = fma(-r, hx, E[3][w]) * ia;
+                A.En[3][gi] = fma(-r, hy, E[4][w]) * ia;
+                A.En[4][gi] = fma(-r, hz, E[5][w]) * ia;
             }
         }
         par ^= 1;
