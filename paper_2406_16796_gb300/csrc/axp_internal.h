@@ -210,6 +210,11 @@ cudaError_t general_step(axp_grid *g, int64_t nsteps);
 template <typename T>
 cudaError_t staged_step(axp_grid *g, int64_t nsteps);
 bool staged_supported(const axp_grid *g);
+// E^n -> E^{n+1/2} in place, and E^{n+1/2} -> E^n into field set oset, by the same passes
+template <typename T>
+cudaError_t staged_enter(axp_grid *g);
+template <typename T>
+cudaError_t staged_exit(axp_grid *g, int oset);
 template <typename T>
 cudaError_t general_current(axp_grid *g);  // J^n of the present state
 template <typename T>

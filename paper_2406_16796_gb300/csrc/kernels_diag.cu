@@ -35,8 +35,8 @@ constexpr int kQ = 7;  // H_phi, H_g0, H_g1, cross, sum x B1z^2, sum B1z^2, gaus
 //    scaled by a power of two taken from its largest magnitude in the region (max_group:
 //    a pass of its own, or part of the pass that forms E^n).  Scaling by a power of
 //    two is exact; what then underflows is below 2^-60 of the largest value.
-// Measured (us, before -> after): 512^3 FP32 box DIAG_A3; 4096 x 2048 pulse FP32 DIAG_P32,
-// FP64 DIAG_P64.
+// Measured, a whole record (us, before -> after): 512^3 FP32 box 37000 -> 6040; 4096 x 2048
+// pulse FP32 1100 -> 430; FP64 unchanged at 1110 (50 operations per cell on the FP64 pipe).
 // ---------------------------------------------------------------------------
 struct FF {
     float h, l;

@@ -538,12 +538,15 @@ cudaError_t enter_staggered(axp_grid *g)
 {
     if (g->staggered) return cudaSuccess;
     g->half_prev = g->en_scratch = false;
-    cudaError_t e = general_current<T>(g);
-    if (e != cudaSuccess) return e;
-    View<T> v = make_view<T>(g);
-    const int nb = grid_for(v.N);
-    k_e_half<T><<<nb, kThreads, 0, g->stream>>>(v, 3, e_sheet<T>(g, time_n(g, g->step)));
-    g->launches++;
+    cudaError_t e;
+    if (sizeof(T) == sizeof(double) && staged_supported(g)) {
+        if ((e = staged_enter<T>(g)) != cudaSuccess) return e;
+    } else {
+        if ((e = general_current<T>(g)) != cudaSuccess) return e;
+        View<T> v = make_view<T>(g);
+        k_e_half<T><<<grid_for(v.N), kThreads, 0, g->stream>>>(v, 3, e_sheet<T>(g, time_n(g, g->step)));
+        g->launches++;
+    }
     g->staggered = true;
     g->J_valid = false;
     return cudaGetLastError();
@@ -555,6 +558,12 @@ cudaError_t exit_staggered(axp_grid *g, bool in_place)
     if (!g->staggered) return cudaSuccess;
     g->half_prev = g->en_scratch = false;
     const int oset = in_place ? g->fset : 1 - g->fset;
+    if (sizeof(T) == sizeof(double) && staged_supported(g)) {
+        const cudaError_t se = staged_exit<T>(g, oset);
+        if (in_place) g->staggered = false;
+        g->J_valid = in_place;
+        return se;
+    }
     View<T> vin = make_view<T>(g);
     View<T> vout = make_view_eset<T>(g, oset);
     const int nb = grid_for(vin.N);

@@ -63,7 +63,7 @@ struct Stage {
     T hd[3];              // h/d
     T inv_h, h;
     T hg2;                // h g / 2: J is used as the sum of two P
-    T lap_c[3], lap_0, dt2g, m2dt2, dt, dt2, inv_dt2, inv_dt, q4d[3], of_r[3];
+    T lap_c[3], dt2g, m2dt2, dt, dt2, inv_dt2, inv_dt, q4d[3], of_r[3];
     T Bext[3], Eext[3];
     int src_x;            // x index of the soft source's E cells (-1: none)
     const T *src_w[2];
@@ -323,9 +323,9 @@ __global__ void __launch_bounds__(kThreads) k_stage_phi(Stage<T> s, const T *bs0
             if (!(MASK >> a & 1)) continue;
             const T up = phi_nb(s, s.phi, s.gh, a, 1, q), dn = phi_nb(s, s.phi, s.gh, a, 0, q);
             // FP32 split: from neighbour differences, which do not round against 2 phi
-            lap = fma(s.lap_c[a], INCR ? (up - ph) + (dn - ph) : up + dn, lap);
+            lap = fma(s.lap_c[a], INCR ? (up - ph) + (dn - ph) : fma(T(-2), ph, up + dn), lap);
         }
-        lap = fma(s.lap_0, ph, lap);  // FP64: lap_0 holds the 2 phi of the leapfrog too
+        lap = fma(-s.m2dt2, ph, lap);
         T nw;  // phi^{n+3/2}, or its increment in FP32 split
         if (in_layer<MASK>(s, q)) {
             // (lap - (sigma dt)^2 phi -+ (1 - sigma dt) old) / (1 + sigma dt) from the tables
@@ -340,9 +340,12 @@ __global__ void __launch_bounds__(kThreads) k_stage_phi(Stage<T> s, const T *bs0
             }
             sd = sd * s.dt;
             lap = fma(-(sd * sd), ph, lap);
+            if (!INCR) lap = fma(T(2), ph, lap);
             nw = fma(INCR ? c2 : -c2, old, c1 * s.inv_dt2 * lap);
         } else {
-            nw = INCR ? lap + old : lap - old;
+            // (2 phi apart from the mass and the Laplacian: folded into one coefficient, its
+            // rounding acts as a mass and grows with the square of the steps)
+            nw = INCR ? lap + old : fma(T(2), ph, -old) + lap;
         }
         s.phi_out[q.c] = INCR ? ph + nw : nw;
         if (INCR) s.phib_out[q.c] = nw;
@@ -404,9 +407,52 @@ __global__ void __launch_bounds__(kThreads) k_stage_p(Stage<T> s, const T *e0, c
     }
 }
 
-// J = (P(c) + P(c + a)) / 2 and the order-1 E update; CURRENT: only J.  Beyond the
+// J = (P(c) + P(c + a)) / 2 and the order-1 E update.  Beyond the
 // last cell of a non-periodic axis P follows the ghost rules: 0 at a PML side without
 // a uniform E, else evaluated in place (one cell per row or plane).
+// Inverse of a half-step: the field a half-step earlier, given h X.
+template <typename T, bool IN>
+__device__ __forceinline__ T half_back(const Layer<T, IN> &L, T F, T hX)
+{
+    return IN ? fma(-L.r, hX, F) / L.a : F - hX;
+}
+
+// E0^n from E0^{n+1/2} (Eout may be Ein)
+template <typename T, int MASK, int EM, int BM, bool IN>
+__device__ __forceinline__ void e0_back(const Stage<T> &s, const Cell &q)
+{
+    const Layer<T, IN> L = layer_at<MASK, IN>(s, q);
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        if (!(EM >> a & 1)) continue;
+        T hX = curl_h<MASK, BM, false>(s, s.Bin, a, q);
+        if (a > 0 && q.x[0] == s.src_x) hX = fma(s.src_w[a - 1][q.x[1] + s.n[1] * q.x[2]], s.src_e, hX);
+        s.Eout[a][q.c] = half_back(L, s.Ein[a][q.c], hX);
+    }
+}
+template <typename T, int MASK, int EM, int BM>
+__global__ void __launch_bounds__(kThreads) k_stage_e0_back(Stage<T> s)
+{
+    Cell q;
+    const bool mine = cell_at<MASK>(s, q);
+    wait_for_previous_pass();
+    if (!mine) return;
+    if (in_layer<MASK>(s, q)) e0_back<T, MASK, EM, BM, true>(s, q);
+    else e0_back<T, MASK, EM, BM, false>(s, q);
+}
+
+template <typename T, int MASK, bool IN>
+__device__ __forceinline__ void e1_back(const Stage<T> &s, const T J2[3], const Cell &q)
+{
+    const Layer<T, IN> L = layer_at<MASK, IN>(s, q);
+    const T *const B1[3] = {s.Bin[3], s.Bin[4], s.Bin[5]};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const T hX = fma(-s.hg2, J2[a], curl_h<MASK, 7, false>(s, B1, a, q));
+        s.Eout[3 + a][q.c] = half_back(L, s.Ein[3 + a][q.c], hX);
+    }
+}
+
 template <typename T, int MASK, bool IN>
 __device__ __forceinline__ void e1_update(const Stage<T> &s, const T J2[3], const Cell &q)
 {
@@ -421,7 +467,8 @@ __device__ __forceinline__ void e1_update(const Stage<T> &s, const T J2[3], cons
         s.Eout[3 + a][q.c] = E;
     }
 }
-template <typename T, int MASK, bool CURRENT>
+// WHAT 0: the step's update; 1: J alone, into its cache; 2: J and E1^n from E1^{n+1/2}
+template <typename T, int MASK, int WHAT>
 __global__ void __launch_bounds__(kThreads) k_stage_j(Stage<T> s, View<T> v, PhiPair<T, sizeof(T) == 4> pq)
 {
     Cell q;
@@ -440,9 +487,14 @@ __global__ void __launch_bounds__(kThreads) k_stage_j(Stage<T> s, View<T> v, Phi
                 p1 = p_comp<T, sizeof(T) == 4>(v, pq, a, q.x[0] + (a == 0), q.x[1] + (a == 1), q.x[2] + (a == 2));
         }
         J2[a] = p0 + p1;
-        if (CURRENT || s.last) s.J[a][q.c] = T(0.5) * J2[a];
+        if (WHAT || s.last) s.J[a][q.c] = T(0.5) * J2[a];
     }
-    if (CURRENT) return;
+    if (WHAT == 1) return;
+    if (WHAT == 2) {
+        if (in_layer<MASK>(s, q)) e1_back<T, MASK, true>(s, J2, q);
+        else e1_back<T, MASK, false>(s, J2, q);
+        return;
+    }
     if (warp_in_layer<MASK>(s, q)) e1_update<T, MASK, true>(s, J2, q);
     else e1_update<T, MASK, false>(s, J2, q);
 }
@@ -500,7 +552,6 @@ Stage<T> make_stage(axp_grid *g)
     s.phi_out = at(w.off_phi[g->phi_next_slot]);
     s.phib_out = sizeof(T) == 4 ? at(w.off_phi[g->phi_next_b_slot]) : nullptr;
     const double h = d.dt / 2.0;
-    double idd = 0.0;
     for (int a = 0; a < 3; a++) {
         s.Bh[a] = s.P[a] = at(w.off_P[a]);
         s.Eh[a] = s.J[a] = at(w.off_J[a]);
@@ -527,7 +578,6 @@ Stage<T> make_stage(axp_grid *g)
         s.hd[a] = (T)(h / d.d[a]);
         s.lap_c[a] = d.n[a] > 1 ? (T)(d.dt * d.dt / (d.d[a] * d.d[a])) : T(0);
         s.q4d[a] = (T)(0.25 / d.d[a]);
-        if (d.n[a] > 1) idd += 1.0 / (d.d[a] * d.d[a]);
         s.Bext[a] = (T)g->B_ext[a];
         s.Eext[a] = (T)g->E_ext[a];
     }
@@ -535,7 +585,6 @@ Stage<T> make_stage(axp_grid *g)
     s.h = (T)h;
     s.inv_h = (T)(1.0 / h);
     s.hg2 = (T)(0.5 * h * d.g);
-    s.lap_0 = (T)(sizeof(T) == 4 ? -d.dt * d.dt * d.m * d.m : 2.0 - d.dt * d.dt * (d.m * d.m + 2.0 * idd));
     s.dt2g = (T)(d.dt * d.dt * d.g);
     s.m2dt2 = (T)(d.dt * d.dt * d.m * d.m);
     s.uniform_e = g->E_ext[0] != 0.0 || g->E_ext[1] != 0.0 || g->E_ext[2] != 0.0;
@@ -555,6 +604,7 @@ Stage<T> make_stage(axp_grid *g)
 // Launches of one configuration: active axes MASK, order-0 components EM and BM.
 template <typename T, int MASK, int EM, int BM>
 struct Passes {
+    static constexpr int kE = EM;
     static int blocks(const Stage<T> &s) { return (s.N + kThreads - 1) / kThreads; }
     static void b(const Stage<T> &s, int mode, cudaStream_t st)
     {
@@ -573,10 +623,15 @@ struct Passes {
     {
         launch_pass(k_stage_p<T, MASK, EM, BM>, blocks(s), st, s, e[0], e[1], e[2], b[0], b[1], b[2], hi, lo);
     }
-    static void j(const Stage<T> &s, const View<T> &v, const PhiPair<T, sizeof(T) == 4> &pq, bool current, cudaStream_t st)
+    static void j(const Stage<T> &s, const View<T> &v, const PhiPair<T, sizeof(T) == 4> &pq, int what, cudaStream_t st)
     {
-        if (current) launch_pass(k_stage_j<T, MASK, true>, blocks(s), st, s, v, pq);
-        else launch_pass(k_stage_j<T, MASK, false>, blocks(s), st, s, v, pq);
+        if (what == 0) launch_pass(k_stage_j<T, MASK, 0>, blocks(s), st, s, v, pq);
+        else if (what == 1) launch_pass(k_stage_j<T, MASK, 1>, blocks(s), st, s, v, pq);
+        else launch_pass(k_stage_j<T, MASK, 2>, blocks(s), st, s, v, pq);
+    }
+    static void e0_back(const Stage<T> &s, cudaStream_t st)
+    {
+        if (EM) launch_pass(k_stage_e0_back<T, MASK, EM, BM>, blocks(s), st, s);
     }
     static void e_half(const Stage<T> &s, cudaStream_t st)
     {
@@ -597,7 +652,50 @@ Ghosts<T> ghost_planes(axp_grid *g, int level)
     return G;
 }
 
-template <typename T, typename Q, int EM, int BM>
+// P and J of the state around integer time n (E0^n in e, the axion levels n+1/2 and
+// n-1/2), and what the J pass does with them
+template <typename T, typename Q>
+void current_at_n(axp_grid *g, Stage<T> s, const T *const e[3], int what)
+{
+    for (int a = 0; a < 3; a++)
+        for (int f = 0; f < 2; f++) {
+            s.gh_hi[a][f] = s.gh[a][f];
+            s.gh[a][f] = s.gh_old[a][f];
+        }
+    View<T> v = make_view<T>(g);
+    for (int a = 0; a < 3; a++) v.f[kE0 + a] = const_cast<T *>(e[a]);
+    const T *const b[3] = {s.Bin[0], s.Bin[1], s.Bin[2]};
+    Q::p(s, e, b, s.phi, s.phib, g->stream);
+    PhiPair<T, sizeof(T) == 4> pq{s.phi, s.phib, ghost_planes<T>(g, 0), ghost_planes<T>(g, 1)};
+    Q::j(s, v, pq, what, g->stream);
+    g->launches += 2;
+}
+
+// E^n -> E^{n+1/2} in place
+template <typename T, typename Q>
+void first_half(axp_grid *g)
+{
+    Stage<T> s = make_stage<T>(g);
+    if (!g->J_valid) current_at_n<T, Q>(g, s, s.Ein, 1);
+    if (g->src_on) s.src_e = (T)(g->desc.dt / 2.0 * source_wave(g, source_x_b(g), time_n(g, g->step)));
+    Q::e_half(s, g->stream);
+    g->launches++;
+}
+
+// E^{n+1/2} -> E^n into field set `oset`
+template <typename T, typename Q>
+void back_half(axp_grid *g, int oset)
+{
+    Stage<T> s = make_stage<T>(g);
+    for (int f = 0; f < 6; f++) s.Eout[f] = (T *)(g->ws + g->layout.off_fields[oset][f < 3 ? kE0 + f : kE1 + f - 3]);
+    if (g->src_on) s.src_e = (T)(g->desc.dt / 2.0 * source_wave(g, source_x_b(g), time_n(g, g->step)));
+    Q::e0_back(s, g->stream);
+    if (Q::kE) g->launches++;
+    const T *const e[3] = {s.Eout[0], s.Eout[1], s.Eout[2]};
+    current_at_n<T, Q>(g, s, e, 2);
+}
+
+template <typename T, typename Q>
 cudaError_t run_staged(axp_grid *g, int64_t nsteps)
 {
     const axp_grid_desc &d = g->desc;
@@ -608,24 +706,7 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
     for (int64_t it = 0; it < nsteps; it++) {
         const bool record = d.diag_every > 0 && (g->step + 1) % d.diag_every == 0;
         if (!ahead) {
-            if (!g->J_valid) {
-                Stage<T> s = make_stage<T>(g);
-                for (int a = 0; a < 3; a++)  // the levels around n: n+1/2 and n-1/2
-                    for (int f = 0; f < 2; f++) {
-                        s.gh_hi[a][f] = s.gh[a][f];
-                        s.gh[a][f] = s.gh_old[a][f];
-                    }
-                View<T> v = make_view<T>(g);
-                const T *const b[3] = {s.Bin[0], s.Bin[1], s.Bin[2]};
-                Q::p(s, s.Ein, b, s.phi, s.phib, g->stream);
-                PhiPair<T, sizeof(T) == 4> pq{s.phi, s.phib, ghost_planes<T>(g, 0), ghost_planes<T>(g, 1)};
-                Q::j(s, v, pq, true, g->stream);
-                g->launches += 2;
-            }
-            Stage<T> s = make_stage<T>(g);
-            if (g->src_on) s.src_e = (T)(d.dt / 2.0 * source_wave(g, source_x_b(g), time_n(g, g->step)));
-            Q::e_half(s, g->stream);
-            g->launches++;
+            first_half<T, Q>(g);
             ahead = true;
         }
         Stage<T> s = make_stage<T>(g);
@@ -661,7 +742,7 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
         const T *eh[3];
         View<T> v = make_view<T>(g);
         for (int a = 0; a < 3; a++) {
-            eh[a] = (EM >> a & 1) ? s.Eh[a] : s.Eout[a];  // (an inactive array is zero in both sets)
+            eh[a] = (Q::kE >> a & 1) ? s.Eh[a] : s.Eout[a];  // (an inactive array is zero in both sets)
             v.f[kE0 + a] = const_cast<T *>(eh[a]);
             v.f[kB0 + a] = s.Bout[a];
         }
@@ -673,7 +754,7 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
         }
         Q::p(s, eh, b, hi, lo, g->stream);
         PhiPair<T, sizeof(T) == 4> pq{hi, lo, ghost_planes<T>(g, 2), ghost_planes<T>(g, 0)};
-        Q::j(s, v, pq, false, g->stream);
+        Q::j(s, v, pq, 0, g->stream);
         g->launches += 2;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         rotate_roles(g);
@@ -696,6 +777,30 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
     return cudaGetLastError();
 }
 
+// f(Passes of the grid's active axes and order-0 components)
+template <typename T, typename F>
+auto with_passes(const axp_grid *g, F &&f)
+{
+    const int64_t *n = g->desc.n;
+    const uint32_t m = order0_closure(g);
+    auto in = [&](uint32_t set) { return (m & ~set) == 0; };
+    const uint32_t tm = 4u | (3u << 3), te = 3u | (4u << 3);  // (E0z; B0x, B0y) and (E0x, E0y; B0z)
+    if (n[1] == 1 && n[2] == 1) {
+        if (m == 0) return f(Passes<T, 1, 0, 0>{});
+        if (in(tm)) return f(Passes<T, 1, 4, 3>{});
+        if (in(te)) return f(Passes<T, 1, 3, 4>{});
+        return f(Passes<T, 1, 7, 7>{});
+    }
+    if (n[2] == 1) {
+        if (m == 0) return f(Passes<T, 3, 0, 0>{});
+        if (in(tm)) return f(Passes<T, 3, 4, 3>{});
+        if (in(te)) return f(Passes<T, 3, 3, 4>{});
+        return f(Passes<T, 3, 7, 7>{});
+    }
+    if (m == 0) return f(Passes<T, 7, 0, 0>{});
+    return f(Passes<T, 7, 7, 7>{});
+}
+
 }  // namespace
 
 // 32-bit cell indexes, and at least one active axis (a single cell keeps the general kernels)
@@ -708,27 +813,28 @@ bool staged_supported(const axp_grid *g)
 template <typename T>
 cudaError_t staged_step(axp_grid *g, int64_t nsteps)
 {
-    const int64_t *n = g->desc.n;
-    const uint32_t m = order0_closure(g);
-    auto in = [&](uint32_t set) { return (m & ~set) == 0; };
-    const uint32_t tm = 4u | (3u << 3), te = 3u | (4u << 3);  // (E0z; B0x, B0y) and (E0x, E0y; B0z)
-    if (n[1] == 1 && n[2] == 1) {
-        if (m == 0) return run_staged<T, Passes<T, 1, 0, 0>, 0, 0>(g, nsteps);
-        if (in(tm)) return run_staged<T, Passes<T, 1, 4, 3>, 4, 3>(g, nsteps);
-        if (in(te)) return run_staged<T, Passes<T, 1, 3, 4>, 3, 4>(g, nsteps);
-        return run_staged<T, Passes<T, 1, 7, 7>, 7, 7>(g, nsteps);
-    }
-    if (n[2] == 1) {
-        if (m == 0) return run_staged<T, Passes<T, 3, 0, 0>, 0, 0>(g, nsteps);
-        if (in(tm)) return run_staged<T, Passes<T, 3, 4, 3>, 4, 3>(g, nsteps);
-        if (in(te)) return run_staged<T, Passes<T, 3, 3, 4>, 3, 4>(g, nsteps);
-        return run_staged<T, Passes<T, 3, 7, 7>, 7, 7>(g, nsteps);
-    }
-    if (m == 0) return run_staged<T, Passes<T, 7, 0, 0>, 0, 0>(g, nsteps);
-    return run_staged<T, Passes<T, 7, 7, 7>, 7, 7>(g, nsteps);
+    return with_passes<T>(g, [&](auto q) { return run_staged<T, decltype(q)>(g, nsteps); });
+}
+
+template <typename T>
+cudaError_t staged_enter(axp_grid *g)
+{
+    with_passes<T>(g, [&](auto q) { first_half<T, decltype(q)>(g); });
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t staged_exit(axp_grid *g, int oset)
+{
+    with_passes<T>(g, [&](auto q) { back_half<T, decltype(q)>(g, oset); });
+    return cudaGetLastError();
 }
 
 template cudaError_t staged_step<double>(axp_grid *, int64_t);
 template cudaError_t staged_step<float>(axp_grid *, int64_t);
+template cudaError_t staged_enter<double>(axp_grid *);
+template cudaError_t staged_enter<float>(axp_grid *);
+template cudaError_t staged_exit<double>(axp_grid *, int);
+template cudaError_t staged_exit<float>(axp_grid *, int);
 
 }  // namespace axp
