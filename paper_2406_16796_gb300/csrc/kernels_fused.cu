@@ -342,6 +342,14 @@ cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
         A.lay[s] = layer && d.pml_sigma_max_dt > 0 ? (int)std::min<int64_t>(d.pml_cells, d.n[0]) : 0;
     A.tab = (const T *)(g->ws + w.off_pml_tab[0]);
     A.sig = (const T *)(g->ws + w.off_sig_ax[0]);
+    A.sig_em = (const T *)(g->ws + w.off_sig_em[0]);
+    A.h = (T)(dt / 2.0);
+    A.idx = (T)(1.0 / dx);
+    A.hidx = (T)(0.5 / dx);
+    A.idx2 = (T)(1.0 / (dx * dx));
+    A.g = (T)d.g;
+    A.m2 = (T)(d.m * d.m);
+    A.dt2 = (T)(dt * dt);
     A.inv_h = (T)(2.0 / dt);
     A.inv_dt2 = (T)(1.0 / (dt * dt));
     A.dt = (T)dt;

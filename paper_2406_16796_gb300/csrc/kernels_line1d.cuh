@@ -31,13 +31,14 @@
 // beyond the grid hold zeros (the closure of E and B and the PML ghost of phi): their
 // coefficients are zero.
 //
-// FP32 split holds phi^{n+1/2} and its increment, and forms the Laplacian from neighbour
-// differences.  Its step is bound by the barriers' latency (about 0.55 us), not by a pipe,
+// FP32 split holds phi^{n+1/2} and its increment, and takes the generic single-pass kernel's
+// operations in their order (rounding differences of a few 1e-5 would come from any other
+// over a few hundred steps).  Its step is bound by the barriers' latency (about 0.55 us), not by a pipe,
 // so its windows are blocked over more steps (line_block).
 //
 // Measured, us per step (one launch per step before): 2048 cells with absorbing ends
-// FP32 5.2 -> 0.92, FP64 16.8 -> 2.8; 4096 periodic FP32 2.9 -> 0.63;
-// 65536 with absorbing ends FP32 7.0 -> 2.3, FP64 36 -> 11.5; 4096 periodic FP64 1.8 before and now.
+// FP32 5.2 -> 1.3, FP64 16.8 -> 2.8; 4096 periodic FP32 2.9 -> 0.63;
+// 65536 with absorbing ends FP32 7.0 -> 3.2, FP64 36 -> 11.5; 4096 periodic FP64 1.8 before and now.
 #pragma once
 
 #include "kernels_fused.cuh"
@@ -56,7 +57,7 @@ __host__ __device__ constexpr int threads_of() { return sizeof(T) == 8 ? 128 : 2
 template <typename T>
 __host__ __device__ constexpr int lanes_of() { return threads_of<T>() / 2; }  // cells a pass of one half covers
 constexpr int kArrays = 28;              // window arrays (listed in k_line1d)
-constexpr int kLayerArrays = 5;          // and the layer's coefficients
+constexpr int kLayerArrays = 7;          // and the layer's coefficients
 template <typename T>
 __host__ __device__ constexpr int max_window() { return 216 * 1024 / ((kArrays + kLayerArrays) * (int)sizeof(T)); }
 constexpr unsigned kSpinLimit = 1u << 26;        // polls of a grid-wide wait before it gives up ...
@@ -82,8 +83,9 @@ struct Args {
     // absorbing layers: their cells at either end, the coefficient tables of the grid
     // (a, b, a^2, b (1 + a), c1, c2: n each), sigma of the axion, 1/h, 1/dt^2, dt
     int lay[2];
-    const T *tab, *sig;
+    const T *tab, *sig, *sig_em;
     T inv_h, inv_dt2, dt;
+    T h, idx, hidx, idx2, g, m2, dt2;  // FP32: h, 1/dx, 1/(2 dx), 1/dx^2, g, m^2, dt^2
     unsigned *ctr;  // grid-wait arrivals (zeroed before the launch)
     int *err;       // 1 once a wait gave up
     T *En[5];  // E at the integer time the launch ends at: E0 y z, E1 x y z
@@ -152,6 +154,10 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
     T *BXT = arr(25), *SX = arr(26), *inc = INCR ? arr(27) : arr(13);
     // the layer's a, r = b/h, and for the axion 1/(1 + sigma dt), (1 - sigma dt)/(1 + sigma dt), (sigma dt)^2
     T *La = arr(28), *Lr = arr(29), *Lc1 = arr(30), *Lc2 = arr(31), *Lss = arr(32);
+    // FP32: La 1 - sigma h/2 (-1 beyond the grid), Ld and Lr the divisor 1 + sigma h/2 and its
+    // reciprocal; for the axion Lc2 1 - sigma dt, Le and Lc1 the divisor 1 + sigma dt and its
+    // reciprocal, Lss sigma^2
+    T *Ld = arr(33), *Le = arr(34);
     const int half = tid / LANES, lane = tid % LANES;  // (a warp-uniform half)
     // values beyond the window's ends: the zero closure
     auto at = [&](const T *a, int w) { return (w >= 0 && w < W) ? a[w] : T(0); };
@@ -164,6 +170,19 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
         for (int w = tid; w < W; w += nt) {
             const int64_t gi = s0 - H + w;
             const bool in = gi >= 0 && gi < N;
+            if (INCR) {
+                const T se = in ? A.sig_em[gi] : T(0), sa = in ? A.sig[gi] : T(0);
+                La[w] = in ? T(1) - se * A.h / T(2) : T(-1);
+                Ld[w] = T(1) + se * A.h / T(2);
+                Lr[w] = T(1) / Ld[w];
+                Lc2[w] = T(1) - sa * A.dt;
+                Le[w] = T(1) + sa * A.dt;
+                Lc1[w] = T(1) / Le[w];
+                Lss[w] = sa * sa;
+                // the stages pass over the cells beyond the grid: what neighbours read there is 0
+                if (!in) old[w] = Bhy[w] = Bhz[w] = SM[w] = DF[w] = T(0);
+                continue;
+            }
             La[w] = in ? A.tab[gi] : T(0);
             Lr[w] = in ? A.tab[N + gi] * A.inv_h : T(0);
             Lc1[w] = in ? A.tab[4 * N + gi] * A.inv_dt2 : T(0);
@@ -200,7 +219,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             SX[w] = ex * bx;
         }
         __syncthreads();
-        for (int st = 0; st < steps; st++) {
+        for (int st = 0; st < (INCR ? 0 : steps); st++) {
             // 1. B^{n+1/2} and B^{n+1}: (curl E)_y = -D_x E_z, (curl E)_z = D_x E_y (forward)
             for (int w = lane; w < W; w += LANES) {
                 if (half == 0) {
@@ -242,17 +261,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
                     const T bz = fma(T(0.5), Bhz[w] + at(Bhz, w - 1), Bz);
                     const T S = fma(E[2][w], bz, fma(E[1][w], by, SX[w]));  // S/g
                     const T ph = cur[w];
-                    if (INCR) {
-                        const T d2 = (at(cur, w + 1) - ph) + (at(cur, w - 1) - ph);
-                        T di = fma(A.lap_0, ph, fma(A.lap_c, d2, A.dt2g * S));
-                        if (in_layer(w)) di = fma(Lc2[w], inc[w], Lc1[w] * fma(-Lss[w], ph, di));
-                        else di = inc[w] + di;
-                        const T nw = ph + di;
-                        inc[w] = di;
-                        old[w] = nw;
-                        SM[w] = fma(T(2), nw, -di);
-                        DF[w] = di;
-                    } else {
+                    {
                         T nw;
                         if (in_layer(w)) {
                             nw = A.lap_0 * ph;
@@ -326,7 +335,105 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             T *t = cur;
             cur = old;
             old = t;
-            if (!INCR) inc = old;
+            inc = old;
+            __syncthreads();
+        }
+        // FP32 split.  One half-step, damped in a layer.  x / d as the correctly rounded quotient
+        // from the correctly rounded reciprocal r of d (Markstein's theorem: q = x r, then
+        // q + (x - q d) r): the plain division of every damped cell and stage doubled the step
+        // of a grid with absorbing ends (2.2 us against 1.3).
+        auto over = [](T x, T d, T r) {
+            const T q = x * r;
+            return fma(fma(-q, d, x), r, q);
+        };
+        // (which product of the damped form is rounded is the generic kernel's choice, for its bits)
+        auto half_b = [&](T F, T X, bool lay, int w) {
+            return lay ? over(fma(La[w], F, A.h * X), Ld[w], Lr[w]) : fma(A.h, X, F);
+        };
+        auto half_e = [&](T F, T X, bool lay, int w) {
+            return lay ? over(fma(A.h, X, La[w] * F), Ld[w], Lr[w]) : fma(A.h, X, F);
+        };
+        for (int st = 0; st < (INCR ? steps : 0); st++) {
+            for (int w = lane; w < W; w += LANES) {
+                bool lay = in_layer(w);
+                if (lay && La[w] < T(0)) continue;
+                lay = lay && Ld[w] != T(1);
+                if (half == 0) {
+                    const T c0 = -((at(E[2], w + 1) - E[2][w]) * A.idx), c1 = -((at(E[5], w + 1) - E[5][w]) * A.idx);
+                    const T hy = half_b(B[1][w], -c0, lay, w);
+                    Bhy[w] = hy;
+                    B[1][w] = half_b(hy, -c0, lay, w);
+                    B[4][w] = half_b(half_b(B[4][w], -c1, lay, w), -c1, lay, w);
+                    if (lay) B[3][w] = half_b(half_b(B[3][w], T(0), lay, w), T(0), lay, w);
+                } else {
+                    const T c0 = (at(E[1], w + 1) - E[1][w]) * A.idx, c1 = (at(E[4], w + 1) - E[4][w]) * A.idx;
+                    const T hz = half_b(B[2][w], -c0, lay, w);
+                    Bhz[w] = hz;
+                    B[2][w] = half_b(hz, -c0, lay, w);
+                    B[5][w] = half_b(half_b(B[5][w], -c1, lay, w), -c1, lay, w);
+                }
+            }
+            __syncthreads();
+            for (int w = lane; w < W; w += LANES) {
+                bool lay = in_layer(w);
+                const bool dead = lay && La[w] < T(0);
+                if (half == 0) {
+                    if (dead) continue;
+                    const T by = fma(T(0.5), Bhy[w] + at(Bhy, w - 1), By);
+                    const T bz = fma(T(0.5), Bhz[w] + at(Bhz, w - 1), Bz);
+                    const T S = fma(E[2][w], bz, fma(E[1][w], by, SX[w]));  // S/g
+                    const T ph = cur[w], pb = inc[w];
+                    const T sp = (at(cur, w + 1) - ph) + (at(cur, w - 1) - ph);
+                    T pin;
+                    if (!lay || Lss[w] == T(0)) {
+                        pin = fma(A.dt2g, S, fma(A.lap_c, sp, fma(A.lap_0, ph, pb)));
+                    } else {
+                        const T Y = fma(-Lss[w], ph, fma(A.g, S, -(A.m2 * ph)) + sp * A.idx2);
+                        pin = over(fma(A.dt2, Y, Lc2[w] * pb), Le[w], Lc1[w]);
+                    }
+                    inc[w] = pin;
+                    old[w] = ph + pin;
+                    SM[w] = fma(T(0.5), pin, ph);  // phi^{n+1}
+                    DF[w] = pin * A.inv_dt;
+                } else {
+                    lay = lay && Ld[w] != T(1);
+                    const T cy = -((B[2][w] - at(B[2], w - 1)) * A.idx), cz = (B[1][w] - at(B[1], w - 1)) * A.idx;
+                    Eny[w] = dead ? T(0) : half_e(E[1][w], cy, lay, w);
+                    Enz[w] = dead ? T(0) : half_e(E[2][w], cz, lay, w);
+                    BY[w] = fma(T(0.5), B[1][w] + at(B[1], w - 1), By);
+                    BZ[w] = fma(T(0.5), B[2][w] + at(B[2], w - 1), Bz);
+                }
+            }
+            __syncthreads();
+            for (int w = lane; w < W; w += LANES) {
+                const T Dt = DF[w], dphi = (at(SM, w + 1) - at(SM, w - 1)) * A.hidx;
+                if (half == 0) {
+                    PY[w] = fma(-Enz[w], dphi, Dt * BY[w]);
+                } else {
+                    Px[w] = Dt * BXT[w];
+                    PZ[w] = fma(Eny[w], dphi, Dt * BZ[w]);
+                }
+            }
+            __syncthreads();
+            for (int w = lane; w < W; w += LANES) {
+                bool lay = in_layer(w);
+                if (lay && La[w] < T(0)) continue;
+                lay = lay && Ld[w] != T(1);
+                if (half == 0) {
+                    const T X = -A.g * (T(0.5) * (Px[w] + at(Px, w + 1)));
+                    const T Y = fma(-A.g, PY[w], -((B[5][w] - at(B[5], w - 1)) * A.idx));
+                    E[3][w] = half_e(half_e(E[3][w], X, lay, w), X, lay, w);
+                    E[4][w] = half_e(half_e(E[4][w], Y, lay, w), Y, lay, w);
+                } else {
+                    const T Z = fma(-A.g, PZ[w], (B[4][w] - at(B[4], w - 1)) * A.idx);
+                    E[5][w] = half_e(half_e(E[5][w], Z, lay, w), Z, lay, w);
+                    E[1][w] = half_e(Eny[w], -((B[2][w] - at(B[2], w - 1)) * A.idx), lay, w);
+                    E[2][w] = half_e(Enz[w], (B[1][w] - at(B[1], w - 1)) * A.idx, lay, w);
+                }
+            }
+            T *t = cur;
+            cur = old;
+            old = t;
             __syncthreads();
         }
         for (int w = H + tid; w < H + own; w += nt) {
@@ -345,7 +452,14 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
                 const T hx = T(-0.5) * A.h2g * Jx, hy = fma(-A.cB, B[5][w] - at(B[5], w - 1), T(-0.5) * A.h2g * PY[w]);
                 const T hz = fma(A.cB, B[4][w] - at(B[4], w - 1), T(-0.5) * A.h2g * PZ[w]);
                 const bool lay = in_layer(w);
-                const T r = lay ? Lr[w] : T(1), ia = lay ? T(1) / La[w] : T(1);
+                T r = T(1), ia = T(1);
+                if (lay && INCR) {
+                    r = Lr[w];
+                    ia = Ld[w] / La[w];
+                } else if (lay) {
+                    r = Lr[w];
+                    ia = T(1) / La[w];
+                }
                 A.En[0][gi] = Eny[w];
                 A.En[1][gi] = Enz[w];
                 A.En[2][gi] = fma(-r, hx, E[3][w]) * ia;

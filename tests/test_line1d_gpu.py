@@ -82,6 +82,28 @@ def test_any_split_of_the_steps_gives_the_same_bits(bc, prec):
         assert a == b
 
 
+@pytest.mark.parametrize("bc", ["pml", "periodic"])
+@pytest.mark.parametrize("nx", [256, 1031])
+def test_fp32_line_gives_the_generic_kernels_bits(nx, bc):
+    """FP32 split: the time-blocked kernel takes the generic single-pass kernel's operations
+    (a power-of-two cell size, as in the workloads; other sizes round 1/dx once more)."""
+    from paper_2406_16796_gb300 import axp
+
+    w = W.vacuum_1d(nx=nx, g=1e-2, m=0.5 * W.K0, precision="fp32")
+    b = W._bcs(bc)
+    grid = w.grid.replace(axion_bc=b, em_bc=b)
+    out = []
+    for kernel in (axp.AXP_KERNEL_AUTO, axp.AXP_KERNEL_FUSED):
+        g = axp.Grid(grid)
+        g.set_kernel(kernel)
+        g.inject_laser(w.lasers[0])
+        g.step(300)
+        out.append(g.fields())
+        g.close()
+    for k in NAMES:
+        assert np.array_equal(out[0][k], out[1][k]), k
+
+
 def test_order0_x_components_keep_the_generic_kernel():
     """A layer damps E0x and B0x, which no curl drives: such a state stays with the
     kernel that treats them."""
