@@ -4,9 +4,13 @@
 // members' sizes, masses, couplings and fields.
 //
 // Work items are (member, x strip, y chunk) tiles of all members, taken from an
-// atomic queue by a grid of resident blocks.  The block finishing the last tile
-// of a member in a launch advances that member's step counter; the last block
-// of the launch rewinds the queue.  A member's buffer roles alternate with
+// atomic queue.  Members of even width, the usual case, run as warp tiles (58 columns,
+// kernels_tm2d_x2.cuh): each warp of a resident grid takes tiles for itself, so members of
+// any width and height fill the chip evenly (16 uneven members of the serving stream, 6.5M
+// cells: 172 us per step with tiles of 250 x 64 cells per block, GROUPAFTER).
+// Members of odd width run as one-column tiles per block, in a launch of their own.  Whoever
+// finishes the last tile of a member in a launch advances that member's step counter; the
+// last to leave rewinds the queue.  A member's buffer roles alternate with
 // period two, so each member carries the kernel parameters of both parities
 // and a tile picks the set its member's step count selects.  Nothing waits on
 // another block: completion is counted with atomics only.
@@ -35,16 +39,19 @@ struct GDev {
     const fused::Params<float> *params;  // [max_grids][2]
     int64_t *done, *steps;               // per member
     int32_t *cnt, *nblk;                 // tiles finished in this launch; tiles per step
-    const GItem *items;
+    const GItem *items;                  // odd-width members' tiles
     int32_t nitems;
-    int32_t *counter, *finished;
+    const int32_t *first;                // warp tiles: first one of each member (max_grids + 1 entries)
+    int32_t members, nwarp;              // entries of `first` in use; warp tiles in all
+    int32_t rows;                        // planes per warp tile
+    int32_t *counter, *finished;         // of the odd-width launch, then of the warp launch
 };
 
 constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct GLayout {
-    size_t params, done, steps, cnt, nblk, items, counter, total;
+    size_t params, done, steps, cnt, nblk, items, first, counter, total;
 };
 
 GLayout glayout(int32_t max_grids, int32_t max_tiles)
@@ -63,29 +70,27 @@ GLayout glayout(int32_t max_grids, int32_t max_tiles)
     off += align_up(sizeof(int32_t) * max_grids);
     L.items = off;
     off += align_up(sizeof(GItem) * (size_t)max_tiles);
+    L.first = off;
+    off += align_up(sizeof(int32_t) * ((size_t)max_grids + 1));
     L.counter = off;
-    off += align_up(2 * sizeof(int32_t));
+    off += align_up(4 * sizeof(int32_t));
     L.total = off;
     return L;
 }
 
-// Blocks of kGroupThreads threads.  A member of even width takes tiles of the
-// two-column form (2 kGroupThreads columns per tile); a member of odd width the
-// one-column tile body (kGroupThreads columns).
+// Admission counts tiles of kVxPair (even width) or kVxOne columns by `chunk` planes.
 constexpr int kGroupThreads = tm2d_x2::NTX;
 constexpr int kVxPair = 2 * kGroupThreads - tm2d_x2::HL - tm2d_x2::HR;  // written columns per tile
 constexpr int kVxOne = kGroupThreads - tm2d::HL - tm2d::HR;
 constexpr size_t kGroupStage = tm2d_x2::stage_bytes(kGroupThreads);
-static_assert(tm2d::stage_bytes<float>(kGroupThreads) <= kGroupStage, "one staging buffer serves both forms");
-
 __host__ __device__ inline int group_vx(int64_t nx) { return nx % 2 == 0 ? kVxPair : kVxOne; }
 
-__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group(GDev D)
+constexpr size_t kOddStage = tm2d::stage_bytes<float>(kGroupThreads);
+
+// members of odd width: one tile per block at a time
+__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group_odd(GDev D)
 {
-    // the published rows of either form
-    constexpr size_t kRowsOne = sizeof(float) * 2 * tm2d::NROWS * tm2d::RS;
-    constexpr size_t kRowsPair = sizeof(float2) * 2 * tm2d_x2::NROWS * tm2d_x2::RS;
-    __shared__ __align__(16) unsigned char rows_raw[kRowsOne > kRowsPair ? kRowsOne : kRowsPair];
+    __shared__ float rows[2][tm2d::NROWS][tm2d::RS];
     extern __shared__ __align__(16) unsigned char group_dyn[];
     __shared__ fused::Params<float> sP;
     __shared__ int s_item;
@@ -108,13 +113,7 @@ __global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group(GDev D)
             const int *src = (const int *)(D.params + 2 * (size_t)I.member + (done & 1));
             for (int k = threadIdx.x; k < kWords; k += kGroupThreads) ((int *)&sP)[k] = src[k];
             __syncthreads();
-            if (sP.n[0] % 2 == 0)
-                tm2d_x2::tile(sP, I.bx, I.by,
-                              *reinterpret_cast<float2(*)[2][tm2d_x2::NROWS][tm2d_x2::RS]>(rows_raw),
-                              reinterpret_cast<float2 *>(group_dyn));
-            else
-                tm2d::tile<float, true>(sP, I.bx, I.by, *reinterpret_cast<float(*)[2][tm2d::NROWS][tm2d::RS]>(rows_raw),
-                                        reinterpret_cast<float *>(group_dyn));
+            tm2d::tile<float, true>(sP, I.bx, I.by, rows, reinterpret_cast<float *>(group_dyn));
             __syncthreads();
             if (threadIdx.x == 0) {
                 __threadfence();  // this tile's stores before the count that publishes them
@@ -132,6 +131,57 @@ __global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group(GDev D)
             // every block has taken its last item: rewind the queue for the next launch
             *D.counter = 0;
             *D.finished = 0;
+        }
+    }
+}
+
+// members of even width: each warp takes warp tiles for itself.  No block-wide barrier is
+// met inside the loop, and no warp waits for another.
+__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group(GDev D)
+{
+    constexpr int kWarps = kGroupThreads / 32;
+    __shared__ __align__(16) float yring[kWarps][tm2d_x2::YR][tm2d_x2::NY + 1];
+    __shared__ fused::Params<float> sP[kWarps];
+    extern __shared__ __align__(16) unsigned char group_dyn[];
+    const int w = (int)(threadIdx.x / 32), lane = (int)(threadIdx.x % 32);
+    constexpr int kWords = sizeof(fused::Params<float>) / sizeof(int);
+    static_assert(sizeof(fused::Params<float>) % sizeof(int) == 0, "Params copied as words");
+    int32_t *counter = D.counter + 2, *finished = D.finished + 2;
+    for (;;) {
+        int u = 0;
+        if (lane == 0) u = atomicAdd(counter, 1);
+        u = __shfl_sync(0xffffffffu, u, 0);
+        if (u >= D.nwarp) break;
+        int lo = 0, hi = D.members;  // the member with first[lo] <= u < first[lo + 1]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) / 2;
+            if (__ldg(D.first + mid) <= u) lo = mid;
+            else hi = mid;
+        }
+        const int m = lo, tile = u - __ldg(D.first + m);
+        // the member's step count is stable while any of its tiles is unfinished
+        const int64_t done = (int64_t)__ldcg(D.done + m);
+        if (done >= (int64_t)__ldcg(D.steps + m)) continue;
+        const int *src = (const int *)(D.params + 2 * (size_t)m + (done & 1));
+        __syncwarp();
+        for (int k = lane; k < kWords; k += 32) ((int *)&sP[w])[k] = src[k];
+        __syncwarp();
+        const int strips = (sP[w].n[0] + tm2d_x2::WVX - 1) / tm2d_x2::WVX, m0 = tile / strips * D.rows;
+        tm2d_x2::tile_span<true>(sP[w], tile % strips, m0, min(sP[w].n[1], m0 + D.rows), nullptr,
+                                 reinterpret_cast<float2 *>(group_dyn), yring[w]);
+        __threadfence();  // this tile's stores before the count that publishes them
+        __syncwarp();
+        if (lane == 0 && atomicAdd(D.cnt + m, 1) == D.nblk[m] - 1) {
+            D.cnt[m] = 0;
+            D.done[m] = done + 1;
+        }
+    }
+    if (lane == 0) {
+        __threadfence();
+        if (atomicAdd(finished, 1) == (int)gridDim.x * kWarps - 1) {
+            // every warp has taken its last item: rewind the queue for the next launch
+            *counter = 0;
+            *finished = 0;
         }
     }
 }
@@ -162,8 +212,9 @@ struct axp_group {
     };
     std::vector<Member> members;
     int32_t chunk;  // y planes per tile
+    bool chunk_given;  // by axp_group_set_chunk; else warp tiles take the planes that fill the chip best
     bool dirty;
-    int grid_blocks;
+    int grid_blocks, odd_blocks;  // resident blocks of the two kernels
     int64_t launches;
     bool use_graph;
     cudaGraphExec_t graph;
@@ -187,36 +238,83 @@ int32_t tiles_of(const axp_grid *g, int32_t chunk)
     return (int32_t)(strips * chunks);
 }
 
+// Planes per warp tile: the fewest waves of resident warps times rows + 6 planes of
+// pipeline, over all members.
+int32_t warp_rows(const axp_group *G)
+{
+    if (G->chunk_given) return G->chunk;
+    const int64_t slots = (int64_t)G->grid_blocks * (kGroupThreads / 32);
+    int32_t best = 64;
+    double best_cost = 0.0;
+    for (int32_t rows = 16; rows <= 512; rows++) {
+        int64_t tiles = 0;
+        for (const auto &M : G->members)
+            if (M.active && M.g->desc.n[0] % 2 == 0)
+                tiles += (M.g->desc.n[0] + tm2d_x2::WVX - 1) / tm2d_x2::WVX * ((M.g->desc.n[1] + rows - 1) / rows);
+        const double cost = (double)((tiles + slots - 1) / slots) * (double)(rows + 6);
+        if (rows == 16 || cost < best_cost) {
+            best_cost = cost;
+            best = rows;
+        }
+    }
+    return best;
+}
+
 axp_status rebuild(axp_group *G)
 {
     std::vector<GItem> items;
+    std::vector<int32_t> first(G->max_grids + 1, 0), nblk(G->max_grids, 0);
+    G->D.rows = warp_rows(G);
+    int64_t tiles = 0, warp_tiles = 0;
     for (int m = 0; m < G->max_grids; m++) {
         const auto &M = G->members[m];
+        first[m] = (int32_t)warp_tiles;
         if (!M.active) continue;
-        const int vx = group_vx(M.g->desc.n[0]);
-        const int strips = (int)((M.g->desc.n[0] + vx - 1) / vx);
-        const int chunks = (int)((M.g->desc.n[1] + G->chunk - 1) / G->chunk);
+        tiles += M.nblk;
+        const int64_t nx = M.g->desc.n[0], ny = M.g->desc.n[1];
+        if (nx % 2 == 0) {
+            const int64_t n = (nx + tm2d_x2::WVX - 1) / tm2d_x2::WVX * ((ny + G->D.rows - 1) / G->D.rows);
+            nblk[m] = (int32_t)n;
+            warp_tiles += n;
+            continue;
+        }
+        const int vx = group_vx(nx);
+        const int strips = (int)((nx + vx - 1) / vx);
+        const int chunks = (int)((ny + G->chunk - 1) / G->chunk);
+        nblk[m] = strips * chunks;
         for (int by = 0; by < chunks; by++)
             for (int bx = 0; bx < strips; bx++) items.push_back({m, bx, by, 0});
     }
-    if ((int64_t)items.size() > G->max_tiles) return AXP_E_NOMEM;
+    first[G->max_grids] = (int32_t)warp_tiles;
+    if (tiles > G->max_tiles || warp_tiles > INT32_MAX) return AXP_E_NOMEM;
     cudaError_t e = cudaSuccess;
     if (!items.empty())
         e = cudaMemcpyAsync(G->ws + G->L.items, items.data(), items.size() * sizeof(GItem), cudaMemcpyHostToDevice,
                             G->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(G->ws + G->L.first, first.data(), first.size() * sizeof(int32_t), cudaMemcpyHostToDevice, G->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(G->ws + G->L.nblk, nblk.data(), nblk.size() * sizeof(int32_t), cudaMemcpyHostToDevice, G->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(G->stream);
     if (e != cudaSuccess) return cuda_st(e);
     G->D.nitems = (int32_t)items.size();
+    G->D.nwarp = (int32_t)warp_tiles;
     G->dirty = false;
     return AXP_OK;
 }
 
 cudaError_t enqueue(axp_group *G, int64_t nsteps)
 {
-    const int grid = std::max(1, std::min(G->grid_blocks, G->D.nitems));
     for (int64_t s = 0; s < nsteps; s++) {
-        k_tm2d_group<<<grid, kGroupThreads, kGroupStage, G->stream>>>(G->D);
-        G->launches++;
+        if (G->D.nwarp > 0) {
+            const int most = (G->D.nwarp + kGroupThreads / 32 - 1) / (kGroupThreads / 32);
+            k_tm2d_group<<<std::min(G->grid_blocks, most), kGroupThreads, kGroupStage, G->stream>>>(G->D);
+            G->launches++;
+        }
+        if (G->D.nitems > 0) {
+            k_tm2d_group_odd<<<std::min(G->odd_blocks, G->D.nitems), kGroupThreads, kOddStage, G->stream>>>(G->D);
+            G->launches++;
+        }
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -256,6 +354,11 @@ axp_status axp_group_create(int32_t max_grids, int32_t max_tiles, void *dev_work
     G->D.nblk = (int32_t *)(G->ws + L.nblk);
     G->D.items = (const GItem *)(G->ws + L.items);
     G->D.nitems = 0;
+    G->D.first = (const int32_t *)(G->ws + L.first);
+    G->D.members = max_grids;
+    G->D.nwarp = 0;
+    G->D.rows = 64;
+    G->chunk_given = false;
     G->D.counter = (int32_t *)(G->ws + L.counter);
     G->D.finished = G->D.counter + 1;
     G->members.assign(max_grids, axp_group::Member{nullptr, 0, 0, 0});
@@ -273,6 +376,11 @@ axp_status axp_group_create(int32_t max_grids, int32_t max_tiles, void *dev_work
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tm2d_group, kGroupThreads, kGroupStage);
     G->grid_blocks = sms * std::max(1, occ);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tm2d_group_odd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOddStage);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tm2d_group_odd, kGroupThreads, kOddStage);
+    G->odd_blocks = sms * std::max(1, occ);
     if (e == cudaSuccess) e = cudaMemsetAsync(G->ws, 0, L.total, G->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(G->stream);
     if (e != cudaSuccess) {
@@ -322,12 +430,11 @@ axp_status axp_group_add(axp_group *G, axp_grid *g, int64_t steps, int32_t *memb
     P[1] = tm2d_params<float>(g, G->chunk);
     rotate_roles(g);  // period two: back to the present roles
     const int64_t zero = 0;
-    const int32_t nblk = tiles_of(g, G->chunk), zero32 = 0;
+    const int32_t nblk = tiles_of(g, G->chunk), zero32 = 0;  // (the launches' own counts: rebuild)
     e = cudaMemcpyAsync((void *)(G->D.params + 2 * (size_t)m), P, sizeof(P), cudaMemcpyHostToDevice, G->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(G->D.done + m, &zero, sizeof(zero), cudaMemcpyHostToDevice, G->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(G->D.steps + m, &steps, sizeof(steps), cudaMemcpyHostToDevice, G->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(G->D.cnt + m, &zero32, sizeof(zero32), cudaMemcpyHostToDevice, G->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(G->D.nblk + m, &nblk, sizeof(nblk), cudaMemcpyHostToDevice, G->stream);
     // the host sources above must outlive the copies
     if (e == cudaSuccess) e = cudaStreamSynchronize(G->stream);
     if (e != cudaSuccess) return cuda_st(e);
@@ -379,6 +486,7 @@ axp_status axp_group_set_chunk(axp_group *G, int32_t rows)
     for (auto &M : G->members)
         if (M.active) return AXP_E_STATE;  // tiles of present members are fixed
     G->chunk = rows;
+    G->chunk_given = true;
     drop_graph(G);
     G->dirty = true;
     return AXP_OK;
@@ -409,7 +517,7 @@ axp_status axp_group_run(axp_group *G, int64_t nsteps)
         const axp_status st = rebuild(G);
         if (st != AXP_OK) return st;
     }
-    if (G->D.nitems == 0) return AXP_OK;
+    if (G->D.nitems == 0 && G->D.nwarp == 0) return AXP_OK;
     if (!G->use_graph || G->stream == nullptr) return cuda_st(enqueue(G, nsteps));
     if (!G->graph || G->graph_steps != nsteps) {
         drop_graph(G);
@@ -432,7 +540,7 @@ axp_status axp_group_run(axp_group *G, int64_t nsteps)
         }
         G->graph_steps = nsteps;
     }
-    G->launches += nsteps;
+    G->launches += nsteps * ((G->D.nwarp > 0) + (G->D.nitems > 0));
     return cuda_st(cudaGraphLaunch(G->graph, G->stream));
 }
 

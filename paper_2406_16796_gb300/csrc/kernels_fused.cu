@@ -20,6 +20,7 @@ cudaError_t fused_dispatch_f32(int mode, int set, const fused::Params<float> &P,
 cudaError_t tm2d_dispatch_f64(const fused::Params<double> &P, int nchunks, cudaStream_t s, int *occ, int tx);
 cudaError_t tm2d_dispatch_f32(const fused::Params<float> &P, int nchunks, cudaStream_t s, int *occ, int tx);
 cudaError_t tm2d_x2_dispatch_f32(const fused::Params<float> &P, int nchunks, cudaStream_t s, int *occ, int cols);
+cudaError_t tm2d_x2_warps_dispatch_f32(const fused::Params<float> &P, int ntiles, cudaStream_t s, int *resident);
 cudaError_t tm2d_list_dispatch_f64(const fused::Params<double> &P, const int4 *items, int nblocks, int per_block,
                                    cudaStream_t s, int *occ, int tx);
 cudaError_t ax3d_dispatch_f64(const fused::Params<double> &P, int nchunks, cudaStream_t s, int *occ);
@@ -885,6 +886,46 @@ cudaError_t step_graph(axp_grid *g, Launch &&launch_one, cudaGraphExec_t *out)
 // 400 x 400 44 / 107, 1024 x 512 109 / 142, 800 x 800 131 / 142, 1024 x 768 157 / 142.
 constexpr int64_t kSmallTm = 700000;
 
+// FP32 grids of the 2D kernel up to this many cells take the warp tiles: they split a small
+// or ragged grid more evenly.  Beyond it the state no longer fits L2, and the block tiles'
+// longer rows are the better HBM access.  us per step, block / warp tiles: 512 x 256 15.6 / 14.5,
+// 1024 x 512 20.7 / 20.7, 1024 x 1024 41.9 / 27.0, 1536 x 768 37.3 / 29.0, 600 x 2048 33.0 / 35.1,
+// 2048 x 768 38.9 / 40.8, 2048 x 2048 71 / 91, 4096 x 2048 125 / 130.
+constexpr int64_t kWarpMost = 1200000;
+
+// March chunks of the FP32 2D kernel's warp tiles: the fewest waves of resident warps times
+// chunk + 6 planes of pipeline.  A strip at a non-periodic x edge takes 1.35 times as long
+// per plane and a chunk over a y layer 0.32 planes' time more for each of the layer's (and 7
+// pipeline) planes; their chunks are shortened by that (1.0 and 0: 1536 x 768 29.5 us
+// against 27.0; 2.0 and 0.6: 29.0).
+struct WarpPlan {
+    int chunk, first, edge, ntiles;
+};
+WarpPlan warp_plan(const axp_grid *g, int resident)
+{
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
+    const axp_grid_desc &d = g->desc;
+    const bool perx = d.em_bc[0][0] == AXP_BC_PERIODIC, pery = d.em_bc[1][0] == AXP_BC_PERIODIC;
+    const int64_t ny = d.n[1], strips = (d.n[0] + tm2d_x2::WVX - 1) / tm2d_x2::WVX, nedge = perx ? 0 : std::min<int64_t>(strips, 2);
+    const int64_t slots = (int64_t)sms * resident, shorter = pery ? 0 : (int64_t)(0.32 * (double)(d.pml_cells + 7));
+    WarpPlan best{0, 0, 0, 0};
+    double best_cost = 0.0;
+    for (int64_t chunk = std::min<int64_t>(ny, 4); chunk <= ny; chunk++) {
+        const int64_t least = std::min<int64_t>(chunk, 4);
+        const int64_t first = std::min(ny, std::max(least, chunk - shorter));
+        const int64_t edge = std::max(least, (int64_t)((double)(chunk + 6) / 1.35) - 6);
+        const int64_t nin = 1 + (ny - first + chunk - 1) / chunk, nout = (ny + edge - 1) / edge;
+        const int64_t tiles = (strips - nedge) * nin + nedge * nout;
+        const double cost = (double)((tiles + slots - 1) / slots) * (double)(chunk + 6);
+        if (best.chunk == 0 || cost < best_cost) {
+            best_cost = cost;
+            best = WarpPlan{(int)chunk, (int)first, (int)edge, (int)tiles};
+        }
+    }
+    return best;
+}
+
 template <typename T>
 cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
 {
@@ -977,6 +1018,17 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
         nchunks = (int)((nm + chunk - 1) / chunk);
         P.chunk = (int)chunk;
     }
+    WarpPlan wp{0, 0, 0, 0};
+    if constexpr (sizeof(T) == 4) {
+        if (x2 && g->desc.n[0] * g->desc.n[1] <= kWarpMost) {
+            int resident = 0;
+            if ((e = tm2d_x2_warps_dispatch_f32(P, 0, g->stream, &resident)) != cudaSuccess) return e;
+            wp = warp_plan(g, resident);
+            P.chunk = wp.chunk;
+            P.chunk_first = wp.first;
+            P.chunk_edge = wp.edge;
+        }
+    }
     int64_t it = 0;
     if (mode == 1 && !tm && !ax && g->desc.diag_every == 0 && nsteps >= kGraphSteps) {
         auto one = [&](const fused::Params<T> &Pl, cudaStream_t st) {
@@ -1000,7 +1052,10 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
             P.chunk_edge = che;
             P.chunk_first = chf;
         }
-        e = launch(P, nchunks, nullptr);
+        if constexpr (sizeof(T) == 4)
+            e = wp.ntiles > 0 ? tm2d_x2_warps_dispatch_f32(P, wp.ntiles, g->stream, nullptr) : launch(P, nchunks, nullptr);
+        else
+            e = launch(P, nchunks, nullptr);
         if (e != cudaSuccess) return e;
         g->launches++;
         rotate_roles(g);

@@ -21,6 +21,11 @@ cudaError_t tm2d_x2_dispatch_f32(const fused::Params<float> &P, int nchunks, cud
     return tm2d_x2::launch(P, nchunks, s, occ, cols);
 }
 
+cudaError_t tm2d_x2_warps_dispatch_f32(const fused::Params<float> &P, int ntiles, cudaStream_t s, int *resident)
+{
+    return tm2d_x2::launch_warps(P, ntiles, s, resident);
+}
+
 // FP32-split axion box: the two-cell form on an even-width grid
 cudaError_t ax3d_dispatch_f32(const fused::Params<float> &P, int nchunks, cudaStream_t s, int *occ)
 {

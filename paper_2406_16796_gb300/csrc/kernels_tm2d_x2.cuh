@@ -46,32 +46,35 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 min2(float2 a, float2 b) { return make_float2(fminf(a.x, b.x), fminf(a.y, b.y)); }
 __device__ __forceinline__ float2 max2(float2 a, float2 b) { return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y)); }
-// the pair one column to the right / left: (own.y, right.x) and (left.y, own.x)
-__device__ __forceinline__ float2 right_of(float2 own, const float2 *row, int t) { return make_float2(own.y, row[t + 2].x); }
-__device__ __forceinline__ float2 left_of(float2 own, const float2 *row, int t) { return make_float2(row[t].y, own.x); }
 
 enum { R_E0Z, R_E1Y, R_E1Z, R_PHI, R_N0Y2, R_MID3, R_N0Y3, R_PX4, R_N1Z4, R_N1Y4, R_N0Y4, NROWS };
 
-__device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx, const int by,
-                                     float2 (&rows)[2][NROWS][RS], float2 *stage)
-{
-    const int ntx = (int)blockDim.x, vx = 2 * ntx - HL - HR;  // written columns of this launch's tiles
-    for (int i = threadIdx.x; i < 2 * NROWS * RS; i += ntx) (&rows[0][0][0])[i] = make_float2(0.f, 0.f);
+enum { Y_A1, Y_B1, Y_A2, Y_B2, Y_K1, Y_K2, Y_SA, NY };  // a plane's y coefficients
+constexpr int YR = 16;                                    // planes of their ring
+constexpr int WVX = 64 - HL - HR;                         // columns a warp's tile writes
 
-    const int tx = threadIdx.x;
+// One tile: columns from bx times its written columns on, planes [m0, m1).  It belongs to
+// the block (WARP = false: x neighbours across threads go through the shared rows, one
+// barrier per plane) or to one warp of it (WARP = true: 64 columns, x neighbours by
+// shuffles, no barrier and no shared rows; the warps march on their own).  The arithmetic
+// per cell is the same.  The warp form recomputes more halo (6 of 64 columns against 6 of
+// 256) and reads shorter rows, but waits for no other warp and leaves less of a strip
+// unused at a grid's edge; where each is taken: kWarpMost (kernels_fused.cu).
+template <bool WARP>
+__device__ __forceinline__ void tile_span(const fused::Params<float> &P, const int bx, const int m0, const int m1,
+                                          float2 (*rows)[NROWS][RS], float2 *stage, float (*yring)[NY + 1])
+{
+    const int ntx = (int)blockDim.x;
+    const int tx = WARP ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+    const int cols = WARP ? 64 : 2 * ntx, vx = cols - HL - HR;  // the tile's columns, and those written
+    if (!WARP)
+        for (int i = threadIdx.x; i < 2 * NROWS * RS; i += ntx) (&rows[0][0][0])[i] = make_float2(0.f, 0.f);
     const int nx = P.n[0], ny = P.n[1];
     const bool perx = P.per[0], pery = P.per[1];
     const int gx = bx * vx - HL + 2 * tx;  // first column of the pair (even)
     int wx = gx;
     if (wx < 0 || wx >= nx) wx = perx ? ((wx % nx) + nx) % nx : -1;
-    const bool write_col = 2 * tx >= HL && 2 * tx < 2 * ntx - HR && gx >= 0 && gx < nx;
-    const int nstrips = (nx + vx - 1) / vx;
-    const bool xstrip = !perx && (bx == 0 || bx == nstrips - 1);
-    const int chunk = xstrip ? P.chunk_edge : P.chunk;
-    const int first = xstrip ? P.chunk_edge : P.chunk_first;
-    const int m0 = by == 0 ? 0 : first + (by - 1) * chunk;
-    if (m0 >= ny) return;
-    const int m1 = min(ny, by == 0 ? first : m0 + chunk);
+    const bool write_col = 2 * tx >= HL && 2 * tx < cols - HR && gx >= 0 && gx < nx;
     const int gx0 = bx * vx - HL;
     const int wx0 = gx0 + 2 * (tx & ~31), wx1 = wx0 + 63;  // columns of this warp
     const bool tile_fast = perx || (wx0 - 1 >= P.lay[0][0] && wx1 + 1 <= nx - 1 - P.lay[0][1]);
@@ -98,9 +101,6 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
     const float2 kx1 = colcoef(4, P.dt2), kx2 = colcoef(5, 1.f);
     const float2 sxa = xl ? make_float2(P.sig_ax[0][wx], P.sig_ax[0][wx + 1]) : f2(0.f);
 
-    enum { Y_A1, Y_B1, Y_A2, Y_B2, Y_K1, Y_K2, Y_SA, NY };
-    constexpr int YR = 16;
-    __shared__ __align__(16) float yring[YR][NY + 1];
     auto fill_y = [&](int p) {
         if (tx < NY) {
             float *dst = &yring[p & (YR - 1)][tx];
@@ -141,7 +141,7 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
         if (wp < 0 || wp >= ny) wp = pery ? ((wp % ny) + ny) % ny : -1;
         const bool ok = wx >= 0 && wp >= 0;
         const unsigned o = ok ? (unsigned)wx + (unsigned)nx * (unsigned)wp : 0u;
-        float2 *st = stage + ((p - t0) & (NS - 1)) * (NIN * ntx) + tx;
+        float2 *st = stage + ((p - t0) & (NS - 1)) * (NIN * ntx) + threadIdx.x;
         cp_pair(st + 0 * ntx, P.Ein[2] + o, ok);
         cp_pair(st + 1 * ntx, P.Ein[3] + o, ok);
         cp_pair(st + 2 * ntx, P.Ein[4] + o, ok);
@@ -155,7 +155,7 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
         cp_pair(st + 10 * ntx, P.phib + o, ok);
     };
     auto take = [&](int p) {
-        const float2 *st = stage + ((p - t0) & (NS - 1)) * (NIN * ntx) + tx;
+        const float2 *st = stage + ((p - t0) & (NS - 1)) * (NIN * ntx) + threadIdx.x;
         E0z0 = st[0 * ntx];
         E1x0 = st[1 * ntx];
         E1y0 = st[2 * ntx];
@@ -186,14 +186,20 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
 
     auto body = [&](auto edge_tag, int t, int b) {
         constexpr bool EDGE = decltype(edge_tag)::value;
-        float2(*R)[RS] = rows[b];
+        // the pair one column to the right / left: (own.y, right.x) and (left.y, own.x)
+        auto right_of = [&](float2 own, int row) {
+            return make_float2(own.y, WARP ? __shfl_down_sync(0xffffffffu, own.x, 1) : rows[b][row][tx + 2].x);
+        };
+        auto left_of = [&](float2 own, int row) {
+            return make_float2(WARP ? __shfl_up_sync(0xffffffffu, own.y, 1) : rows[b][row][tx].y, own.x);
+        };
         // ---- stage 1: B^{n+1} on plane t-1 ----
         {
             const int p = t - 1;
             const bool in = !EDGE || inside(p);
-            const float2 d0y = sub2(E0z0, E0z1), d0x = sub2(right_of(E0z1, R[R_E0Z], tx), E0z1);
-            const float2 d1zy = sub2(E1z0, E1z1), d1zx = sub2(right_of(E1z1, R[R_E1Z], tx), E1z1);
-            const float2 d1yx = sub2(right_of(E1y1, R[R_E1Y], tx), E1y1), d1xy = sub2(E1x0, E1x1);
+            const float2 d0y = sub2(E0z0, E0z1), d0x = sub2(right_of(E0z1, R_E0Z), E0z1);
+            const float2 d1zy = sub2(E1z0, E1z1), d1zx = sub2(right_of(E1z1, R_E1Z), E1z1);
+            const float2 d1yx = sub2(right_of(E1y1, R_E1Y), E1y1), d1xy = sub2(E1x0, E1x1);
             auto plain = [&]() {
                 N0x1 = fma2(f2(-h2y), d0y, B0x1);
                 N0y1 = fma2(f2(h2x), d0x, B0y1);
@@ -234,7 +240,7 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
         {
             const int p = t - 2;
             const bool in = !EDGE || inside(p);
-            const float2 spx = add2(sub2(right_of(ph2, R[R_PHI], tx), ph2), sub2(left_of(ph2, R[R_PHI], tx), ph2));
+            const float2 spx = add2(sub2(right_of(ph2, R_PHI), ph2), sub2(left_of(ph2, R_PHI), ph2));
             const float2 spy = add2(sub2(ph1, ph2), sub2(ph3, ph2));
             float2 sa = z2;
             if (EDGE && in && P.has_pml) sa = pery ? sxa : max2(sxa, f2(yring[p & (YR - 1)][Y_SA]));
@@ -266,7 +272,7 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
                 store(P.phib_out, gi, pin);
             }
             // E0z^{n+1} = E0z^{n+1/2} + h (curl B0)_z, backward differences
-            const float2 dbx = sub2(N0y2, left_of(N0y2, R[R_N0Y2], tx)), dby = sub2(N0x2, N0x3);
+            const float2 dbx = sub2(N0y2, left_of(N0y2, R_N0Y2)), dby = sub2(N0x2, N0x3);
             if (!EDGE) {
                 EN2 = fma2(f2(hx), dbx, fma2(f2(-hy), dby, E0z2));
             } else {
@@ -282,9 +288,9 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
         {
             const int p = t - 3;
             const float2 bbx = fma2(f2(hinv_dt), add2(N0x3, N0x4), f2(Bxi));
-            const float2 bby = fma2(f2(hinv_dt), add2(N0y3, left_of(N0y3, R[R_N0Y3], tx)), f2(Byi));
+            const float2 bby = fma2(f2(hinv_dt), add2(N0y3, left_of(N0y3, R_N0Y3)), f2(Byi));
             const float2 dpy = mul2(sub2(SM2, SM4), f2(qidy));
-            const float2 dpx = mul2(sub2(right_of(SM3, R[R_MID3], tx), left_of(SM3, R[R_MID3], tx)), f2(qidx));
+            const float2 dpx = mul2(sub2(right_of(SM3, R_MID3), left_of(SM3, R_MID3)), f2(qidx));
             PX3 = fma2(EN3, dpy, mul2(DF3, bbx));
             PY3 = fma2(mul2(EN3, f2(-1.f)), dpx, mul2(DF3, bby));
             if (EDGE && !inside(p)) PX3 = PY3 = z2;
@@ -294,9 +300,11 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
             const int p = t - 4;
             if (p >= m0 && p < m1) {
                 const bool in = !EDGE || inside(p);
-                const float2 sjx = add2(PX4, right_of(PX4, R[R_PX4], tx)), sjy = add2(PY4, PY3);
-                const float2 e1zy = sub2(N1z4, N1z5), e1zx = sub2(N1z4, left_of(N1z4, R[R_N1Z4], tx));
-                const float2 e1yx = sub2(N1y4, left_of(N1y4, R[R_N1Y4], tx)), e1xy = sub2(N1x4, N1x5);
+                const float2 sjx = add2(PX4, right_of(PX4, R_PX4)), sjy = add2(PY4, PY3);
+                const float2 e1zy = sub2(N1z4, N1z5), e1zx = sub2(N1z4, left_of(N1z4, R_N1Z4));
+                const float2 e1yx = sub2(N1y4, left_of(N1y4, R_N1Y4)), e1xy = sub2(N1x4, N1x5);
+                // (a shuffle: taken outside the lanes' branches)
+                const float2 n0l = EDGE ? left_of(N0y4, R_N0Y4) : z2;
                 float2 ex, ey, ez, e0;
                 auto plain = [&]() {
                     ex = fma2(f2(h2y), e1zy, fma2(f2(-hg), sjx, E1x4));
@@ -315,7 +323,7 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
                         const float2 xx = fma2(f2(-g), mul2(f2(0.5f), sjx), mul2(e1zy, f2(idy)));
                         const float2 xy = fma2(f2(-g), mul2(f2(0.5f), sjy), mul2(e1zx, f2(-idx)));
                         const float2 xz = fma2(f2(-gBzi), DF4, fma2(e1yx, f2(idx), mul2(e1xy, f2(-idy))));
-                        const float2 e0yx = sub2(N0y4, left_of(N0y4, R[R_N0Y4], tx)), e0xy = sub2(N0x4, N0x5);
+                        const float2 e0yx = sub2(N0y4, n0l), e0xy = sub2(N0x4, N0x5);
                         ex = fma2(b2, xx, mul2(a2, E1x4));
                         ey = fma2(b2, xy, mul2(a2, E1y4));
                         ez = fma2(b2, xz, mul2(a2, E1z4));
@@ -340,13 +348,13 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
     }
     tm2d::cp_wait<NS - 2>();
     if (!dead) take(t0);
-    __syncthreads();
+    if (!WARP) __syncthreads();
 #pragma unroll 2
     for (int t = t0; t <= t1; ++t) {
         if (!dead && t + NS - 1 <= t1) prefetch(t + NS - 1);
         tm2d::cp_commit();
         const int b = (t - t0) & 1;
-        if (!dead) {
+        if (!WARP && !dead) {
         rows[b][R_E0Z][tx + 1] = E0z1;
         rows[b][R_E1Y][tx + 1] = E1y1;
         rows[b][R_E1Z][tx + 1] = E1z1;
@@ -359,7 +367,8 @@ __device__ __forceinline__ void tile(const fused::Params<float> &P, const int bx
         rows[b][R_N1Y4][tx + 1] = N1y4;
         rows[b][R_N0Y4][tx + 1] = N0y4;
         }
-        __syncthreads();
+        if (WARP) __syncwarp();  // (the y coefficients are copied by the first lanes)
+        else __syncthreads();
         const bool fast = tile_fast && (pery || (t - 6 >= ylo && t + 1 <= yhi));
         if (dead) {
         } else if (fast) {
@@ -391,8 +400,39 @@ template <int UNUSED = 0>
 __global__ void __launch_bounds__(NTX, 2) k_tm2d_x2(fused::Params<float> P)
 {
     __shared__ float2 rows[2][NROWS][RS];
+    __shared__ __align__(16) float yring[YR][NY + 1];
     extern __shared__ __align__(16) unsigned char tm2d_x2_dyn[];
-    tile(P, (int)blockIdx.x, (int)blockIdx.y, rows, reinterpret_cast<float2 *>(tm2d_x2_dyn));
+    const int bx = (int)blockIdx.x, by = (int)blockIdx.y, ny = P.n[1];
+    const int vx = 2 * (int)blockDim.x - HL - HR;
+    const bool xstrip = !P.per[0] && (bx == 0 || bx == (P.n[0] + vx - 1) / vx - 1);
+    const int chunk = xstrip ? P.chunk_edge : P.chunk, first = xstrip ? P.chunk_edge : P.chunk_first;
+    const int m0 = by == 0 ? 0 : first + (by - 1) * chunk;
+    if (m0 >= ny) return;
+    tile_span<false>(P, bx, m0, min(ny, by == 0 ? first : m0 + chunk), rows, reinterpret_cast<float2 *>(tm2d_x2_dyn), yring);
+}
+
+// Warp tiles: the strips at a non-periodic x edge first (chunks of chunk_edge planes, they
+// take longest), then the others (chunks of chunk planes, the first of chunk_first).
+template <int UNUSED = 0>
+__global__ void __launch_bounds__(NTX, 2) k_tm2d_x2_warp(fused::Params<float> P, int nstrips, int ntiles)
+{
+    __shared__ __align__(16) float yring[NTX / 32][YR][NY + 1];
+    extern __shared__ __align__(16) unsigned char tm2d_x2_dyn[];
+    const int w = (int)(threadIdx.x / 32), q = (int)blockIdx.x * (int)(blockDim.x / 32) + w;
+    if (q >= ntiles) return;
+    const int ny = P.n[1], nedge = P.per[0] ? 0 : min(nstrips, 2), ne = nedge * ((ny + P.chunk_edge - 1) / P.chunk_edge);
+    int bx, m0, m1;
+    if (q < ne) {
+        bx = q % nedge == 0 ? 0 : nstrips - 1;
+        m0 = (q / nedge) * P.chunk_edge;
+        m1 = min(ny, m0 + P.chunk_edge);
+    } else {
+        const int r = q - ne, nin = nstrips - nedge, by = r / nin;
+        bx = r % nin + (nedge ? 1 : 0);
+        m0 = by == 0 ? 0 : P.chunk_first + (by - 1) * P.chunk;
+        m1 = min(ny, P.chunk_first + by * P.chunk);
+    }
+    tile_span<true>(P, bx, m0, m1, nullptr, reinterpret_cast<float2 *>(tm2d_x2_dyn), yring[w]);
 }
 
 }  // namespace tm2d_x2
@@ -419,6 +459,22 @@ inline cudaError_t launch(const fused::Params<float> &P, int nchunks, cudaStream
     const int vx = cols - HL - HR;
     dim3 grid((P.n[0] + vx - 1) / vx, nchunks, 1);
     k_tm2d_x2<><<<grid, ntx, dyn, stream>>>(P);
+    return cudaGetLastError();
+}
+
+// ntiles warp tiles of P's chunks; 0 only reports the resident warps per SM.
+inline cudaError_t launch_warps(const fused::Params<float> &P, int ntiles, cudaStream_t stream, int *resident)
+{
+    static int occ = 0;
+    if (occ == 0) {
+        cudaError_t e = cudaFuncSetAttribute(k_tm2d_x2_warp<>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage_bytes());
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tm2d_x2_warp<>, NTX, stage_bytes());
+        if (e != cudaSuccess) return e;
+    }
+    if (resident) *resident = occ * (NTX / 32);
+    if (ntiles <= 0) return cudaSuccess;
+    const int nstrips = (P.n[0] + WVX - 1) / WVX;
+    k_tm2d_x2_warp<><<<(ntiles + NTX / 32 - 1) / (NTX / 32), NTX, stage_bytes(), stream>>>(P, nstrips, ntiles);
     return cudaGetLastError();
 }
 
