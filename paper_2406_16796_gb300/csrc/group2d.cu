@@ -7,7 +7,7 @@
 // atomic queue.  Members of even width, the usual case, run as warp tiles (58 columns,
 // kernels_tm2d_x2.cuh): each warp of a resident grid takes tiles for itself, so members of
 // any width and height fill the chip evenly (16 uneven members of the serving stream, 6.5M
-// cells: 172 us per step with tiles of 250 x 64 cells per block, GROUPAFTER).
+// cells: 172 us per step with tiles of 250 x 64 cells per block, 136 now).
 // Members of odd width run as one-column tiles per block, in a launch of their own.  Whoever
 // finishes the last tile of a member in a launch advances that member's step counter; the
 // last to leave rewinds the queue.  A member's buffer roles alternate with

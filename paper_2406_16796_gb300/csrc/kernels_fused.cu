@@ -883,7 +883,7 @@ cudaError_t step_graph(axp_grid *g, Launch &&launch_one, cudaGraphExec_t *out)
 // FP64 grids of the 2D kernel up to this many cells take the folded passes: a block of
 // the 2D kernel marches at least 14 planes through one SM's FP64 units, which leaves a
 // small grid's step a serial chain.  us per step, passes / 2D kernel: 96 x 64 15 / 47,
-// 400 x 400 44 / 107, 1024 x 512 109 / 142, 800 x 800 131 / 142, 1024 x 768 157 / 142.
+// 400 x 400 42 / 107, 1024 x 512 103 / 142, 800 x 800 126 / 142, 1024 x 768 150 / 142.
 constexpr int64_t kSmallTm = 700000;
 
 // FP32 grids of the 2D kernel up to this many cells take the warp tiles: they split a small

@@ -25,10 +25,10 @@
 // out and the unit is compiled without contraction, for the same reason.
 //
 // Measured on one GB300 (us per step, before: the literal or the generic kernel):
-//   2D TM laser, outflow axion sides, FP64, 1024 x 512       686 -> 120
-//   3D laser, absorbing x sides, FP64, 160 x 96 x 96        1922 -> 535
+//   2D TM laser, outflow axion sides, FP64, 1024 x 512       686 -> 115
+//   3D laser, absorbing x sides, FP64, 160 x 96 x 96        1922 -> 547
 //   2D laser polarised in the plane, FP32 split, 1024 x 512  130 -> 33
-//   2D TM laser, absorbing sides, FP64, 400 x 400            160 -> 44 (the 2D kernel)
+//   2D TM laser, absorbing sides, FP64, 400 x 400            160 -> 42 (the 2D kernel)
 // ncu: the FP64 passes keep the FP64 pipe 76-84% busy while an SM is active.
 #include <algorithm>
 
@@ -216,7 +216,7 @@ __device__ __forceinline__ T ebar(const Stage<T> &s, const T *const E[3], int a,
 {
     if (!(EM >> a & 1)) return s.Eext[a];
     const T f = E[a][q.c];
-    if (!(MASK >> a & 1)) return f + s.Eext[a];
+    if (!(MASK >> a & 1)) return s.uniform_e ? f + s.Eext[a] : f;
     return fma(T(0.5), f + ldz(E[a], q.dn[a], q.hd[a]), s.Eext[a]);
 }
 
@@ -315,7 +315,8 @@ __global__ void __launch_bounds__(kThreads) k_stage_phi(Stage<T> s, const T *bs0
         const T *const Bs[3] = {bs0, bs1, bs2};
         T S = T(0);
 #pragma unroll
-        for (int a = 0; a < 3; a++) S = fma(ebar<MASK, EM>(s, s.Ein, a, q), bbar<MASK, BM>(s, Bs, a, q), S);
+        for (int a = 0; a < 3; a++)
+            if ((EM >> a & 1) || s.uniform_e) S = fma(ebar<MASK, EM>(s, s.Ein, a, q), bbar<MASK, BM>(s, Bs, a, q), S);
         const T ph = s.phi[q.c], old = s.phib[q.c];
         T lap = s.dt2g * S;
 #pragma unroll
@@ -401,8 +402,8 @@ __global__ void __launch_bounds__(kThreads) k_stage_p(Stage<T> s, const T *e0, c
     for (int a = 0; a < 3; a++) {
         const int b = (a + 1) % 3, c = (a + 2) % 3;
         T p = Dt * bbar<MASK, BM>(s, B, a, q);
-        if (MASK >> c & 1) p = fma(-e[b], g[c], p);
-        if (MASK >> b & 1) p = fma(e[c], g[b], p);
+        if ((MASK >> c & 1) && ((EM >> b & 1) || s.uniform_e)) p = fma(-e[b], g[c], p);
+        if ((MASK >> b & 1) && ((EM >> c & 1) || s.uniform_e)) p = fma(e[c], g[b], p);
         s.P[a][q.c] = p;
     }
 }
