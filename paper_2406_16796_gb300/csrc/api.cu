@@ -793,16 +793,14 @@ axp_status axp_read_field(axp_grid *g, int32_t which, double *dst, size_t bytes)
     const axp_status lat = latched_status(g);
     if (lat != AXP_OK) return lat;
     if (!is_fp32(g)) return cuda_status(cudaMemcpy(dst, field_ptr(g, which), bytes, cudaMemcpyDeviceToHost));
-    std::vector<float> tmp(N), inc;
-    e = cudaMemcpy(tmp.data(), field_ptr(g, which == AXP_PHI_OLD ? AXP_PHI_CUR : which), N * 4,
-                   cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && which == AXP_PHI_OLD) {
-        inc.resize(N);
-        e = cudaMemcpy(inc.data(), g->ws + g->layout.off_phi[g->phi_b_slot], N * 4, cudaMemcpyDeviceToHost);
-    }
-    if (e != cudaSuccess) return cuda_status(e);
-    for (int64_t c = 0; c < N; c++) dst[c] = which == AXP_PHI_OLD ? (double)tmp[c] - (double)inc[c] : (double)tmp[c];
-    return AXP_OK;
+    // FP32: widened on the device, into the current's scratch (three float arrays in a row hold
+    // the array as doubles; P is formed anew whenever it is needed)
+    double *wide = (double *)(g->ws + g->layout.off_P[0]);
+    const float *from = (const float *)field_ptr(g, which == AXP_PHI_OLD ? AXP_PHI_CUR : which);
+    const float *less = which == AXP_PHI_OLD ? (const float *)(g->ws + g->layout.off_phi[g->phi_b_slot]) : nullptr;
+    if ((e = widen(from, less, wide, N, g->stream)) == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    if (e == cudaSuccess) e = cudaMemcpy(dst, wide, (size_t)N * 8, cudaMemcpyDeviceToHost);
+    return cuda_status(e);
 }
 
 axp_status axp_write_field(axp_grid *g, int32_t which, const double *src, size_t bytes)

@@ -227,6 +227,8 @@ template <typename T>
 cudaError_t inject_axion(axp_grid *g, const axp_axion_desc &A);
 template <typename T>
 cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled);
+// dst = src (less `less`, where given) in double, n elements
+cudaError_t widen(const float *src, const float *less, double *dst, int64_t n, cudaStream_t stream);
 // macroparticles: workspace size and layout, the deposit of j^n with the move of
 // the positions to t_{n+1/2}, the push between the field half-steps (fields of the
 // view at t_{n+1/2}), and the positions at t_n into the read-back scratch

@@ -512,8 +512,23 @@ __global__ void __launch_bounds__(256) k_batch_diag(Dev D, const int *slots, axp
 constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
+// Read-out of one array of one slot, in pieces of at most kReadCells: gathered into a scratch
+// on the device (where the slot's present buffer is known), copied into pinned memory of the
+// batch and widened from there into the caller's.  One launch, one copy and one
+// synchronisation where there were two copies and two synchronisations.  The caller's pages
+// are touched by the host only: a copy straight into fresh pageable memory takes the GPU's
+// page faults (512 reads of 15.5k cells: 54 ms that way, 16-20 ms before, 12.5-17 ms now).
+constexpr int64_t kReadCells = 1 << 17;
+
+__global__ void __launch_bounds__(256) k_batch_gather(Dev D, int slot, int which, int64_t first, int n, float *dst)
+{
+    const Slot S = D.slots[slot];
+    const float *src = arr(D, S.parity, which, S.off) + first;
+    for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < n; i += (int)(gridDim.x * blockDim.x)) dst[i] = src[i];
+}
+
 struct Layout {
-    size_t pool, slots, items, counter, diag, total;
+    size_t pool, slots, items, counter, diag, read, total;
 };
 
 Layout layout(int32_t max_instances, int64_t max_cells)
@@ -531,6 +546,8 @@ Layout layout(int32_t max_instances, int64_t max_cells)
     off += kAlign;
     L.diag = off;  // one record per slot, then the list of slots asked for
     off += align_up((size_t)max_instances * (sizeof(axp_diag) + sizeof(int)));
+    L.read = off;
+    off += align_up((size_t)std::min(max_cells, kReadCells) * sizeof(float));
     L.total = off;
     return L;
 }
@@ -565,6 +582,7 @@ struct axp_batch {
     bool use_graph;
     cudaGraphExec_t graph;
     int64_t graph_steps;
+    float *host;  // pinned, of the first axp_batch_read_state on
 };
 
 extern "C" {
@@ -609,6 +627,7 @@ axp_status axp_batch_create(int32_t max_instances, int64_t max_cells, void *dev_
     b->use_graph = false;
     b->graph = nullptr;
     b->graph_steps = -1;
+    b->host = nullptr;
     int dev = 0;
     cudaGetDevice(&dev);
     b->sms = 152;
@@ -629,6 +648,7 @@ axp_status axp_batch_destroy(axp_batch *b)
     // the caller frees the workspace after this returns: let queued work finish
     cudaStreamSynchronize(b->stream);
     if (b->graph) cudaGraphExecDestroy(b->graph);
+    if (b->host) cudaFreeHost(b->host);
     delete b;
     return AXP_OK;
 }
@@ -872,16 +892,23 @@ axp_status axp_batch_read_state(axp_batch *b, int32_t slot, int32_t which, doubl
         return AXP_E_INVAL;
     const int64_t nx = b->slots[slot].nx;
     if (bytes != (size_t)nx * sizeof(double)) return AXP_E_INVAL;
-    Slot S;
-    cudaError_t e = cudaMemcpyAsync(&S, b->D.slots + slot, sizeof(Slot), cudaMemcpyDeviceToHost, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return cuda_st(e);
-    std::vector<float> tmp(nx);
-    const float *src = b->D.pool + ((int64_t)(S.parity * kArr + which) * b->max_cells + S.off);
-    e = cudaMemcpyAsync(tmp.data(), src, nx * sizeof(float), cudaMemcpyDeviceToHost, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return cuda_st(e);
-    for (int64_t i = 0; i < nx; i++) host_dst[i] = tmp[i];
+    float *scratch = (float *)(b->ws + b->L.read);
+    const int64_t piece = std::min(b->max_cells, kReadCells);
+    cudaError_t e = cudaSuccess;
+    if (!b->host && (e = cudaMallocHost((void **)&b->host, (size_t)piece * sizeof(float))) != cudaSuccess) {
+        b->host = nullptr;
+        return cuda_st(e);
+    }
+    for (int64_t c = 0; c < nx; c += piece) {
+        const int n = (int)std::min(piece, nx - c);
+        k_batch_gather<<<std::min((n + 255) / 256, 152 * 8), 256, 0, b->stream>>>(b->D, slot, which, c, n, scratch);
+        e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(b->host, scratch, (size_t)n * sizeof(float), cudaMemcpyDeviceToHost, b->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+        if (e != cudaSuccess) return cuda_st(e);
+        for (int i = 0; i < n; i++) host_dst[c + i] = b->host[i];
+    }
     return AXP_OK;
 }
 
