@@ -331,12 +331,13 @@ cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
     const double dx = d.d[0], dt = d.dt;
     A.cB = (T)(dt / 2.0 / dx);
     A.c2B = (T)(dt / dx);
-    A.h2g = (T)(dt * d.g);
+    A.h2g = (T)(sizeof(T) == 8 ? d.g : dt * d.g);  // (of dt P; P)
+    A.hgx = (T)(0.5 * d.g);
     A.lap_0 = (T)(sizeof(T) == 8 ? 2.0 - dt * dt * (d.m * d.m + 2.0 / (dx * dx)) : -dt * dt * d.m * d.m);
     A.lap_c = (T)(dt * dt / (dx * dx));
     A.dt2g = (T)(dt * dt * d.g);
     A.inv_dt = (T)(1.0 / dt);
-    A.q4dx = (T)(1.0 / (4.0 * dx));
+    A.q4dx = (T)(dt / (4.0 * dx));
     for (int a = 0; a < 3; a++) A.Bext[a] = (T)g->B_ext[a];
     const Workspace &w = g->layout;
     for (int s = 0; s < 2; s++)

@@ -37,8 +37,10 @@
 // so its windows are blocked over more steps (line_block).
 //
 // Measured, us per step (one launch per step before): 2048 cells with absorbing ends
-// FP32 5.2 -> 1.3, FP64 16.8 -> 2.8; 4096 periodic FP32 2.9 -> 0.63;
-// 65536 with absorbing ends FP32 7.0 -> 3.2, FP64 36 -> 11.5; 4096 periodic FP64 1.8 before and now.
+// FP32 5.2 -> 1.3, FP64 16.8 -> 2.7; 4096 periodic FP32 2.9 -> 0.63;
+// 65536 with absorbing ends FP32 7.0 -> 3.2, FP64 36 -> 11.0.  Periodic FP64 (blocked before too):
+// 4096 cells 1.80 -> 1.71, 65536 10.9 -> 10.4 with three of 29 FP64 operations of the longer
+// half taken out of a step (an FP64 instruction takes a warp 64 to 76 cycles, whatever its lanes).
 #pragma once
 
 #include "kernels_fused.cuh"
@@ -74,11 +76,12 @@ struct Args {
     // step constants
     T cB;           // h/dx: one B or E0 half-step per difference
     T c2B;          // 2h/dx: the two half-steps of E1 (and of B1) per difference
-    T h2g;          // 2hg: the current's term in E1's two half-steps
+    T h2g;          // 2hg (FP64: 2hg/dt): the current's term in E1's two half-steps
+    T hgx;          // FP64: half of it, for the face sum of P_x
     // FP64: phi^{n+3/2} = lap_0 phi + lap_c (phi+ + phi-) - phi^{n-1/2} + dt2g S/g;
     // FP32: the increment grows by lap_0 phi + lap_c (second difference) + dt2g S/g
     T lap_0, lap_c, dt2g;
-    T inv_dt, q4dx;        // 1/dt; 1/(4 dx) for the central gradient of 2 phi^{n+1}
+    T inv_dt, q4dx;        // 1/dt; dt/(4 dx) for dt times the central gradient of 2 phi^{n+1}
     T Bext[3];
     // absorbing layers: their cells at either end, the coefficient tables of the grid
     // (a, b, a^2, b (1 + a), c1, c2: n each), sigma of the axion, 1/h, 1/dt^2, dt
@@ -142,7 +145,8 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
     // y z, E0^{n+1} y z, 2 phi^{n+1}, dt D_t phi^{n+1}, P (3), Bbar0^{n+1} y z (with B_ext),
     // two values that stay fixed over a window's steps (E0x and B0x do not change in 1D, no
     // curl along x: Bbar0_x = B0x + B_ext,x and the source's term Ebar0_x Bbar0_x), and
-    // FP32's increment
+    // FP32's increment (FP64: phi+ + phi- for the next step).  FP64 holds dt P: D_t phi and the
+    // gradient then take no product of their own
     auto arr = [&](int q) { return l1_sm + (size_t)q * Wm; };
     T *E[6], *B[6];
     for (int q = 0; q < 6; q++) {
@@ -151,7 +155,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
     }
     T *cur = arr(12), *old = arr(13), *Bhy = arr(14), *Bhz = arr(15), *Eny = arr(16), *Enz = arr(17);
     T *SM = arr(18), *DF = arr(19), *Px = arr(20), *PY = arr(21), *PZ = arr(22), *BY = arr(23), *BZ = arr(24);
-    T *BXT = arr(25), *SX = arr(26), *inc = INCR ? arr(27) : arr(13);
+    T *BXT = arr(25), *SX = arr(26), *inc = INCR ? arr(27) : arr(13), *SP = arr(27);
     // the layer's a, r = b/h, and for the axion 1/(1 + sigma dt), (1 - sigma dt)/(1 + sigma dt), (sigma dt)^2
     T *La = arr(28), *Lr = arr(29), *Lc1 = arr(30), *Lc2 = arr(31), *Lss = arr(32);
     // FP32: La 1 - sigma h/2 (-1 beyond the grid), Ld and Lr the divisor 1 + sigma h/2 and its
@@ -217,6 +221,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             const T bx = B[0][w] + Bx;
             BXT[w] = bx;
             SX[w] = ex * bx;
+            if (!INCR) SP[w] = at(cur, w + 1) + at(cur, w - 1);
         }
         __syncthreads();
         for (int st = 0; st < (INCR ? 0 : steps); st++) {
@@ -265,12 +270,12 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
                         T nw;
                         if (in_layer(w)) {
                             nw = A.lap_0 * ph;
-                            nw = fma(A.lap_c, at(cur, w + 1) + at(cur, w - 1), nw);
+                            nw = fma(A.lap_c, SP[w], nw);
                             nw = fma(A.dt2g, S, nw);
                             nw = fma(-Lc2[w], old[w], Lc1[w] * fma(-Lss[w], ph, nw));
                         } else {
                             nw = fma(A.lap_0, ph, -old[w]);
-                            nw = fma(A.lap_c, at(cur, w + 1) + at(cur, w - 1), nw);
+                            nw = fma(A.lap_c, SP[w], nw);
                             nw = fma(A.dt2g, S, nw);
                         }
                         old[w] = nw;  // phi^{n+3/2} over phi^{n-1/2} (read by this cell only)
@@ -292,12 +297,13 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
                 }
             }
             __syncthreads();
-            // 3. P^{n+1} at the cell centres
+            // 3. dt P^{n+1} at the cell centres
             for (int w = lane; w < W; w += LANES) {
-                const T Dt = DF[w] * A.inv_dt;
+                const T Dt = DF[w];
                 const T dphi = (at(SM, w + 1) - at(SM, w - 1)) * A.q4dx;
                 if (half == 0) {
                     PY[w] = fma(-Enz[w], dphi, Dt * BY[w]);
+                    SP[w] = at(old, w + 1) + at(old, w - 1);  // of phi^{n+3/2}
                 } else {
                     Px[w] = Dt * BXT[w];
                     PZ[w] = fma(Eny[w], dphi, Dt * BZ[w]);
@@ -307,15 +313,15 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             // 4. J^{n+1}; E1^{n+3/2}; E0^{n+3/2}
             for (int w = lane; w < W; w += LANES) {
                 if (half == 0) {
-                    const T Jx = T(0.5) * (Px[w] + at(Px, w + 1)), dz = B[5][w] - at(B[5], w - 1);
+                    const T Jx = Px[w] + at(Px, w + 1), dz = B[5][w] - at(B[5], w - 1);
                     if (in_layer(w)) {
                         // two half-steps: a^2 E + (1 + a) r h X
                         const T a = La[w], r2 = T(0.5) * Lr[w];
-                        const T xx = r2 * (-A.h2g * Jx), xy = r2 * fma(-A.c2B, dz, -A.h2g * PY[w]);
+                        const T xx = r2 * (-A.hgx * Jx), xy = r2 * fma(-A.c2B, dz, -A.h2g * PY[w]);
                         E[3][w] = fma(a, fma(a, E[3][w], xx), xx);
                         E[4][w] = fma(a, fma(a, E[4][w], xy), xy);
                     } else {
-                        E[3][w] = fma(-A.h2g, Jx, E[3][w]);
+                        E[3][w] = fma(-A.hgx, Jx, E[3][w]);
                         E[4][w] = fma(-A.c2B, dz, fma(-A.h2g, PY[w], E[4][w]));
                     }
                 } else {
