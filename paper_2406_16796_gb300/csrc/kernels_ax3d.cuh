@@ -224,17 +224,26 @@ __global__ void __launch_bounds__(Geo<T>::NT, 1) k_ax3d(fused::Params<T> P)
 // come from its own other cell and, across pairs, by 16-lane shuffles.  The
 // pair starts at an even x (written columns per tile: 28), so with an even nx
 // every pair lies inside the grid and is 8-byte aligned.
+//
+// The kernel is bound by latency with 16 warps an SM, and by what L1 has left beside the shared
+// memory: the y neighbours of E_x, E_z and phi are therefore read where plane t - 1 was staged,
+// and only B^{n+1}_x, _z and D_t phi are published (190 -> 160 KB, 106 -> 98 registers; three
+// stores fewer a plane).  512^3 1745 -> 1603 us per step, 256^3 232 -> 209.  Tried and slower at
+// 512^3: five staged planes 1788, three 1959; 40 rows 1808 to 2474, 48 rows 1910, 28 rows 1620;
+// 16-byte copies past L1 1852.
 namespace x2 {
 constexpr int TXP = 16;             // pairs per tile row (threads along x)
 constexpr int TY = 32;              // tile rows (threads along y)
 constexpr int NT = TXP * TY;        // 512 threads
+constexpr int NSP = 4;              // staged planes: t - 1, t and two in flight
 constexpr int HLX = 2, HRX = 2;     // halo columns along x (even: pairs stay aligned)
 constexpr int VXC = 2 * TXP - HLX - HRX;  // written columns per tile: 28
 constexpr int VYR = TY - HL - HR;   // written rows per tile: 29
 constexpr int PXP = TXP + 2;        // published row, in pairs, with a guard pair each side
 constexpr int PYR = TY + 2;
 constexpr int PLANE = PXP * PYR;
-constexpr size_t smem_bytes() { return ((size_t)2 * NPUB * PLANE + (size_t)NS * NIN * NT) * sizeof(float2); }
+enum { Q_NX, Q_NZ, Q_DT, NQ };      // published values
+constexpr size_t smem_bytes() { return ((size_t)2 * NQ * PLANE + (size_t)NSP * NIN * NT) * sizeof(float2); }
 
 __device__ __forceinline__ float2 f2(float s) { return make_float2(s, s); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -256,10 +265,10 @@ __global__ void __launch_bounds__(x2::NT, 1) k_ax3d_x2(fused::Params<T> P)
     using namespace x2;
     constexpr int PL = x2::PLANE;
     extern __shared__ __align__(16) unsigned char ax3d_x2_dyn[];
-    float2 *pub = reinterpret_cast<float2 *>(ax3d_x2_dyn);  // [2][NPUB][PYR][PXP]
-    float2 *stage = pub + 2 * NPUB * PL;                     // [NS][NIN][NT]
+    float2 *pub = reinterpret_cast<float2 *>(ax3d_x2_dyn);  // [2][NQ][PYR][PXP]
+    float2 *stage = pub + 2 * NQ * PL;                       // [NSP][NIN][NT]
     const int tid = threadIdx.x, tx = tid % TXP, ty = tid / TXP;
-    for (int i = tid; i < 2 * NPUB * PL; i += NT) pub[i] = make_float2(0.f, 0.f);
+    for (int i = tid; i < 2 * NQ * PL; i += NT) pub[i] = make_float2(0.f, 0.f);
 
     const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
     const int gx = (int)blockIdx.x * VXC - HLX + 2 * tx, gy = (int)blockIdx.y * VYR - HL + ty;
@@ -279,18 +288,18 @@ __global__ void __launch_bounds__(x2::NT, 1) k_ax3d_x2(fused::Params<T> P)
 
     const float2 z = make_float2(0.f, 0.f);
     float2 Ex0 = z, Ex1 = z, Ex2 = z, Ey0 = z, Ey1 = z, Ey2 = z, Ez0 = z, Ez1 = z, Ez2 = z;
-    float2 Bx0 = z, Bx1 = z, By0 = z, By1 = z, Bz0 = z, Bz1 = z;
     float2 Nx1 = z, Nx2 = z, Nx3 = z, Ny1 = z, Ny2 = z, Ny3 = z, Nz1 = z, Nz2 = z;
-    float2 ph0 = z, ph1 = z, ph2 = z, pb0 = z, pb1 = z;
+    float2 ph0 = z, ph1 = z, ph2 = z;
     float2 D1 = z, D2 = z;
 
     auto gidx = [&](int p) -> int64_t {
         const int wp = p < 0 ? p + nz : (p >= nz ? p - nz : p);
         return col + plane_stride * (int64_t)wp;
     };
+    auto slot = [&](int p) { return stage + ((p - t0) & (NSP - 1)) * (NIN * NT) + tid; };
     auto prefetch = [&](int p) {
         const int64_t o = gidx(p);
-        float2 *st = stage + ((p - t0) & (NS - 1)) * (NIN * NT) + tid;
+        float2 *st = slot(p);
         cp_pair(st + 0 * NT, P.Ein[3] + o);
         cp_pair(st + 1 * NT, P.Ein[4] + o);
         cp_pair(st + 2 * NT, P.Ein[5] + o);
@@ -299,17 +308,6 @@ __global__ void __launch_bounds__(x2::NT, 1) k_ax3d_x2(fused::Params<T> P)
         cp_pair(st + 5 * NT, P.Bin[5] + o);
         cp_pair(st + 6 * NT, P.phi + o);
         cp_pair(st + 7 * NT, P.phib + o);
-    };
-    auto take = [&](int p) {
-        const float2 *st = stage + ((p - t0) & (NS - 1)) * (NIN * NT) + tid;
-        Ex0 = st[0 * NT];
-        Ey0 = st[1 * NT];
-        Ez0 = st[2 * NT];
-        Bx0 = st[3 * NT];
-        By0 = st[4 * NT];
-        Bz0 = st[5 * NT];
-        ph0 = st[6 * NT];
-        pb0 = st[7 * NT];
     };
     // the new state is read again only in the next step, after the whole box has
     // streamed through L2: stores are marked evict-first
@@ -320,35 +318,40 @@ __global__ void __launch_bounds__(x2::NT, 1) k_ax3d_x2(fused::Params<T> P)
     auto xp = [&](float2 v) { return make_float2(v.y, __shfl_down_sync(all, v.x, 1, TXP)); };
     auto xm = [&](float2 v) { return make_float2(__shfl_up_sync(all, v.y, 1, TXP), v.x); };
 
-    for (int j = 0; j < NS - 1; j++) {
+    for (int j = 0; j < NSP - 2; j++) {
         if (t0 + j <= t1) prefetch(t0 + j);
         tm2d::cp_commit();
     }
-    tm2d::cp_wait<NS - 2>();
-    take(t0);
+    tm2d::cp_wait<NSP - 3>();
     __syncthreads();
     for (int t = t0; t <= t1; ++t) {
-        if (t + NS - 1 <= t1) prefetch(t + NS - 1);
-        tm2d::cp_commit();
-        float2 *Q = pub + (t & 1) * (NPUB * PL);
-        Q[P_EX * PL + me] = Ex1;
-        Q[P_EZ * PL + me] = Ez1;
-        Q[P_PHI * PL + me] = ph1;
-        Q[P_NX * PL + me] = Nx2;
-        Q[P_NZ * PL + me] = Nz2;
-        Q[P_DT * PL + me] = D2;
+        const float2 *C = slot(t), *L = slot(t - 1);
+        Ex0 = C[0 * NT];
+        Ey0 = C[1 * NT];
+        Ez0 = C[2 * NT];
+        ph0 = C[6 * NT];
+        float2 *Q = pub + (t & 1) * (NQ * PL);
+        Q[Q_NX * PL + me] = Nx2;
+        Q[Q_NZ * PL + me] = Nz2;
+        Q[Q_DT * PL + me] = D2;
         const float2 Ez_xp = xp(Ez1), Ey_xp = xp(Ey1), ph_xp = xp(ph1), ph_xm = xm(ph1), D_xp = xp(D2);
         const float2 Nz_xm = xm(Nz2), Ny_xm = xm(Ny2);
         __syncthreads();
-        const float2 *qEx = Q + P_EX * PL + me, *qEz = Q + P_EZ * PL + me;
-        const float2 *qph = Q + P_PHI * PL + me, *qNx = Q + P_NX * PL + me;
-        const float2 *qNz = Q + P_NZ * PL + me, *qDt = Q + P_DT * PL + me;
+        // into the slot of plane t - 2, which all have read by the barrier
+        if (t + NSP - 2 <= t1) prefetch(t + NSP - 2);
+        tm2d::cp_commit();
+        // Plane t - 1 as its threads staged it.  Beyond the tile's first and last rows, and before
+        // plane t0, these read other or unset values of the stage: what comes of them stays in
+        // the halo, which is not written.
+        const float2 *qEx = L, *qEz = L + 2 * NT, *qph = L + 6 * NT;
+        const float2 *qNx = Q + Q_NX * PL + me, *qNz = Q + Q_NZ * PL + me, *qDt = Q + Q_DT * PL + me;
+        const float2 Bx1 = L[3 * NT], By1 = L[4 * NT], Bz1 = L[5 * NT], pb1 = L[7 * NT];
         // ---- stage 1: B^{n+1} on plane t-1 ----
         {
             const int p = t - 1;
-            Nx1 = fma2(mh2y, sub2(qEz[PXP], Ez1), fma2(h2z, sub2(Ey0, Ey1), Bx1));
+            Nx1 = fma2(mh2y, sub2(qEz[TXP], Ez1), fma2(h2z, sub2(Ey0, Ey1), Bx1));
             Ny1 = fma2(mh2z, sub2(Ex0, Ex1), fma2(h2x, sub2(Ez_xp, Ez1), By1));
-            Nz1 = fma2(mh2x, sub2(Ey_xp, Ey1), fma2(h2y, sub2(qEx[PXP], Ex1), Bz1));
+            Nz1 = fma2(mh2x, sub2(Ey_xp, Ey1), fma2(h2y, sub2(qEx[TXP], Ex1), Bz1));
             if (write_col && p >= m0 && p < m1) {
                 const int64_t gi = col + plane_stride * (int64_t)p;
                 store(P.Bout[3], gi, Nx1);
@@ -360,7 +363,7 @@ __global__ void __launch_bounds__(x2::NT, 1) k_ax3d_x2(fused::Params<T> P)
         {
             const int p = t - 1;
             const float2 spx = add2(sub2(ph_xp, ph1), sub2(ph_xm, ph1));
-            const float2 spy = add2(sub2(qph[PXP], ph1), sub2(qph[-PXP], ph1));
+            const float2 spy = add2(sub2(qph[TXP], ph1), sub2(qph[-TXP], ph1));
             const float2 spz = add2(sub2(ph0, ph1), sub2(ph2, ph1));
             float2 acc = fma2(c0, ph1, pb1);
             acc = fma2(cx, spx, acc);
@@ -385,12 +388,10 @@ __global__ void __launch_bounds__(x2::NT, 1) k_ax3d_x2(fused::Params<T> P)
             }
         }
         Ex2 = Ex1; Ex1 = Ex0; Ey2 = Ey1; Ey1 = Ey0; Ez2 = Ez1; Ez1 = Ez0;
-        Bx1 = Bx0; By1 = By0; Bz1 = Bz0;
         Nx3 = Nx2; Nx2 = Nx1; Ny3 = Ny2; Ny2 = Ny1; Nz2 = Nz1;
-        ph2 = ph1; ph1 = ph0; pb1 = pb0;
+        ph2 = ph1; ph1 = ph0;
         D2 = D1;
-        tm2d::cp_wait<NS - 2>();
-        if (t < t1) take(t + 1);
+        tm2d::cp_wait<NSP - 3>();  // plane t + 1
     }
     tm2d::cp_wait<0>();
 }
