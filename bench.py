@@ -488,8 +488,8 @@ def group_measurement(members, steps, hbm_peak, hbm_src):
 BYTES_PER_PARTICLE = (13 + 12) * 8
 # k_particles_push on the magnetised plasma (4.8M particles, 2D), one-pass ncu
 # capture of one launch: FP64-pipe warp instructions and DRAM bytes
-PUSH_FP64_WARP_INST_PER_PARTICLE = 110118800 / 4800000
-PUSH_TRAFFIC_PER_PARTICLE = (843438848 + 531257856) / 4800000
+PUSH_FP64_WARP_INST_PER_PARTICLE = 80738912 / 4800000
+PUSH_TRAFFIC_PER_PARTICLE = (757643008 + 449397248) / 4800000
 
 
 def plasma_oracle_rate(nx=1200, steps=2):
@@ -516,7 +516,7 @@ def plasma_oracle_rate(nx=1200, steps=2):
 def plasma_measurement(steps, warmup, hbm_peak, hbm_src, world, cpu=False):
     """Weak laser in a magnetised plasma (perturbed-particle current): 12000 x
     100 cells, 4 electrons per cell (4.8M), the laser in the first-order fields;
-    FP64, one grid per GPU.  Each step is the general field kernels plus one
+    FP64, one grid per GPU.  Each step is the folded field passes plus one
     particle push that gathers, kicks, drifts and deposits both orders."""
     import torch
 
@@ -541,7 +541,7 @@ def plasma_measurement(steps, warmup, hbm_peak, hbm_src, world, cpu=False):
            "particles": plasma.count, "precision": "fp64", "steps": steps, "ms_per_step": per * 1e3,
            "value": plasma.count * steps * world / el, "unit": "particle-steps/s",
            "cell_updates_per_s": grid.cells * steps * world / el, "gpu_launches": launches,
-           "kernel": "k_particles_push and the general field kernels",
+           "kernel": "k_particles_push and the folded field passes",
            "roofline": {"bound": "alu", "achieved": fp64_ach, "peak": fp64_peak, "unit": "Gop/s (FP64 pipe)",
                         "frac": fp64_ach / fp64_peak, "kernel": "k_particles_push",
                         "executed_fp64_ops_per_particle": PUSH_FP64_WARP_INST_PER_PARTICLE * 32,
@@ -746,7 +746,7 @@ def gpu_arm(args):
     el = max_over_ranks(el, world)
     value = cells * args.steps * world / el
     ms = el / args.steps * 1e3
-    per_launch = el / max(1, launches)  # the fused path launches one kernel per step
+    per_launch = el / args.steps  # (one launch a step, or the folded passes of one)
 
     peaks = load_peaks()
     hbm_peak = peaks.get("hbm_gbs", 6800.0)
@@ -756,8 +756,9 @@ def gpu_arm(args):
     hbm = {"achieved": hbm_achieved, "peak": hbm_peak, "unit": "GB/s", "frac": hbm_achieved / hbm_peak,
            "peak_source": hbm_src, "algorithmic_bytes_per_cell": bpc}
     kern = {axp.AXP_KERNEL_TM2D: "k_tm2d (one launch per step)",
-            axp.AXP_KERNEL_TM2D_LIST: "k_tm2d_list (one launch per step)",
-            axp.AXP_KERNEL_FUSED: "k_fused (one launch per step)"}.get(path, "general kernels (8 launches per step)")
+            axp.AXP_KERNEL_TM2D_LIST: "k_tm2d_list (one launch per step)"}.get(path)
+    if kern is None or launches > args.steps:  # (small FP64 grids of the 2D kernel's path too)
+        kern = "folded passes (4 launches per step)"
     if prec == "fp64":
         sm_count = torch.cuda.get_device_properties(local).multi_processor_count
         sm_mhz = clk.get("sm_mhz") or peaks.get("sm_max_mhz", 2070.0)
@@ -833,15 +834,14 @@ def gpu_arm(args):
         for L in w32.lasers:
             g32.inject_laser(L)
         k32 = 4 * args.steps
-        el32, l32 = timed_run(g32, k32, args.warmup, g32.stream)
-        per32 = el32 / max(1, l32)
+        el32, _ = timed_run(g32, k32, args.warmup, g32.stream)
+        per32 = el32 / k32
         ach = bytes_per_cell("fp32") * cells / per32 / 1e9
         # FP32 split on an even-width grid takes the two-column form of the 2D kernel
         path32 = g32.kernel_path()
         kern32 = ("k_tm2d_x2 (one launch per step)" if (path32 == axp.AXP_KERNEL_TM2D and args.nx % 2 == 0)
                   else "k_tm2d (one launch per step)" if path32 == axp.AXP_KERNEL_TM2D
-                  else "k_fused (one launch per step)" if path32 == axp.AXP_KERNEL_FUSED
-                  else "general kernels (8 launches per step)")
+                  else "folded passes (4 launches per step)")
         other = {"precision": "fp32_split", "value": cells * k32 * world / el32, "unit": "cell-updates/s",
                  "steps": k32, "ms_per_step": el32 / k32 * 1e3, "kernel": kern32,
                  "roofline": {"bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s",
