@@ -441,8 +441,8 @@ def fp64_sequential_sample(reqs, served, sample=8, seed=20240628):
 
 
 # k_tm2d_group on the first 40 2D requests of the seeded stream (21,932,100 cells),
-# one-pass ncu capture of one launch: 1054.2 + 919.8 MB
-TRAFFIC_GROUP40 = 1974.2e6
+# one-pass ncu capture of one launch: 1015.0 + 918.3 MB
+TRAFFIC_GROUP40 = 1933.3e6
 
 
 def group_measurement(members, steps, hbm_peak, hbm_src):
