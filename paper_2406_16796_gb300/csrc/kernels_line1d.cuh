@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
     T *BXT = arr(25), *SX = arr(26), *inc = INCR ? arr(27) : arr(13), *SP = arr(27);
     // the layer's a, r = b/h, and for the axion 1/(1 + sigma dt), (1 - sigma dt)/(1 + sigma dt), (sigma dt)^2
     T *La = arr(28), *Lr = arr(29), *Lc1 = arr(30), *Lc2 = arr(31), *Lss = arr(32);
-    // FP32: La 1 - sigma h/2 (-1 beyond the grid), Ld and Lr the divisor 1 + sigma h/2 and its
-    // reciprocal; for the axion Lc2 1 - sigma dt, Le and Lc1 the divisor 1 + sigma dt and its
+    // FP32: La 1 - sigma h/2 (of either sign: sigma h may exceed 2), Ld and Lr the divisor
+    // 1 + sigma h/2 and its reciprocal (0 beyond the grid, which marks those cells); for the axion Lc2 1 - sigma dt, Le and Lc1 the divisor 1 + sigma dt and its
     // reciprocal, Lss sigma^2
     T *Ld = arr(33), *Le = arr(34);
     const int half = tid / LANES, lane = tid % LANES;  // (a warp-uniform half)
@@ -176,9 +176,9 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             const bool in = gi >= 0 && gi < N;
             if (INCR) {
                 const T se = in ? A.sig_em[gi] : T(0), sa = in ? A.sig[gi] : T(0);
-                La[w] = in ? T(1) - se * A.h / T(2) : T(-1);
-                Ld[w] = T(1) + se * A.h / T(2);
-                Lr[w] = T(1) / Ld[w];
+                La[w] = T(1) - se * A.h / T(2);
+                Ld[w] = in ? T(1) + se * A.h / T(2) : T(0);
+                Lr[w] = in ? T(1) / Ld[w] : T(0);
                 Lc2[w] = T(1) - sa * A.dt;
                 Le[w] = T(1) + sa * A.dt;
                 Lc1[w] = T(1) / Le[w];
@@ -348,6 +348,8 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
         // from the correctly rounded reciprocal r of d (Markstein's theorem: q = x r, then
         // q + (x - q d) r): the plain division of every damped cell and stage doubled the step
         // of a grid with absorbing ends (2.2 us against 1.3).
+        // Below about 1e-30 the residual underflows and the quotient's last bit may differ: dividing
+        // there costs 9% of a pulse's whole call, whose far tails are that small.
         auto over = [](T x, T d, T r) {
             const T q = x * r;
             return fma(fma(-q, d, x), r, q);
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
         for (int st = 0; st < (INCR ? steps : 0); st++) {
             for (int w = lane; w < W; w += LANES) {
                 bool lay = in_layer(w);
-                if (lay && La[w] < T(0)) continue;
+                if (lay && Ld[w] == T(0)) continue;
                 lay = lay && Ld[w] != T(1);
                 if (half == 0) {
                     const T c0 = -((at(E[2], w + 1) - E[2][w]) * A.idx), c1 = -((at(E[5], w + 1) - E[5][w]) * A.idx);
@@ -382,7 +384,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             __syncthreads();
             for (int w = lane; w < W; w += LANES) {
                 bool lay = in_layer(w);
-                const bool dead = lay && La[w] < T(0);
+                const bool dead = lay && Ld[w] == T(0);
                 if (half == 0) {
                     if (dead) continue;
                     const T by = fma(T(0.5), Bhy[w] + at(Bhy, w - 1), By);
@@ -423,7 +425,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             __syncthreads();
             for (int w = lane; w < W; w += LANES) {
                 bool lay = in_layer(w);
-                if (lay && La[w] < T(0)) continue;
+                if (lay && Ld[w] == T(0)) continue;
                 lay = lay && Ld[w] != T(1);
                 if (half == 0) {
                     const T X = -A.g * (T(0.5) * (Px[w] + at(Px, w + 1)));
