@@ -359,7 +359,10 @@ axp_status axp_load_state(axp_grid *grid, const void *host_src, size_t bytes);
  * allocate nothing; bytes must equal axp_rows_bytes(nrows).  The state's
  * representation (integer time, or the staggered state of the single-pass
  * kernels) must be the same on both sides: slabs that exchange rows take the
- * same kernel path and the same steps.  AXP_E_INVAL for rows outside the
+ * same kernel path and the same steps.  Rows may bring order-0 components that
+ * were never injected or written here: records, conversions and the multi-pass
+ * step then take all of them; a single-pass kernel takes those of the set it
+ * was chosen for (the 2D TM kernel: E0z, B0x, B0y).  AXP_E_INVAL for rows outside the
  * grid; AXP_E_STATE for a grid with macroparticles (they do not move between
  * slabs).
  *

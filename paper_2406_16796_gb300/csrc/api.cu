@@ -621,7 +621,8 @@ static axp_status run_steps(axp_grid *g, int64_t nsteps)
         // AUTO: the folded multi-pass kernels; forced GENERAL: the literal ones.  (An
         // attached but empty particle set keeps the literal kernels' bits.)
         const bool staged = g->kernel_choice == AXP_KERNEL_AUTO && staged_supported(g) && !(g->parts && g->parts->count == 0);
-        if (e == cudaSuccess && staged) e = is_fp32(g) ? staged_step<float>(g, nsteps) : staged_step<double>(g, nsteps);
+        const uint32_t m = order0_present(g);
+        if (e == cudaSuccess && staged) e = is_fp32(g) ? staged_step<float>(g, nsteps, m) : staged_step<double>(g, nsteps, m);
         else if (e == cudaSuccess) e = is_fp32(g) ? general_step<float>(g, nsteps) : general_step<double>(g, nsteps);
     } else {
         e = cudaSuccess;
@@ -1134,6 +1135,7 @@ axp_status axp_load_state(axp_grid *g, const void *src, size_t bytes)
     }
     g->step = h.step;
     g->J_valid = false;  // recomputed from the loaded state when a step needs it
+    g->rows_in = false;
     g->phi_active = h.phi_active != 0;
     g->win_axis = h.win_axis;
     g->win_cells = h.win_cells;
@@ -1212,6 +1214,7 @@ static axp_status rows_copy(axp_grid *g, int64_t row0, int64_t nrows, char *dev,
                  : cudaMemcpyAsync(arr[q] + off, dev + q * chunk, chunk, cudaMemcpyDeviceToDevice, g->stream);
     if (!pack) {
         g->J_valid = false;
+        g->rows_in = true;
         g->cfg_version++;
     }
     return cuda_status(e);

@@ -147,6 +147,9 @@ struct axp_grid {
     int64_t launches;
     uint32_t active;       // bit per field array that may be non-zero
     bool phi_active;
+    // rows of another grid arrived (axp_unpack_rows): order-0 components that were never
+    // injected or written here may be non-zero
+    bool rows_in;
     void *group;           // the axp_group stepping this grid, or null
     // CUDA graphs of consecutive fused 1D steps, one per buffer-role configuration;
     // cfg_version changes whenever fields, background or kernel choice change
@@ -207,8 +210,9 @@ View<T> make_view_eset(axp_grid *g, int eset);
 template <typename T>
 cudaError_t general_step(axp_grid *g, int64_t nsteps);
 // the folded multi-pass step on the state as it stands (integer time or staggered)
+// (order0: mask of the order-0 components it computes)
 template <typename T>
-cudaError_t staged_step(axp_grid *g, int64_t nsteps);
+cudaError_t staged_step(axp_grid *g, int64_t nsteps, uint32_t order0);
 bool staged_supported(const axp_grid *g);
 // E^n -> E^{n+1/2} in place, and E^{n+1/2} -> E^n into field set oset, by the same passes
 template <typename T>
@@ -251,6 +255,10 @@ template <typename T>
 cudaError_t exit_staggered(axp_grid *g, bool in_place);
 // mask of E0/B0 components that can become non-zero (bits 0-2 E0xyz, 3-5 B0xyz)
 uint32_t order0_closure(const axp_grid *g);
+// the components that may hold data: all of them once rows of another grid have arrived.
+// Records, conversions and the multi-pass step go by this; a single-pass kernel computes
+// the components of its own set (chosen by the closure) whatever the rows hold.
+inline uint32_t order0_present(const axp_grid *g) { return g->rows_in ? 63u : order0_closure(g); }
 cudaError_t ensure_integer(axp_grid *g);
 // buffer roles after one more fused step (field sets and axion slots alternate)
 void rotate_roles(axp_grid *g);

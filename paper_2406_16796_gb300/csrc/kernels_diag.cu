@@ -603,11 +603,10 @@ cudaError_t e_level_from_halves(axp_grid *g, const Sums<T> &s, uint32_t mask)
     const int oset = 1 - g->fset;
     const int fe[6] = {kE0, kE0 + 1, kE0 + 2, kE1, kE1 + 1, kE1 + 2};
     L.mask = 0;
-    const uint32_t closure = order0_closure(g);  // the components a step moves, injected or driven
     for (int f = 0; f < 6; f++) {
         L.lo[f] = (T *)(g->ws + w.off_fields[oset][fe[f]]);
         L.hi[f] = (const T *)(g->ws + w.off_fields[g->fset][fe[f]]);
-        if (f >= 3 || (closure >> f & 1u)) L.mask |= 1u << f;
+        if (f >= 3 || (mask >> f & 1u)) L.mask |= 1u << f;  // (injected, driven or from another grid's rows)
     }
     for (int a = 0; a < 3; a++) {
         const bool lay = g->desc.em_bc[a][0] != AXP_BC_PERIODIC && g->desc.pml_cells > 0 && g->desc.pml_sigma_max_dt > 0;
@@ -640,7 +639,7 @@ cudaError_t diag_compute_rows(axp_grid *g, axp_diag *dev_dst, int axis, int64_t 
     // the time-blocked 1D kernel leaves E^n in the current's scratch (J: E0y, E0z, E1x; P: E1y, E1z)
     const bool scratch = g->staggered && g->en_scratch && g->en_scratch_cfg == g->cfg_version;
     const bool wide = (int64_t)g->desc.n[0] * g->desc.n[1] * g->desc.n[2] >= (int64_t)1 << 30;  // (64-bit indexes)
-    const uint32_t mask = order0_closure(g);
+    const uint32_t mask = order0_present(g);
     if (g->staggered && !halves && !scratch) {
         const cudaError_t e = exit_staggered<T>(g, false);
         if (e != cudaSuccess) return e;

@@ -949,8 +949,10 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     // place of the generic kernel in 2D and 3D, and on small FP64 grids of the 2D kernel
     const bool small_tm = tm && sizeof(T) == 8 && g->desc.n[0] * g->desc.n[1] <= kSmallTm;
     g->en_scratch = false;
+    // (after rows of another grid have arrived, the whole set of the kernel they stand for:
+    // a slab without a laser takes its neighbour's)
     if (g->kernel_choice == AXP_KERNEL_AUTO && (small_tm || (path == AXP_KERNEL_FUSED && mode >= 2)) && staged_supported(g))
-        return staged_step<T>(g, nsteps);
+        return staged_step<T>(g, nsteps, small_tm && g->rows_in ? kSets[1] : order0_present(g));
     int tm_tx = tm2d::TX;  // tile width of the 2D kernel (chosen below)
     // FP32 split on an even-width grid without a soft source: the two-column form
     const bool x2 = tm && tm2d_x2_eligible<T>(g);

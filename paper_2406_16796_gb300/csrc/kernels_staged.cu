@@ -778,12 +778,11 @@ cudaError_t run_staged(axp_grid *g, int64_t nsteps)
     return cudaGetLastError();
 }
 
-// f(Passes of the grid's active axes and order-0 components)
+// f(Passes of the grid's active axes and the order-0 components m)
 template <typename T, typename F>
-auto with_passes(const axp_grid *g, F &&f)
+auto with_passes(const axp_grid *g, uint32_t m, F &&f)
 {
     const int64_t *n = g->desc.n;
-    const uint32_t m = order0_closure(g);
     auto in = [&](uint32_t set) { return (m & ~set) == 0; };
     const uint32_t tm = 4u | (3u << 3), te = 3u | (4u << 3);  // (E0z; B0x, B0y) and (E0x, E0y; B0z)
     if (n[1] == 1 && n[2] == 1) {
@@ -812,27 +811,27 @@ bool staged_supported(const axp_grid *g)
 }
 
 template <typename T>
-cudaError_t staged_step(axp_grid *g, int64_t nsteps)
+cudaError_t staged_step(axp_grid *g, int64_t nsteps, uint32_t order0)
 {
-    return with_passes<T>(g, [&](auto q) { return run_staged<T, decltype(q)>(g, nsteps); });
+    return with_passes<T>(g, order0, [&](auto q) { return run_staged<T, decltype(q)>(g, nsteps); });
 }
 
 template <typename T>
 cudaError_t staged_enter(axp_grid *g)
 {
-    with_passes<T>(g, [&](auto q) { first_half<T, decltype(q)>(g); });
+    with_passes<T>(g, order0_present(g), [&](auto q) { first_half<T, decltype(q)>(g); });
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t staged_exit(axp_grid *g, int oset)
 {
-    with_passes<T>(g, [&](auto q) { back_half<T, decltype(q)>(g, oset); });
+    with_passes<T>(g, order0_present(g), [&](auto q) { back_half<T, decltype(q)>(g, oset); });
     return cudaGetLastError();
 }
 
-template cudaError_t staged_step<double>(axp_grid *, int64_t);
-template cudaError_t staged_step<float>(axp_grid *, int64_t);
+template cudaError_t staged_step<double>(axp_grid *, int64_t, uint32_t);
+template cudaError_t staged_step<float>(axp_grid *, int64_t, uint32_t);
 template cudaError_t staged_enter<double>(axp_grid *);
 template cudaError_t staged_enter<float>(axp_grid *);
 template cudaError_t staged_exit<double>(axp_grid *, int);
