@@ -259,9 +259,9 @@ int64_t line_seg(const axp_grid *g)
 // pass of 64 cells (12, 14, 15: 1.80, 1.77, 1.76 us per step; 16 takes two passes).  The
 // bits of a run do not depend on it.
 template <typename T>
-int line_block(int64_t seg)
+int line_block(int64_t seg, bool layer)
 {
-    const int lanes = line1d::lanes_of<T>(), most = line1d::max_window<T>();
+    const int lanes = line1d::lanes_of<T>(), most = line1d::max_window<T>(layer);
     const double pass = sizeof(T) == 8 ? 1.6 : 0.45;
     int best = 0;
     double best_cost = 0.0;
@@ -300,10 +300,11 @@ bool line_takes(const axp_grid *g, int kind)
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, g->device) != cudaSuccess || !coop) return false;
     const int64_t seg = line_seg(g);
     if (seg < 1) return false;
-    // periodic FP64 windows as ever: up to 964 cells a block; the others while a step of theirs
-    // is cheaper than a launch of the generic kernel (kLineMost cells)
-    if (kind == 0) return seg + 2 * 18 <= 1000 && line_block<double>(seg) >= 1;
-    return d.n[0] <= kLineMost && (d.precision == AXP_FP64 ? line_block<double>(seg) : line_block<float>(seg)) >= 1;
+    // periodic FP64: room for 15 steps in a window, up to 964 cells a block (146,528 on 152 SMs;
+    // 145,000 cells 23 us a step, the generic kernel 33); the others while a step of theirs is
+    // cheaper than a launch of the generic kernel (kLineMost cells)
+    if (kind == 0) return seg + 2 * 18 <= line1d::max_window<double>(false) && line_block<double>(seg, false) >= 1;
+    return d.n[0] <= kLineMost && (d.precision == AXP_FP64 ? line_block<double>(seg, !per) : line_block<float>(seg, !per)) >= 1;
 }
 bool block1d_supported(const axp_grid *g) { return line_takes(g, 0); }
 
@@ -320,13 +321,13 @@ cudaError_t block1d_step(axp_grid *g, int64_t nsteps)
     std::memset(&A, 0, sizeof(A));
     A.n = d.n[0];
     A.seg = (int)line_seg(g);
-    A.tblock = line_block<T>(A.seg);
+    const bool layer = d.em_bc[0][0] != AXP_BC_PERIODIC;
+    A.tblock = line_block<T>(A.seg, layer);
     A.halo = A.tblock + 3;
     const int blocks = (int)((d.n[0] + A.seg - 1) / A.seg);
-    const bool layer = d.em_bc[0][0] != AXP_BC_PERIODIC;
     const size_t smem = (size_t)(line1d::kArrays + (layer ? line1d::kLayerArrays : 0)) * (A.seg + 2 * A.halo) * sizeof(T);
     const void *kern = layer ? (const void *)line1d::k_line1d<T, true> : (const void *)line1d::k_line1d<T, false>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, line1d::kWindowBytes);
     if (e != cudaSuccess) return e;
     const double dx = d.d[0], dt = d.dt;
     A.cB = (T)(dt / 2.0 / dx);

@@ -60,8 +60,16 @@ template <typename T>
 __host__ __device__ constexpr int lanes_of() { return threads_of<T>() / 2; }  // cells a pass of one half covers
 constexpr int kArrays = 28;              // window arrays (listed in k_line1d)
 constexpr int kLayerArrays = 7;          // and the layer's coefficients
+// A window's largest shared memory: 1000 cells of a periodic FP64 grid (218.75 of the 227 KB a
+// block may have), 789 cells with layers (their own arrays on top: 216 KB); twice that in FP32.
+constexpr int kWindowBytes = 1000 * kArrays * (int)sizeof(double);
+constexpr int kLayerWindow = 789;
+static_assert(kLayerWindow * (kArrays + kLayerArrays) * (int)sizeof(double) <= kWindowBytes, "layered windows fit");
 template <typename T>
-__host__ __device__ constexpr int max_window() { return 216 * 1024 / ((kArrays + kLayerArrays) * (int)sizeof(T)); }
+__host__ __device__ constexpr int max_window(bool layer)
+{
+    return (layer ? kLayerWindow : 1000) * (int)(sizeof(double) / sizeof(T));
+}
 constexpr unsigned kSpinLimit = 1u << 26;        // polls of a grid-wide wait before it gives up ...
 constexpr unsigned long long kWaitNs = 1000000000ull;  // ... or one second, whichever comes first
 

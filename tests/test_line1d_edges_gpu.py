@@ -45,3 +45,24 @@ def test_layers_of_any_strength_are_damped(axion, nx, pml, sigma):
     for k in NAMES:
         assert np.all(np.abs(out[0][k] - out[1][k]) <= 1e-34), (k, rel(out[0][k], out[1][k]))
         assert rel(out[0][k], ref[k]) < 1e-4, (k, rel(out[0][k], ref[k]))
+
+
+@pytest.mark.parametrize("nx", [118712, 118714, 131072, 146528])
+def test_large_periodic_grids_keep_the_kernel(nx):
+    """Up to 964 cells a block (152 SMs), chosen by AUTO and by name, with the generic
+    kernel's fields."""
+    from paper_2406_16796_gb300 import axp
+
+    grid = line(nx, "periodic", "fp64")
+    st = W.random_state(grid, seed=44, active=LASER)
+    out = []
+    for kernel in (axp.AXP_KERNEL_BLOCK1D, axp.AXP_KERNEL_FUSED):
+        g = axp.Grid(grid)
+        assert g.kernel_path() == axp.AXP_KERNEL_BLOCK1D
+        g.load(st)
+        g.set_kernel(kernel)
+        g.step(40)
+        out.append(g.fields())
+        g.close()
+    for k in NAMES:
+        assert rel(out[0][k], out[1][k]) < 1e-12, (k, rel(out[0][k], out[1][k]))
