@@ -3,7 +3,8 @@
 //
 // A 1D grid of a few thousand cells is far too small to fill the GPU: launched
 // one step at a time its steps cost launch and synchronisation latency, not
-// arithmetic.  Here one cooperative launch runs a whole run of steps.  Each
+// arithmetic.  Here one cooperative launch (a plain one where no wait is met) runs a
+// whole run of steps.  Each
 // block owns `seg` consecutive cells and holds them, with `halo` cells on each
 // side, in shared memory; it advances that window `tblock` steps on its own,
 // writes its owned cells to the other buffer set and meets the other blocks at
@@ -178,6 +179,8 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
     const int64_t wl = LAYER ? A.lay[0] - (s0 - H) : 0, wh = LAYER ? N - A.lay[1] - (s0 - H) : W;
     const bool layered = LAYER && (wl > 0 || wh < W);  // this window's body
     auto in_layer = [&](int w) { return LAYER && layered && (w < wl || w >= wh); };
+    // (a plain launch may be set up while the kernel before it ends; it waits here for that
+    // kernel's memory, of which the layer's tables are no part)
     if (LAYER && layered) {
         for (int w = tid; w < W; w += nt) {
             const int64_t gi = s0 - H + w;
@@ -204,6 +207,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
         }
     }
 
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     int par = 0;
     unsigned waits = 0;
     for (int64_t done = 0; done < A.nsteps; done += A.tblock) {

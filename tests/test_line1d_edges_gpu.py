@@ -66,3 +66,49 @@ def test_large_periodic_grids_keep_the_kernel(nx):
         g.close()
     for k in NAMES:
         assert rel(out[0][k], out[1][k]) < 1e-12, (k, rel(out[0][k], out[1][k]))
+
+
+def us_per_call(g, steps, calls=300):
+    import time
+
+    best = 1e9
+    for _ in range(7):
+        g.synchronize()
+        t0 = time.perf_counter()
+        for _ in range(calls):
+            g.step(steps)
+        g.synchronize()
+        best = min(best, (time.perf_counter() - t0) / calls)
+    return best * 1e6
+
+
+@pytest.mark.parametrize("nx,bc", [(256, "periodic"), (4096, "periodic"), (65536, "periodic"), (2048, "pml")])
+def test_single_steps_cost_no_more_than_a_launch_of_the_generic_kernel(nx, bc):
+    """step(1) in FP32: a run of one window takes neither the counter's reset nor a
+    cooperative launch (both together: 1.2 to 2.0 times the generic kernel's call)."""
+    from paper_2406_16796_gb300 import axp
+
+    t = []
+    for kernel in (axp.AXP_KERNEL_AUTO, axp.AXP_KERNEL_FUSED):
+        g = axp.Grid(line(nx, bc, "fp32"))
+        g.load(W.random_state(g.spec, seed=44, active=LASER, scale0=1e-3))
+        g.set_kernel(kernel)
+        t.append(us_per_call(g, 1))
+        g.close()
+    assert t[0] < 1.15 * t[1], t
+
+
+def test_runs_of_one_window_and_of_several_mix():
+    """Any split of the steps, periodic FP64 too: the same bits, whichever launch a run takes."""
+    from paper_2406_16796_gb300 import axp
+
+    out = []
+    for chunks in ([200], [1] * 20 + [14, 15, 16, 100, 35], [60, 1, 139]):
+        g = axp.Grid(line(4999, "periodic", "fp64"))
+        g.load(W.random_state(g.spec, seed=44, active=LASER))
+        for c in chunks:
+            g.step(c)
+        out.append(g.fields())
+        g.close()
+    for k in NAMES:
+        assert np.array_equal(out[0][k], out[1][k]) and np.array_equal(out[0][k], out[2][k]), k
