@@ -179,6 +179,9 @@ struct axp_grid {
     int64_t tm_plan_key;
     int32_t tm_tx, tm_chunk, tm_chunk_first, tm_chunk_edge, tm_nchunks;
     int32_t tm_list_blocks, tm_list_per_block;
+    // the plan of its FP32 form in warp tiles (warp_tiles 0: not made yet); it depends on the
+    // descriptor and the device alone
+    int32_t warp_chunk, warp_first, warp_edge, warp_tiles;
     std::vector<int4> tm_items;  // the work lists (host copy)
     bool tm_items_uploaded;      // tm_items are in off_sched
     // the other field set holds E^{n-1/2} of the present staggered state E^{n+1/2}:

@@ -923,19 +923,17 @@ constexpr int64_t kWarpMost = 1200000;
 // chunk + 6 planes of pipeline.  A strip at a non-periodic x edge takes 1.35 times as long
 // per plane and a chunk over a y layer 0.32 planes' time more for each of the layer's (and 7
 // pipeline) planes; their chunks are shortened by that (1.0 and 0: 1536 x 768 29.5 us
-// against 27.0; 2.0 and 0.6: 29.0).
-struct WarpPlan {
-    int chunk, first, edge, ntiles;
-};
-WarpPlan warp_plan(const axp_grid *g, int resident)
+// against 27.0; 2.0 and 0.6: 29.0).  Made once per handle: on every call the search took
+// 0.36 ms of the host's time at 16 x 65536 cells, against a step of 57 us.
+void warp_plan(axp_grid *g, int resident)
 {
+    if (g->warp_tiles > 0) return;
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
     const axp_grid_desc &d = g->desc;
     const bool perx = d.em_bc[0][0] == AXP_BC_PERIODIC, pery = d.em_bc[1][0] == AXP_BC_PERIODIC;
     const int64_t ny = d.n[1], strips = (d.n[0] + tm2d_x2::WVX - 1) / tm2d_x2::WVX, nedge = perx ? 0 : std::min<int64_t>(strips, 2);
     const int64_t slots = (int64_t)sms * resident, shorter = pery ? 0 : (int64_t)(0.32 * (double)(d.pml_cells + 7));
-    WarpPlan best{0, 0, 0, 0};
     double best_cost = 0.0;
     for (int64_t chunk = std::min<int64_t>(ny, 4); chunk <= ny; chunk++) {
         const int64_t least = std::min<int64_t>(chunk, 4);
@@ -944,12 +942,15 @@ WarpPlan warp_plan(const axp_grid *g, int resident)
         const int64_t nin = 1 + (ny - first + chunk - 1) / chunk, nout = (ny + edge - 1) / edge;
         const int64_t tiles = (strips - nedge) * nin + nedge * nout;
         const double cost = (double)((tiles + slots - 1) / slots) * (double)(chunk + 6);
-        if (best.chunk == 0 || cost < best_cost) {
+        if (g->warp_tiles == 0 || cost < best_cost) {
             best_cost = cost;
-            best = WarpPlan{(int)chunk, (int)first, (int)edge, (int)tiles};
+            g->warp_chunk = (int32_t)chunk;
+            g->warp_first = (int32_t)first;
+            g->warp_edge = (int32_t)edge;
+            g->warp_tiles = (int32_t)tiles;
         }
+        if (tiles <= slots) break;  // one wave: longer chunks only add planes to it
     }
-    return best;
 }
 
 template <typename T>
@@ -981,6 +982,7 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     int tm_tx = tm2d::TX;  // tile width of the 2D kernel (chosen below)
     // FP32 split on an even-width grid without a soft source: the two-column form
     const bool x2 = tm && tm2d_x2_eligible<T>(g);
+    const bool warps = x2 && g->desc.n[0] * g->desc.n[1] <= kWarpMost;
     auto dispatch_2d = [&](const fused::Params<T> &Pl, int nch, int *occp, int width) -> cudaError_t {
         if constexpr (sizeof(T) == 4) {
             if (x2) return tm2d_x2_dispatch_f32(Pl, nch, g->stream, occp, width);
@@ -1022,6 +1024,15 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
                 nchunks = (int)((nz + chunk - 1) / chunk);
             }
         }
+    } else if (warps) {
+        if constexpr (sizeof(T) == 4) {
+            int resident = 0;
+            if ((e = tm2d_x2_warps_dispatch_f32(P, 0, g->stream, &resident)) != cudaSuccess) return e;
+            warp_plan(g, resident);
+            P.chunk = g->warp_chunk;
+            P.chunk_first = g->warp_first;
+            P.chunk_edge = g->warp_edge;
+        }
     } else if (tm) {
         if ((e = tm2d_plan<T>(g)) != cudaSuccess) return e;
         tm_tx = g->tm_tx;
@@ -1045,17 +1056,6 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
         int64_t chunk = (nm + nc - 1) / nc;
         nchunks = (int)((nm + chunk - 1) / chunk);
         P.chunk = (int)chunk;
-    }
-    WarpPlan wp{0, 0, 0, 0};
-    if constexpr (sizeof(T) == 4) {
-        if (x2 && g->desc.n[0] * g->desc.n[1] <= kWarpMost) {
-            int resident = 0;
-            if ((e = tm2d_x2_warps_dispatch_f32(P, 0, g->stream, &resident)) != cudaSuccess) return e;
-            wp = warp_plan(g, resident);
-            P.chunk = wp.chunk;
-            P.chunk_first = wp.first;
-            P.chunk_edge = wp.edge;
-        }
     }
     int64_t it = 0;
     if (mode == 1 && !tm && !ax && g->desc.diag_every == 0 && nsteps >= kGraphSteps) {
@@ -1081,7 +1081,7 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
             P.chunk_first = chf;
         }
         if constexpr (sizeof(T) == 4)
-            e = wp.ntiles > 0 ? tm2d_x2_warps_dispatch_f32(P, wp.ntiles, g->stream, nullptr) : launch(P, nchunks, nullptr);
+            e = warps ? tm2d_x2_warps_dispatch_f32(P, g->warp_tiles, g->stream, nullptr) : launch(P, nchunks, nullptr);
         else
             e = launch(P, nchunks, nullptr);
         if (e != cudaSuccess) return e;
