@@ -415,7 +415,8 @@ axp_status axp_get_window_offset(const axp_grid *grid, int64_t *cells);
  * generic single-pass kernel (1D/2D/3D, periodic, reflect and PML edges);
  * AXP_KERNEL_TM2D forces the single-pass kernel specialised for 2D grids with
  * an (E0z; B0x, B0y) laser and periodic or PML edges (at most 2^32 cells), on
- * its uniform launch grid of x strips by march chunks;
+ * its uniform launch grid of x strips by march chunks (AUTO runs FP32 grids of
+ * even width and up to 1.2M cells in tiles of one warp each, the same bits);
  * AXP_KERNEL_TM2D_LIST forces the same kernel on per-block work lists (FP64
  * grids without a soft source): the host cuts each x strip into tiles of about
  * equal cost and lets two short tiles share a block, so that every block, all

@@ -982,7 +982,8 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     int tm_tx = tm2d::TX;  // tile width of the 2D kernel (chosen below)
     // FP32 split on an even-width grid without a soft source: the two-column form
     const bool x2 = tm && tm2d_x2_eligible<T>(g);
-    const bool warps = x2 && g->desc.n[0] * g->desc.n[1] <= kWarpMost;
+    // (forced, the 2D kernel keeps its uniform launch grid of block tiles)
+    const bool warps = x2 && g->kernel_choice == AXP_KERNEL_AUTO && g->desc.n[0] * g->desc.n[1] <= kWarpMost;
     auto dispatch_2d = [&](const fused::Params<T> &Pl, int nch, int *occp, int width) -> cudaError_t {
         if constexpr (sizeof(T) == 4) {
             if (x2) return tm2d_x2_dispatch_f32(Pl, nch, g->stream, occp, width);
