@@ -10,6 +10,8 @@
 #include <new>
 #include <vector>
 
+#include <unistd.h>
+
 #include "axp_internal.h"
 
 using namespace axp;
@@ -782,6 +784,9 @@ static void *field_ptr(axp_grid *g, int which)
     return g->ws + g->layout.off_phi[g->phi_b_slot];
 }
 
+// largest FP32 array that axp_read_field widens on the host
+constexpr int64_t kReadHost = 1 << 16;
+
 axp_status axp_read_field(axp_grid *g, int32_t which, double *dst, size_t bytes)
 {
     if (!g || !dst || which < 0 || which > AXP_PHI_OLD) return AXP_E_INVAL;
@@ -794,8 +799,26 @@ axp_status axp_read_field(axp_grid *g, int32_t which, double *dst, size_t bytes)
     const axp_status lat = latched_status(g);
     if (lat != AXP_OK) return lat;
     if (!is_fp32(g)) return cuda_status(cudaMemcpy(dst, field_ptr(g, which), bytes, cudaMemcpyDeviceToHost));
-    // FP32: widened on the device, into the current's scratch (three float arrays in a row hold
-    // the array as doubles; P is formed anew whenever it is needed)
+    // FP32.  A small array goes through a float copy on the host: fewer steps (16384 cells into
+    // fresh memory 0.025 ms, widened on the device 0.033; 65536 cells 0.06 both ways).
+    if (N <= kReadHost) {
+        std::vector<float> tmp((size_t)N), inc;
+        e = cudaMemcpy(tmp.data(), field_ptr(g, which == AXP_PHI_OLD ? AXP_PHI_CUR : which), N * 4, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess && which == AXP_PHI_OLD) {
+            inc.resize((size_t)N);
+            e = cudaMemcpy(inc.data(), g->ws + g->layout.off_phi[g->phi_b_slot], N * 4, cudaMemcpyDeviceToHost);
+        }
+        if (e != cudaSuccess) return cuda_status(e);
+        for (int64_t c = 0; c < N; c++) dst[c] = which == AXP_PHI_OLD ? (double)tmp[c] - (double)inc[c] : (double)tmp[c];
+        return AXP_OK;
+    }
+    // A larger one is widened on the device, into the current's scratch (three float arrays in a
+    // row hold the array as doubles; P is formed anew whenever it is needed).  The host touches
+    // the caller's pages first: left to the copy, each page of fresh memory costs a fault of
+    // the GPU's (512 x 512 cells 0.25 ms against 0.13, 256 x 256 0.18 against 0.06).
+    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    for (size_t b = 0; b < bytes; b += page) ((volatile char *)dst)[b] = 0;
+    ((volatile char *)dst)[bytes - 1] = 0;
     double *wide = (double *)(g->ws + g->layout.off_P[0]);
     const float *from = (const float *)field_ptr(g, which == AXP_PHI_OLD ? AXP_PHI_CUR : which);
     const float *less = which == AXP_PHI_OLD ? (const float *)(g->ws + g->layout.off_phi[g->phi_b_slot]) : nullptr;
