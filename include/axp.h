@@ -34,7 +34,8 @@
  * AXP_FP32_SPLIT stores all arrays in float, keeps E0/B0 and E1/B1 apart as
  * the paper's FPS method does (Sec. 2.2), holds phi as phi^{n+1/2} plus the
  * increment phi^{n+1/2} - phi^{n-1/2}, takes the uniform background fields as
- * double constants, and accumulates every diagnostic in double.
+ * double constants, and accumulates every diagnostic in double or in sums of
+ * floats that lose less (error-free, three floats to a sum).
  *
  * Errors: every call returns an axp_status; nothing is thrown across the
  * ABI.  Kernel launch errors are returned by the call that launched;

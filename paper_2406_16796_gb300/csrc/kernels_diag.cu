@@ -26,17 +26,22 @@ constexpr int kQ = 7;  // H_phi, H_g0, H_g1, cross, sum x B1z^2, sum B1z^2, gaus
 // cycle per SM: 36.7 ms for the 512^3 FP32 box, whose 8 arrays cross HBM in 0.7 ms).
 //  * Only the components that can be non-zero are read (template masks).
 //  * Constants (1/2, dV, 1/d^2, m^2, 1/dt^2) are applied to the sums, not per cell.
-//  * FP64 grids work in double.  FP32 grids work in pairs of floats (a value as the
-//    sum hi + lo of two floats, 48 bits; error-free sums and products after Dekker and
-//    Knuth, products by fma), on the FP32 pipe that is 64 times wider.  Each input is an
-//    exact float, so the pairs hold differences and squares of them as a double would
-//    to 2^-48, and a thread's partial sum is turned into a double once.
+//  * FP64 grids work in double.  FP32 grids do no less, mostly on the FP32 pipe that is 64
+//    times wider: each input is a float, so a difference or a product of two is exactly a
+//    pair of floats (error-free sums and products after Knuth and Dekker, products by
+//    fma), and a thread adds such pairs into three floats with error-free sums (what is
+//    dropped is below 2^-70).  The thread's sum becomes a double once, with one rounding where
+//    a sum of doubles takes one per term.  The Gauss residual, a sum of scaled differences
+//    that cancel, is formed and squared in double, its floats widened by their bits: the FP64
+//    pipe is idle otherwise (the E1 and B1 sums there too: 512^3 6.5 -> 8.8 ms).
+//    Worst relative error of H_g0, H_g1 and sum_B1z2 against exact sums, 48 states of 300 to
+//    2.1M cells: 3.2e-16 (literal doubles 2.5e-16; pairs of floats 2.4e-14).
 //  * Floats span less than squares of small fields need, so each group of fields is
 //    scaled by a power of two taken from its largest magnitude in the region (max_group:
 //    a pass of its own, or part of the pass that forms E^n).  Scaling by a power of
 //    two is exact; what then underflows is below 2^-60 of the largest value.
-// Measured, a whole record (us, before -> after): 512^3 FP32 box 37000 -> 6040; 4096 x 2048
-// pulse FP32 1100 -> 430; FP64 unchanged at 1110 (50 operations per cell on the FP64 pipe).
+// Measured, a whole record (us, against the literal doubles): 512^3 FP32 box 37000 -> 6540; 4096 x 2048
+// pulse FP32 1100 -> 530; FP64 unchanged at 1110 (50 operations per cell on the FP64 pipe).
 // ---------------------------------------------------------------------------
 struct FF {
     float h, l;
@@ -46,37 +51,40 @@ __device__ __forceinline__ FF two_sum(float a, float b)
     const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
     return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
 }
-__device__ __forceinline__ FF quick_sum(float a, float b)  // |a| >= |b|
+__device__ __forceinline__ FF two_prod(float a, float b)
 {
-    const float s = __fadd_rn(a, b);
-    return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ FF operator+(FF a, FF b)
-{
-    const FF s = two_sum(a.h, b.h);
-    return quick_sum(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ FF operator*(FF a, FF b)
-{
-    const float p = __fmul_rn(a.h, b.h);
-    const float e = __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p)));
-    return quick_sum(p, e);
-}
-__device__ __forceinline__ FF operator*(FF a, float b)
-{
-    const float p = __fmul_rn(a.h, b);
-    return quick_sum(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+    const float p = __fmul_rn(a, b);
+    return {p, __fmaf_rn(a, b, -p)};
 }
 
-// a running sum of pairs: the high words by an error-free sum, the low words as they come
-// (the pair is normalised once, when the thread's sum becomes a double)
-__device__ __forceinline__ void accumulate(FF &acc, FF x)
+// a float as a double, by its bits: a conversion instruction takes the FP64 pipe.  (Zero, and
+// what has no normal exponent, apart.)
+__device__ __forceinline__ double as_double(float x)
+{
+    const int u = __float_as_int(x);
+    const unsigned e = (unsigned)u & 0x7f800000u;
+    if (e - 1u >= 0x7f800000u - 1u) return x == 0.0f ? 0.0 : (double)x;
+    return __hiloint2double(((u >> 3) & (int)0x8fffffff) + (896 << 20), u << 29);
+}
+__device__ __forceinline__ double as_double(double x) { return x; }
+
+// a thread's running sum of pairs: high and middle words by error-free sums; the last takes
+// what those leave over, 2^-48 of the sum and less, in plain float
+struct Acc3 {
+    float h, m, l;
+};
+__device__ __forceinline__ void accumulate_low(Acc3 &acc, FF x)  // a term 2^-23 of its sum or less
+{
+    const FF u = two_sum(acc.m, x.h);
+    acc.m = u.h;
+    acc.l = __fadd_rn(acc.l, __fadd_rn(u.l, x.l));
+}
+__device__ __forceinline__ void accumulate(Acc3 &acc, FF x)
 {
     const FF s = two_sum(acc.h, x.h);
     acc.h = s.h;
-    acc.l = __fadd_rn(acc.l, __fadd_rn(s.l, x.l));
+    accumulate_low(acc, two_sum(x.l, s.l));
 }
-__device__ __forceinline__ void accumulate(double &acc, double x) { acc = acc + x; }
 
 // Sums of 7 quantities over a warp: at each of the first three steps a lane keeps half of
 // its values and adds its partner's, so 9 additions take the place of 35 (an FP64
@@ -105,35 +113,69 @@ __device__ __forceinline__ void block_sums(double v[8], double sh[8][kDiagThread
     __syncthreads();
 }
 
-// the arithmetic of the sums: V holds a term, from values T
+// the arithmetic of the sums of values T: Acc a running sum
 template <typename T>
 struct Ops;
 template <>
 struct Ops<double> {
-    using V = double;
-    static __device__ __forceinline__ V of(double a) { return a; }
-    static __device__ __forceinline__ V diff(double a, double b) { return a - b; }
-    static __device__ __forceinline__ V prod(double a, double b) { return a * b; }
-    static __device__ __forceinline__ V square(V a) { return a * a; }
-    static __device__ __forceinline__ double total(V a) { return a; }
+    using Acc = double;
+    static __device__ __forceinline__ void add_prod(Acc &s, double a, double b) { s = fma(a, b, s); }
+    static __device__ __forceinline__ void add_square_of_diff(Acc &s, double a, double b)
+    {
+        const double d = a - b;
+        s = fma(d, d, s);
+    }
+    static __device__ __forceinline__ void add_sum_times(Acc &s, double a, double b, double c) { s = fma(a + b, c, s); }
+    static __device__ __forceinline__ void add_square_times(Acc &s, double a, int k) { s = fma((double)k, a * a, s); }
+    static __device__ __forceinline__ double diff(double a, double b) { return a - b; }
+    static __device__ __forceinline__ double total(Acc a) { return a; }
+    static __device__ __forceinline__ double total(Acc a, Acc b) { return a + b; }
     static __device__ __forceinline__ double scaled(double a, double) { return a; }
 };
 template <>
 struct Ops<float> {
-    using V = FF;
-    static __device__ __forceinline__ V of(float a) { return {a, 0.0f}; }
-    static __device__ __forceinline__ V diff(float a, float b) { return two_sum(a, -b); }
-    static __device__ __forceinline__ V prod(float a, float b)
+    using Acc = Acc3;
+    static __device__ __forceinline__ void add_prod(Acc &s, float a, float b) { accumulate(s, two_prod(a, b)); }
+    // (a - b)^2, exact: h^2 + 2 h l + l^2 (l is 0 for neighbours within a factor of 2)
+    static __device__ __forceinline__ void add_square_of_diff(Acc &s, float a, float b)
     {
-        const float p = __fmul_rn(a, b);
-        return {p, __fmaf_rn(a, b, -p)};
+        const FF d = two_sum(a, -b);
+        accumulate(s, two_prod(d.h, d.h));
+        if (d.l != 0.0f) {
+            accumulate_low(s, two_prod(__fadd_rn(d.h, d.h), d.l));
+            s.l = __fmaf_rn(d.l, d.l, s.l);
+        }
     }
-    static __device__ __forceinline__ V square(V a)  // (not normalised: for accumulate)
+    static __device__ __forceinline__ void add_sum_times(Acc &s, float a, float b, float c)
     {
-        const float p = __fmul_rn(a.h, a.h);
-        return {p, __fmaf_rn(__fadd_rn(a.h, a.h), a.l, __fmaf_rn(a.h, a.h, -p))};
+        const FF d = two_sum(a, b);
+        accumulate(s, two_prod(d.h, c));
+        if (d.l != 0.0f) accumulate_low(s, two_prod(d.l, c));
     }
-    static __device__ __forceinline__ double total(V a) { return (double)a.h + (double)a.l; }
+    // k a^2; a float holds integers up to 2^24, larger ones come as two
+    static __device__ __forceinline__ void add_square_times(Acc &s, float a, int k)
+    {
+        const FF p = two_prod(a, a);
+        const int low = k > (1 << 24) ? k & 0xfff : 0;
+        const float k1 = (float)(k - low);
+        accumulate(s, two_prod(p.h, k1));
+        accumulate_low(s, two_prod(p.l, k1));
+        if (low) {
+            accumulate(s, two_prod(p.h, (float)low));
+            accumulate_low(s, two_prod(p.l, (float)low));
+        }
+    }
+    static __device__ __forceinline__ double diff(float a, float b)
+    {
+        const FF d = two_sum(a, -b);
+        const double x = as_double(d.h);
+        return __any_sync(__activemask(), d.l != 0.0f) ? x + as_double(d.l) : x;
+    }
+    static __device__ __forceinline__ double total(const Acc &a) { return (double)a.h + ((double)a.m + (double)a.l); }
+    static __device__ __forceinline__ double total(const Acc &a, const Acc &b)
+    {
+        return ((double)a.h + (double)b.h) + (((double)a.m + (double)b.m) + ((double)a.l + (double)b.l));
+    }
     static __device__ __forceinline__ float scaled(float a, float s) { return __fmul_rn(a, s); }
 };
 
@@ -147,14 +189,15 @@ struct Sums {
     unsigned N;
     T Bext[3], Eext[3];
     int ext;                           // bits: non-zero background components, E (0-2) and B (3-5)
-    double d[3], lo0, dt, g, m2;
+    double d[3], lo0, dt, m2;
+    double rd[3], kg, kgb[3];          // 1/d; g/2 times phi^n over what mid_at gives, and that times B_ext
     unsigned *top;      // FP32: largest magnitude of E0/B0, E1/B1, phi (float bits)
     double *partials;
     axp_diag *out;
     int64_t step;
 };
 
-constexpr int kSums = 11;  // phi: Dt^2, mid^2, 3 forward differences; E0B0^2; E1B1^2 less B1z; cross; x B1z^2; B1z^2; R^2
+constexpr int kSums = 10;  // phi: Dt^2, mid^2, 3 forward differences; E0B0^2; E1B1^2 less B1z; cross; x B1z^2; B1z^2
 
 // a power of two near 1 / (largest magnitude), kept well inside the floats' range
 __device__ __forceinline__ float scale_of(double top)
@@ -180,16 +223,20 @@ __device__ __forceinline__ T mid_at(const Sums<T> &s, int a, int side, const Cel
     return INCR ? T(0.5) * sum : sum;
 }
 
+// Resident blocks: the 3D form waits on memory more and takes a fourth in spite of a few spills
+// (512^3 FP32: 7.3 ms with three, 6.5 with four; 1024 x 512 0.094 and 0.104).
+template <typename T>
+__host__ __device__ constexpr int diag_blocks_per_sm(int mask) { return sizeof(T) == 4 && mask != 7 ? 3 : 4; }
+
 // EM, BM: the order-0 components present
 template <typename T, int MASK, int EM, int BM>
-__global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 ? 3 : 4) k_diag_sums(Sums<T> s)
+__global__ void __launch_bounds__(kDiagThreads, diag_blocks_per_sm<T>(MASK)) k_diag_sums(Sums<T> s)
 {
     using O = Ops<T>;
-    using V = typename O::V;
     constexpr bool INCR = sizeof(T) == 4;
-    // scales: of phi, of the order-0 and order-1 fields, of the order-0 fields with the
-    // background, and of the Gauss residual (1 in double)
-    T sp = T(1), s0 = T(1), s1 = T(1), sx = T(1), sr = T(1);
+    // scales: of phi, of the order-0 and order-1 fields, and of the order-0 fields with the
+    // background (1 in double)
+    T sp = T(1), s0 = T(1), s1 = T(1), sx = T(1);
     if (INCR) {
         const double t0 = __uint_as_float(s.top[0]), t1 = __uint_as_float(s.top[1]), tp = __uint_as_float(s.top[2]);
         double ext = 0.0;
@@ -198,22 +245,10 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 ? 3 : 4) k_diag_s
         s0 = scale_of(t0);
         s1 = scale_of(t1);
         sx = scale_of(max(t0, ext));
-        sr = scale_of(max(t1, fabs(s.g) * max(t0, ext) * tp));
     }
-    V acc[kSums];
-#pragma unroll
-    for (int k = 0; k < kSums; k++) acc[k] = O::of(T(0));
-    V rd[3], kg;  // 1/d, and g/2 times the Gauss sum's scale over phi's
-#pragma unroll
-    for (int a = 0; a < 3; a++) {
-        const double x = 1.0 / s.d[a];
-        if constexpr (INCR) rd[a] = {(float)x, (float)(x - (double)(float)x)};
-        else rd[a] = x;
-    }
+    typename O::Acc acc[kSums] = {};
+    double gauss = 0.0;        // sum of R^2
     constexpr double half = INCR ? 1.0 : 0.5;  // phi^n over what mid_at gives
-    const double kd = half * 0.5 * s.g * ((double)sr / (double)sp);
-    if constexpr (INCR) kg = {(float)kd, (float)(kd - (double)(float)kd)};
-    else kg = kd;
     for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < s.N; c += gridDim.x * blockDim.x) {
         Cell q;
         cell_of_index<MASK>(s.n, s.per, c, q);
@@ -223,18 +258,17 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 ? 3 : 4) k_diag_s
         if (!in) continue;
         const T hi = s.phi[c], b = s.phib[c];
         const T mid = O::scaled(INCR ? hi - T(0.5) * b : hi + b, sp);
-        if constexpr (INCR) accumulate(acc[0], O::prod(O::scaled(b, sp), O::scaled(b, sp)));
-        else accumulate(acc[0], O::square(O::diff(hi, b)));
-        accumulate(acc[1], O::prod(mid, mid));
-        V R = O::of(T(0));
+        if constexpr (INCR) O::add_prod(acc[0], O::scaled(b, sp), O::scaled(b, sp));
+        else O::add_square_of_diff(acc[0], hi, b);
+        O::add_prod(acc[1], mid, mid);
+        double R = 0.0;
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             if (!(MASK >> a & 1)) continue;
-            const T up = O::scaled(mid_at<T, MASK>(s, a, 1, q), sp), dn = O::scaled(mid_at<T, MASK>(s, a, 0, q), sp);
-            accumulate(acc[2 + a], O::square(O::diff(up, mid)));
+            const T up = mid_at<T, MASK>(s, a, 1, q), dn = mid_at<T, MASK>(s, a, 0, q);
+            O::add_square_of_diff(acc[2 + a], O::scaled(up, sp), mid);
             // div E1 + g Bbar0 . grad_c phi, term by term along the axis
-            V t = O::diff(O::scaled(s.E1[a][c], sr), O::scaled(ldz(s.E1[a], q.dn[a], q.hd[a]), sr));
-            T bb = s.Bext[a];
+            double t = O::diff(s.E1[a][c], ldz(s.E1[a], q.dn[a], q.hd[a]));
             if (BM >> a & 1) {
                 const int p = (a + 1) % 3, r = (a + 2) % 3;
                 const T *B = s.B0[a];
@@ -250,42 +284,42 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 ? 3 : 4) k_diag_s
                     f = f + h;
                     w = w * T(0.5);
                 }
-                bb = w * f + bb;
+                t = fma(O::diff(up, dn), s.kg * as_double(w * f + s.Bext[a]), t);
+            } else if (s.ext >> (3 + a) & 1) {
+                t = fma(O::diff(up, dn), s.kgb[a], t);
             }
-            if ((BM >> a & 1) || (s.ext >> (3 + a) & 1)) t = t + (O::diff(up, dn) * kg) * bb;
-            R = R + t * rd[a];
+            R = fma(t, s.rd[a], R);
         }
-        accumulate(acc[10], O::square(R));
+        gauss = fma(R, R, gauss);
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             const T e1 = O::scaled(s.E1[a][c], s1), b1 = O::scaled(s.B1[a][c], s1);
-            accumulate(acc[6], O::prod(e1, e1));
-            const V bb = O::prod(b1, b1);
+            O::add_prod(acc[6], e1, e1);
             if (a < 2) {
-                accumulate(acc[6], bb);
+                O::add_prod(acc[6], b1, b1);
             } else {
-                accumulate(acc[9], bb);
-                accumulate(acc[8], bb * T(q.x[0] + 1));
+                O::add_prod(acc[9], b1, b1);
+                O::add_square_times(acc[8], b1, q.x[0] + 1);
             }
             if (EM >> a & 1) {
                 const T e0 = s.E0[a][c];
-                accumulate(acc[5], O::prod(O::scaled(e0, s0), O::scaled(e0, s0)));
-                accumulate(acc[7], O::diff(O::scaled(e0, sx), -O::scaled(s.Eext[a], sx)) * e1);
+                O::add_prod(acc[5], O::scaled(e0, s0), O::scaled(e0, s0));
+                O::add_sum_times(acc[7], O::scaled(e0, sx), O::scaled(s.Eext[a], sx), e1);
             } else if (s.ext >> a & 1) {
-                accumulate(acc[7], O::prod(O::scaled(s.Eext[a], sx), e1));
+                O::add_prod(acc[7], O::scaled(s.Eext[a], sx), e1);
             }
             if (BM >> a & 1) {
                 const T b0 = s.B0[a][c];
-                accumulate(acc[5], O::prod(O::scaled(b0, s0), O::scaled(b0, s0)));
-                accumulate(acc[7], O::diff(O::scaled(b0, sx), -O::scaled(s.Bext[a], sx)) * b1);
+                O::add_prod(acc[5], O::scaled(b0, s0), O::scaled(b0, s0));
+                O::add_sum_times(acc[7], O::scaled(b0, sx), O::scaled(s.Bext[a], sx), b1);
             } else if (s.ext >> (3 + a) & 1) {
-                accumulate(acc[7], O::prod(O::scaled(s.Bext[a], sx), b1));
+                O::add_prod(acc[7], O::scaled(s.Bext[a], sx), b1);
             }
         }
     }
     // each thread's sums as doubles, the scales undone; then a fixed tree over the block
     const double up = 1.0 / ((double)sp * (double)sp), u0 = 1.0 / ((double)s0 * (double)s0);
-    const double u1 = 1.0 / ((double)s1 * (double)s1), ux = 1.0 / ((double)sx * (double)s1), ur = 1.0 / ((double)sr * (double)sr);
+    const double u1 = 1.0 / ((double)s1 * (double)s1), ux = 1.0 / ((double)sx * (double)s1);
     const double dV = s.d[0] * s.d[1] * s.d[2];
     double tot[8];
     tot[7] = 0.0;
@@ -293,14 +327,14 @@ __global__ void __launch_bounds__(kDiagThreads, sizeof(T) == 4 ? 3 : 4) k_diag_s
 #pragma unroll
     for (int a = 0; a < 3; a++)
         if (MASK >> a & 1) hphi += half * half * O::total(acc[2 + a]) / (s.d[a] * s.d[a]);
-    const double bz2 = O::total(acc[9]) * u1;
+    const double bz2 = O::total(acc[9]) * u1;  // (H_g1: both parts as one sum, rounded once)
     tot[0] = 0.5 * dV * up * hphi;
     tot[1] = 0.5 * dV * u0 * O::total(acc[5]);
-    tot[2] = 0.5 * dV * (u1 * O::total(acc[6]) + bz2);
+    tot[2] = 0.5 * dV * u1 * O::total(acc[6], acc[9]);
     tot[3] = dV * ux * O::total(acc[7]);
     tot[4] = dV * (s.lo0 * bz2 + s.d[0] * u1 * O::total(acc[8]));
     tot[5] = dV * bz2;
-    tot[6] = dV * ur * O::total(acc[10]);
+    tot[6] = dV * gauss;
     __shared__ double sh[8][kDiagThreads / 32];
     block_sums(tot, sh);
     if (threadIdx.x < kQ) {
@@ -557,6 +591,8 @@ static Sums<T> make_sums(axp_grid *g, const View<T> &v)
         s.Bext[a] = v.Bext[a];
         s.Eext[a] = v.Eext[a];
         s.d[a] = (double)v.d[a];
+        s.rd[a] = 1.0 / s.d[a];
+        s.kgb[a] = (sizeof(T) == 4 ? 0.5 : 0.25) * (double)v.g * (double)v.Bext[a];
         s.ext = (a ? s.ext : 0) | (v.Eext[a] != T(0) ? 1 << a : 0) | (v.Bext[a] != T(0) ? 8 << a : 0);
     }
     s.phi = v.phi_cur;
@@ -564,7 +600,7 @@ static Sums<T> make_sums(axp_grid *g, const View<T> &v)
     s.N = (unsigned)v.N;
     s.lo0 = (double)v.lo[0];
     s.dt = (double)v.dt;
-    s.g = (double)v.g;
+    s.kg = (sizeof(T) == 4 ? 0.5 : 0.25) * (double)v.g;
     s.m2 = (double)v.m2;
     s.top = sizeof(T) == 4 ? (unsigned *)(g->ws + g->layout.off_flag) + 8 : nullptr;
     s.partials = (double *)(g->ws + g->layout.off_partials);
@@ -666,8 +702,8 @@ cudaError_t diag_compute_rows(axp_grid *g, axp_diag *dev_dst, int axis, int64_t 
         g->launches++;
     }
     double *partials = s.partials;
-    // one wave of blocks (4 per SM; FP32: 3): a wave and a part of the next costs two
-    const int nb = wide ? g->layout.diag_blocks : std::min(g->layout.diag_blocks, 152 * (sizeof(T) == 4 ? 3 : 4));
+    // one wave of blocks: a wave and a part of the next costs two
+    const int nb = wide ? g->layout.diag_blocks : std::min(g->layout.diag_blocks, 152 * diag_blocks_per_sm<T>(g->desc.n[2] > 1 ? 7 : 3));
     if (wide) {
         PhiPair<T, sizeof(T) == 4> q{v.phi_cur, v.phi_b, ghosts_lvl<T>(g, 0), ghosts_lvl<T>(g, 1)};
         k_diag_partial<T, sizeof(T) == 4><<<nb, kDiagThreads, 0, g->stream>>>(v, q, partials);
