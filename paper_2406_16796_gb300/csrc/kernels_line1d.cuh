@@ -141,6 +141,9 @@ __device__ __forceinline__ bool grid_wait(unsigned *ctr, unsigned target, int *e
 template <typename T, bool LAYER>
 __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
 {
+    // (a plain launch may be set up while the kernel before it ends, and waits here for that
+    // kernel's memory)
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     constexpr bool INCR = sizeof(T) == 4;
     constexpr int LANES = lanes_of<T>();
     extern __shared__ __align__(16) unsigned char l1_raw[];
@@ -179,8 +182,6 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
     const int64_t wl = LAYER ? A.lay[0] - (s0 - H) : 0, wh = LAYER ? N - A.lay[1] - (s0 - H) : W;
     const bool layered = LAYER && (wl > 0 || wh < W);  // this window's body
     auto in_layer = [&](int w) { return LAYER && layered && (w < wl || w >= wh); };
-    // (a plain launch may be set up while the kernel before it ends; it waits here for that
-    // kernel's memory, of which the layer's tables are no part)
     if (LAYER && layered) {
         for (int w = tid; w < W; w += nt) {
             const int64_t gi = s0 - H + w;
@@ -207,11 +208,16 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
         }
     }
 
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     int par = 0;
     unsigned waits = 0;
+    // E1^{n+1} of a damped cell at the launch's last step, for a record: taken between the two
+    // half-steps (undoing the second would divide by 1 - sigma h/2, which may be zero)
+    auto keep = [&](int q, int w, T v) {
+        if (w >= H && w < H + own) A.En[q][s0 + (w - H)] = v;
+    };
     for (int64_t done = 0; done < A.nsteps; done += A.tblock) {
         const int steps = (int)min((int64_t)A.tblock, A.nsteps - done);
+        const int last = done + steps >= A.nsteps ? steps - 1 : -1;  // the launch's last step
         for (int w = tid; w < W; w += nt) {
             int64_t gi = s0 - H + w;
             const bool in = !LAYER || (gi >= 0 && gi < N);
@@ -237,6 +243,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
         }
         __syncthreads();
         for (int st = 0; st < (INCR ? 0 : steps); st++) {
+            const bool fin = LAYER && st == last;
             // 1. B^{n+1/2} and B^{n+1}: (curl E)_y = -D_x E_z, (curl E)_z = D_x E_y (forward)
             for (int w = lane; w < W; w += LANES) {
                 if (half == 0) {
@@ -330,8 +337,13 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
                         // two half-steps: a^2 E + (1 + a) r h X
                         const T a = La[w], r2 = T(0.5) * Lr[w];
                         const T xx = r2 * (-A.hgx * Jx), xy = r2 * fma(-A.c2B, dz, -A.h2g * PY[w]);
-                        E[3][w] = fma(a, fma(a, E[3][w], xx), xx);
-                        E[4][w] = fma(a, fma(a, E[4][w], xy), xy);
+                        const T mx = fma(a, E[3][w], xx), my = fma(a, E[4][w], xy);
+                        E[3][w] = fma(a, mx, xx);
+                        E[4][w] = fma(a, my, xy);
+                        if (fin) {
+                            keep(2, w, mx);
+                            keep(3, w, my);
+                        }
                     } else {
                         E[3][w] = fma(-A.hgx, Jx, E[3][w]);
                         E[4][w] = fma(-A.c2B, dz, fma(-A.h2g, PY[w], E[4][w]));
@@ -340,7 +352,9 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
                     const T dy = B[4][w] - at(B[4], w - 1);
                     if (in_layer(w)) {
                         const T a = La[w], xz = T(0.5) * Lr[w] * fma(A.c2B, dy, -A.h2g * PZ[w]);
-                        E[5][w] = fma(a, fma(a, E[5][w], xz), xz);
+                        const T mz = fma(a, E[5][w], xz);
+                        E[5][w] = fma(a, mz, xz);
+                        if (fin) keep(4, w, mz);
                         E[1][w] = fma(T(1) + a, Eny[w], -a * E[1][w]);
                         E[2][w] = fma(T(1) + a, Enz[w], -a * E[2][w]);
                     } else {
@@ -374,6 +388,7 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             return lay ? over(fma(A.h, X, La[w] * F), Ld[w], Lr[w]) : fma(A.h, X, F);
         };
         for (int st = 0; st < (INCR ? steps : 0); st++) {
+            const bool fin = LAYER && st == last;
             for (int w = lane; w < W; w += LANES) {
                 bool lay = in_layer(w);
                 if (lay && Ld[w] == T(0)) continue;
@@ -442,11 +457,18 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
                 if (half == 0) {
                     const T X = -A.g * (T(0.5) * (Px[w] + at(Px, w + 1)));
                     const T Y = fma(-A.g, PY[w], -((B[5][w] - at(B[5], w - 1)) * A.idx));
-                    E[3][w] = half_e(half_e(E[3][w], X, lay, w), X, lay, w);
-                    E[4][w] = half_e(half_e(E[4][w], Y, lay, w), Y, lay, w);
+                    const T mx = half_e(E[3][w], X, lay, w), my = half_e(E[4][w], Y, lay, w);
+                    E[3][w] = half_e(mx, X, lay, w);
+                    E[4][w] = half_e(my, Y, lay, w);
+                    if (lay && fin) {
+                        keep(2, w, mx);
+                        keep(3, w, my);
+                    }
                 } else {
                     const T Z = fma(-A.g, PZ[w], (B[4][w] - at(B[4], w - 1)) * A.idx);
-                    E[5][w] = half_e(half_e(E[5][w], Z, lay, w), Z, lay, w);
+                    const T mz = half_e(E[5][w], Z, lay, w);
+                    E[5][w] = half_e(mz, Z, lay, w);
+                    if (lay && fin) keep(4, w, mz);
                     E[1][w] = half_e(Eny[w], -((B[2][w] - at(B[2], w - 1)) * A.idx), lay, w);
                     E[2][w] = half_e(Enz[w], (B[1][w] - at(B[1], w - 1)) * A.idx, lay, w);
                 }
@@ -466,25 +488,18 @@ __global__ void __launch_bounds__(threads_of<T>()) k_line1d(Args<T> A)
             A.phi[1 - par][0][gi] = cur[w];
             A.phi[1 - par][1][gi] = inc[w];
             if (done + A.tblock >= A.nsteps) {
-                // E^{n+1} of the last step, for a record taken here: E1 less the second of
-                // its two half-steps, E0 as the step formed it
+                // E^{n+1} of the last step, for a record taken here: E0 as the step formed it,
+                // E1 less the second of its two half-steps (a damped cell's: kept above)
+                A.En[0][gi] = Eny[w];
+                A.En[1][gi] = Enz[w];
+                if constexpr (LAYER)
+                    if (in_layer(w) && !(INCR && Ld[w] == T(1))) continue;
                 const T Jx = T(0.5) * (Px[w] + at(Px, w + 1));
                 const T hx = T(-0.5) * A.h2g * Jx, hy = fma(-A.cB, B[5][w] - at(B[5], w - 1), T(-0.5) * A.h2g * PY[w]);
                 const T hz = fma(A.cB, B[4][w] - at(B[4], w - 1), T(-0.5) * A.h2g * PZ[w]);
-                const bool lay = in_layer(w);
-                T r = T(1), ia = T(1);
-                if (lay && INCR) {
-                    r = Lr[w];
-                    ia = Ld[w] / La[w];
-                } else if (lay) {
-                    r = Lr[w];
-                    ia = T(1) / La[w];
-                }
-                A.En[0][gi] = Eny[w];
-                A.En[1][gi] = Enz[w];
-                A.En[2][gi] = fma(-r, hx, E[3][w]) * ia;
-                A.En[3][gi] = fma(-r, hy, E[4][w]) * ia;
-                A.En[4][gi] = fma(-r, hz, E[5][w]) * ia;
+                A.En[2][gi] = E[3][w] - hx;
+                A.En[3][gi] = E[4][w] - hy;
+                A.En[4][gi] = E[5][w] - hz;
             }
         }
         par ^= 1;

@@ -112,3 +112,26 @@ def test_runs_of_one_window_and_of_several_mix():
         g.close()
     for k in NAMES:
         assert np.array_equal(out[0][k], out[1][k]) and np.array_equal(out[0][k], out[2][k]), k
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-10), ("fp32", 1e-4)])
+def test_record_beside_a_layer_that_stops_the_field(prec, tol):
+    """One layer cell with sigma dt = 4 (1 - sigma h / 2 = 0): the record's divergence next to it
+    takes E^n of that cell, which no half-step can be undone to."""
+    grid = line(300, "pml", prec, 1).replace(d=(1 / 16, 1 / 16, 1 / 16), dt=1 / 32, pml_sigma_max_dt=4.0, g=0.0)
+    st = W.random_state(grid, seed=44, active=LASER)
+    for k in ("phi_cur", "phi_old"):
+        st[k] = np.zeros_like(st[k])
+    from paper_2406_16796_gb300 import axp
+
+    g = axp.Grid(grid)
+    og = oracle.OracleGrid(grid.replace(precision="fp64"))
+    g.load(st)
+    og.load(st)
+    for n in (1, 30):
+        g.step(n)
+        og.step(n)
+        rec, ref = g.diagnostics(), og.diagnostics()
+        for key in ("H_g0", "H_g1", "gauss_l2", "sum_B1z2"):
+            assert abs(rec[key] - ref[key]) <= tol * abs(ref[key]), (key, n, rec[key], ref[key])
+    g.close()
