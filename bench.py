@@ -617,7 +617,7 @@ def boundary_measurement():
     out = {"workload": "bc_check_400x400", "paper_reflectivity": 0.01}
     for bc in ("pml", "outflow"):
         r = bccheck.reflectivity(bc, n=400)
-        out[bc] = {k: r[k] for k in ("energy", "amplitude", "steps", "seconds", "cell_updates_per_s", "kernel")}
+        out[bc] = {k: r[k] for k in ("energy", "amplitude", "steps", "seconds", "cell_updates_per_s", "kernel", "launches_per_step")}
     return out
 
 

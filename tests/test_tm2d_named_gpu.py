@@ -152,3 +152,10 @@ def test_fp32_1d_grids_around_the_line_between_kernels(nx, bc, one_launch):
     og.step(10)
     same(g, og, 1e-4)
     g.close()
+
+
+@pytest.mark.parametrize("bc,prec,per_step", [("outflow", "fp64", 4), ("pml", "fp64", 4), ("pml", "fp32", 1)])
+def test_boundary_benchmark_says_what_ran(bc, prec, per_step):
+    from paper_2406_16796_gb300 import bccheck
+
+    assert bccheck.reflectivity(bc, precision=prec, n=200, t_end=3.0)["launches_per_step"] == per_step
