@@ -433,8 +433,9 @@ axp_status axp_get_window_offset(const axp_grid *grid, int64_t *cells);
  * kernels' staggered scheme reduced to 1D, its curl updates folded into one
  * multiply-add per difference (within 1e-12 of the general path after 20000
  * steps), over windows held in shared memory for blocks of steps, in one
- * cooperative launch per run of steps; any split of a run into launches gives
- * the same bits.  Should one of its
+ * launch per run of steps (cooperative where the run is longer than a window's
+ * steps); any split of a run into launches gives the same bits.  It takes
+ * grids of up to 964 cells per SM (146,528 on 152 SMs).  Should one of its
  * bounded grid-wide waits give up, the next synchronising call on the handle
  * (axp_synchronize, diagnostics, reads, axp_save_state) returns
  * AXP_E_TIMEOUT.  Forcing a kernel that does not support the grid makes

@@ -34,14 +34,15 @@ constexpr int kQ = 7;  // H_phi, H_g0, H_g1, cross, sum x B1z^2, sum B1z^2, gaus
 //    a sum of doubles takes one per term.  The Gauss residual, a sum of scaled differences
 //    that cancel, is formed and squared in double, its floats widened by their bits: the FP64
 //    pipe is idle otherwise (the E1 and B1 sums there too: 512^3 6.5 -> 8.8 ms).
-//    Worst relative error of H_g0, H_g1 and sum_B1z2 against exact sums, 48 states of 300 to
+//    Worst relative error of H_g0, H_g1 and sum_B1z2 against exact sums, 52 states of 300 to
 //    2.1M cells: 3.2e-16 (literal doubles 2.5e-16; pairs of floats 2.4e-14).
 //  * Floats span less than squares of small fields need, so each group of fields is
 //    scaled by a power of two taken from its largest magnitude in the region (max_group:
 //    a pass of its own, or part of the pass that forms E^n).  Scaling by a power of
 //    two is exact; what then underflows is below 2^-60 of the largest value.
-// Measured, a whole record (us, against the literal doubles): 512^3 FP32 box 37000 -> 6540; 4096 x 2048
-// pulse FP32 1100 -> 530; FP64 unchanged at 1110 (50 operations per cell on the FP64 pipe).
+// Measured, a whole record while stepping (us, literal doubles before; cells of 0.05 x 0.07 x 0.06, a
+// background along every axis): 512^3 FP32 box 53600 -> 6540; 4096 x 2048 pulse FP32 3970 -> 530, FP64
+// 3840 -> 1080 (49 operations per cell on the FP64 pipe, 87% busy).  Pairs of floats took 6170 and 430.
 // ---------------------------------------------------------------------------
 struct FF {
     float h, l;

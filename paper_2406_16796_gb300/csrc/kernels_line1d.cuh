@@ -34,7 +34,8 @@
 //
 // FP32 split holds phi^{n+1/2} and its increment, and takes the generic single-pass kernel's
 // operations in their order (rounding differences of a few 1e-5 would come from any other
-// over a few hundred steps).  Its step is bound by the barriers' latency (about 0.55 us), not by a pipe,
+// over a few hundred steps): its bits where the cell size is a power of two (other sizes round
+// 1/dx once more) and no damped quotient is below 1e-30.  Its step is bound by the barriers' latency (about 0.55 us), not by a pipe,
 // so its windows are blocked over more steps (line_block).
 //
 // Measured, us per step (one launch per step before): 2048 cells with absorbing ends

@@ -6,7 +6,7 @@
 // per cycle per SM), so each quantity is formed once and every constant is folded;
 // an FP32 step by memory and launch latency.  The literal kernels
 // (kernels_general.cu) take 8 launches and several hundred FP64 operations per 3D cell
-// (their divisions included); these take 4 launches and about 170:
+// (their divisions included); these take 4 launches and 187:
 //   B      B^{n+1} of both orders; B0^{n+1/2} is kept in scratch
 //   phi    S and phi^{n+3/2}; E0^{n+1} (to scratch) and E0^{n+3/2}
 //   P      the axion current's P at the cell centres
@@ -29,7 +29,10 @@
 //   3D laser, absorbing x sides, FP64, 160 x 96 x 96        1922 -> 547
 //   2D laser polarised in the plane, FP32 split, 1024 x 512  130 -> 33
 //   2D TM laser, absorbing sides, FP64, 400 x 400            160 -> 42 (the 2D kernel)
-// ncu: the FP64 passes keep the FP64 pipe 76-84% busy while an SM is active.
+// ncu: the FP64 passes keep the FP64 pipe 73 to 84% busy while an SM is active on the two larger
+// grids (93 operations per cell of the 1024 x 512 one, 187 of the 3D one), 63 to 66% at 400 x 400,
+// where a pass is less than one wave of blocks
+// (profiles/k_stage_warp_line_records_counters.md).
 #include <algorithm>
 
 #include "cells.cuh"
@@ -408,9 +411,6 @@ __global__ void __launch_bounds__(kThreads) k_stage_p(Stage<T> s, const T *e0, c
     }
 }
 
-// J = (P(c) + P(c + a)) / 2 and the order-1 E update.  Beyond the
-// last cell of a non-periodic axis P follows the ghost rules: 0 at a PML side without
-// a uniform E, else evaluated in place (one cell per row or plane).
 // Inverse of a half-step: the field a half-step earlier, given h X.
 template <typename T, bool IN>
 __device__ __forceinline__ T half_back(const Layer<T, IN> &L, T F, T hX)
@@ -468,6 +468,9 @@ __device__ __forceinline__ void e1_update(const Stage<T> &s, const T J2[3], cons
         s.Eout[3 + a][q.c] = E;
     }
 }
+// J = (P(c) + P(c + a)) / 2 and the order-1 E update.  Beyond the
+// last cell of a non-periodic axis P follows the ghost rules: 0 at a PML side without
+// a uniform E, else evaluated in place (one cell per row or plane).
 // WHAT 0: the step's update; 1: J alone, into its cache; 2: J and E1^n from E1^{n+1/2}
 template <typename T, int MASK, int WHAT>
 __global__ void __launch_bounds__(kThreads) k_stage_j(Stage<T> s, View<T> v, PhiPair<T, sizeof(T) == 4> pq)
