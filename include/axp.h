@@ -362,8 +362,9 @@ axp_status axp_load_state(axp_grid *grid, const void *host_src, size_t bytes);
  * kernels) must be the same on both sides: slabs that exchange rows take the
  * same kernel path and the same steps.  Rows may bring order-0 components that
  * were never injected or written here: records, conversions and the multi-pass
- * step then take all of them; a single-pass kernel takes those of the set it
- * was chosen for (the 2D TM kernel: E0z, B0x, B0y).  AXP_E_INVAL for rows outside the
+ * step then take all of them, and so does AUTO's generic kernel in 1D and 2D; a
+ * specialised kernel takes those of its set (the 2D TM kernel: E0z, B0x, B0y;
+ * the 3D axion box: none).  AXP_E_INVAL for rows outside the
  * grid; AXP_E_STATE for a grid with macroparticles (they do not move between
  * slabs).
  *
@@ -407,8 +408,9 @@ axp_status axp_get_window_offset(const axp_grid *grid, int64_t *cells);
  * single-pass kernel that supports the grid's shape, boundaries and active
  * field components, else multi-pass kernels with folded arithmetic (within
  * 1e-12 of the literal ones in FP64; reported as AXP_KERNEL_GENERAL).  The same
- * passes step the staggered state of the generic kernel's 2D and 3D grids and of
- * the 2D TM kernel's small FP64 grids, where they are faster; the path reported
+ * passes step the staggered state of the generic kernel's 2D and 3D grids (in FP32
+ * not the large 2D ones) and of the 2D TM kernel's small FP64 grids, where they are
+ * faster; the path reported
  * is then still that kernel's, whose state it is.  Likewise 1D grids in FP32 split
  * or with absorbing ends run on the time-blocked 1D kernel and report the generic one.
  * AXP_KERNEL_GENERAL forces the general kernels (one pass per stage of the

@@ -912,6 +912,44 @@ cudaError_t step_graph(axp_grid *g, Launch &&launch_one, cudaGraphExec_t *out)
 // 400 x 400 42 / 107, 1024 x 512 103 / 142, 800 x 800 126 / 142, 1024 x 768 150 / 142.
 constexpr int64_t kSmallTm = 700000;
 
+// Whether a 2D FP32 grid of the generic kernel is faster on it than on the folded passes.  The
+// passes read and write the state four times, which shows once it leaves L2; the generic
+// kernel marches strips of 251 columns whose edge body, at a non-periodic x side, holds
+// up a whole strip, and pays a floor on small grids.  Estimates in us, c and p the cells in millions without
+// and with the last strip's padding, fitted to 203 grids of 0.13M to 8.4M cells (it picks
+// the slower one on three of them, by 2 to 7%):
+//   passes: 4 + 43 c (no order-0 field), 2 + 55 c (a TM or TE laser), 2 + 70 c (all components)
+//   generic, x periodic: 14 + 17 p, 14 + 24.5 p, 8 + 48 p, at least 42, 44, 40; a layer along y 30 (37), a
+//   reflecting y side 6 more; no order-0 field and another x side: 5 + 29 p (37 p with layers
+//   along x, 34.5 p along y); with a laser the passes at once.
+// us per step, passes / generic: TE periodic 768 x 768 34.7 / 41.5, 1024 x 1024 59.4 / 45.5, 4096 x 2048
+// 462 / 240; all periodic 1024 x 512 37 / 39, 4096 x 2048 574 / 419; no laser, reflecting
+// 1024 x 1024 52 / 62, 4096 x 2048 363 / 255; TE with layers 4096 x 2048 465 / 662.
+bool generic_2d_is_faster(const axp_grid *g, int set)
+{
+    const axp_grid_desc &d = g->desc;
+    constexpr int VX = fused::Tile<float, 2>::VX;
+    auto side = [&](int a) {  // 0: periodic, 1: reflecting, 2: a layer at either end
+        if (d.em_bc[a][0] == AXP_BC_PERIODIC) return 0;
+        for (int s = 0; s < 2; s++)
+            if (d.em_bc[a][s] == AXP_BC_PML || d.axion_bc[a][s] == AXP_BC_PML) return 2;
+        return 1;
+    };
+    const int kind = set == 0 ? 0 : (set == 3 ? 2 : 1), x = side(0), y = side(1);
+    const double c = 1e-6 * (double)d.n[0] * (double)d.n[1];
+    const double p = 1e-6 * (double)((d.n[0] + VX - 1) / VX * VX) * (double)d.n[1];
+    const double passes = (kind == 0 ? 4.0 : 2.0) + (kind == 0 ? 43.0 : kind == 1 ? 55.0 : 70.0) * c;
+    double generic;
+    if (x == 0) {
+        generic = kind == 0 ? std::max(42.0, 14.0 + 17.0 * p) : kind == 1 ? std::max(44.0, 14.0 + 24.5 * p) : std::max(40.0, 8.0 + 48.0 * p);
+        generic += y == 0 ? 0.0 : y == 1 ? 6.0 : (kind == 2 ? 37.0 : 30.0);
+    } else {
+        if (kind != 0) return false;
+        generic = x == 2 ? std::max(77.0, 5.0 + 37.0 * p) : y == 2 ? std::max(72.0, 5.0 + 34.5 * p) : std::max(60.0, 5.0 + 29.0 * p);
+    }
+    return generic < passes;
+}
+
 // FP32 grids of the 2D kernel up to this many cells take the warp tiles: they split a small
 // or ragged grid more evenly.  Beyond it the state no longer fits L2, and the block tiles'
 // longer rows are the better HBM access.  us per step, block / warp tiles: 512 x 256 15.6 / 14.5,
@@ -968,16 +1006,19 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     }
     const bool tm = path == AXP_KERNEL_TM2D || path == AXP_KERNEL_TM2D_LIST, ax = path == AXP_KERNEL_AX3D;
     const int mode = grid_mode(g);
-    const int set = pick_set(g);
+    // (rows of another grid may hold any component: the generic kernel then takes all of them)
+    const int set = g->kernel_choice == AXP_KERNEL_AUTO && path == AXP_KERNEL_FUSED && mode <= 2 && g->rows_in ? 3 : pick_set(g);
     cudaError_t e = enter_staggered<T>(g);
     if (e != cudaSuccess) return e;
     // AUTO runs the folded passes on the same staggered state where they are faster: in
-    // place of the generic kernel in 2D and 3D, and on small FP64 grids of the 2D kernel
+    // place of the generic kernel in 2D and 3D (FP32 2D: by the estimate above), and on
+    // small FP64 grids of the 2D kernel
     const bool small_tm = tm && sizeof(T) == 8 && g->desc.n[0] * g->desc.n[1] <= kSmallTm;
     g->en_scratch = false;
     // (after rows of another grid have arrived, the whole set of the kernel they stand for:
     // a slab without a laser takes its neighbour's)
-    if (g->kernel_choice == AXP_KERNEL_AUTO && (small_tm || (path == AXP_KERNEL_FUSED && mode >= 2)) && staged_supported(g))
+    const bool for_generic = path == AXP_KERNEL_FUSED && mode >= 2 && !(sizeof(T) == 4 && mode == 2 && generic_2d_is_faster(g, set));
+    if (g->kernel_choice == AXP_KERNEL_AUTO && (small_tm || for_generic) && staged_supported(g))
         return staged_step<T>(g, nsteps, small_tm && g->rows_in ? kSets[1] : order0_present(g));
     int tm_tx = tm2d::TX;  // tile width of the 2D kernel (chosen below)
     // FP32 split on an even-width grid without a soft source: the two-column form

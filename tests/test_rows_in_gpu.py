@@ -21,6 +21,8 @@ GRIDS = {
     "2d_uniform_e": dict(n=(40, 31, 1), B=(0.2, 0.9, 0.3), E=(0.3, 0.1, -0.2)),
     "2d_reflect": dict(n=(45, 29, 1), B=(0.2, 0.9, 0.3), ax=bcs("reflect", "pml"), em=bcs("reflect", "pml"), E=(0.1, 0.0, 0.0)),
     "3d_uniform_e": dict(n=(19, 11, 7), B=(0.2, 0.9, 0.3), E=(0.3, 0.1, -0.2)),
+    "2d_generic": dict(n=(1255, 800, 1), B=(0.2, 0.9, 0.3), ax=bcs("periodic", "reflect"), em=bcs("periodic", "reflect")),
+    "1d_generic": dict(n=(300, 1, 1), B=(0.2, 0.9, 0.3), ax=bcs("reflect"), em=bcs("reflect")),
     "1d_uniform_e": dict(n=(300, 1, 1), B=(0.2, 0.9, 0.3), E=(0.3, 0.1, -0.2)),
 }
 
