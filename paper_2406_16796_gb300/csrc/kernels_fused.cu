@@ -906,11 +906,30 @@ cudaError_t step_graph(axp_grid *g, Launch &&launch_one, cudaGraphExec_t *out)
     return cudaSuccess;
 }
 
-// FP64 grids of the 2D kernel up to this many cells take the folded passes: a block of
-// the 2D kernel marches at least 14 planes through one SM's FP64 units, which leaves a
-// small grid's step a serial chain.  us per step, passes / 2D kernel: 96 x 64 15 / 47,
-// 400 x 400 42 / 107, 1024 x 512 103 / 142, 800 x 800 126 / 142, 1024 x 768 150 / 142.
+// Whether a FP64 grid of the 2D kernel is faster on the folded passes: a block of the 2D kernel
+// marches at least 14 planes through one SM's FP64 units, which leaves a small grid's step a
+// serial chain, most of all where the march crosses absorbing layers.  With layers on every
+// side: up to 700,000 cells (us per step, passes / 2D kernel: 96 x 64 15 / 47, 400 x 400 42 / 107,
+// 1024 x 512 103 / 142, 800 x 800 126 / 142, 1024 x 768 150 / 142).  With a periodic axis below that by
+// estimates in us, c and p the cells in millions without and with the last strip's padding,
+// fitted to 232 grids (it picks the slower one by more than 3% on two of them):
+//   passes 6 + 170 c, 8 + 173 c with layers along y, 10 + 171 c and 0.0012 ny along x;
+//   2D kernel 30 + 105 p, 2500 / ny with layers along y, 8 + 0.03 ny along x
+// (both axes periodic: 512 x 512 53 / 62, 700 x 700 91 / 82, 836 x 836 125 / 107; layers along x: 800 x 800
+// 122 / 131, 4096 x 160 120 / 107; along y: 300 x 1000 61 / 83, 836 x 836 128 / 109).
 constexpr int64_t kSmallTm = 700000;
+bool small_tm_by_passes(const axp_grid *g)
+{
+    const axp_grid_desc &d = g->desc;
+    const double nx = (double)d.n[0], ny = (double)d.n[1], c = 1e-6 * nx * ny;
+    if (d.n[0] * d.n[1] > kSmallTm) return false;
+    const bool lx = d.em_bc[0][0] != AXP_BC_PERIODIC, ly = d.em_bc[1][0] != AXP_BC_PERIODIC;
+    if (lx && ly) return true;
+    constexpr int VX = 128 - tm2d::HL - tm2d::HR;  // (written columns of the tiles it takes here)
+    const double p = 1e-6 * (double)((d.n[0] + VX - 1) / VX * VX) * ny;
+    const double passes = lx ? 10.0 + 171.0 * c + 0.0012 * ny : ly ? 8.0 + 173.0 * c : 6.0 + 170.0 * c;
+    return passes <= 30.0 + 105.0 * p + (lx ? 8.0 + 0.03 * ny : ly ? 2500.0 / ny : 0.0);
+}
 
 // Whether a 2D FP32 grid of the generic kernel is faster on it than on the folded passes.  The
 // passes read and write the state four times, which shows once it leaves L2; the generic
@@ -1013,7 +1032,7 @@ cudaError_t fused_step(axp_grid *g, int64_t nsteps, bool *handled)
     // AUTO runs the folded passes on the same staggered state where they are faster: in
     // place of the generic kernel in 2D and 3D (FP32 2D: by the estimate above), and on
     // small FP64 grids of the 2D kernel
-    const bool small_tm = tm && sizeof(T) == 8 && g->desc.n[0] * g->desc.n[1] <= kSmallTm;
+    const bool small_tm = tm && sizeof(T) == 8 && small_tm_by_passes(g);
     g->en_scratch = false;
     // (after rows of another grid have arrived, the whole set of the kernel they stand for:
     // a slab without a laser takes its neighbour's)

@@ -118,13 +118,21 @@ def test_odd_step_counts_and_tiny_grids(n, bc, steps):
     g.close()
 
 
-@pytest.mark.parametrize("n,per_step", [((836, 836, 1), 4), ((838, 836, 1), 1), ((70, 10001, 1), 1), ((70, 9999, 1), 4)])
-def test_fp64_grids_around_the_line_between_passes_and_kernel(n, per_step):
-    """AUTO: the folded passes up to 700,000 cells, the 2D kernel above."""
+LINES = [((836, 836, 1), ("pml", "pml"), 4), ((838, 836, 1), ("pml", "pml"), 1), ((70, 10001, 1), ("pml", "pml"), 1),
+         ((70, 9999, 1), ("pml", "pml"), 4), ((512, 512, 1), ("periodic", "periodic"), 4), ((700, 700, 1), ("periodic", "periodic"), 1),
+         ((2048, 340, 1), ("pml", "periodic"), 1), ((512, 1024, 1), ("pml", "periodic"), 4), ((836, 836, 1), ("periodic", "pml"), 1),
+         ((300, 1000, 1), ("periodic", "pml"), 4)]
+
+
+@pytest.mark.parametrize("n,bc,per_step", LINES)
+def test_fp64_grids_around_the_line_between_passes_and_kernel(n, bc, per_step):
+    """AUTO: the folded passes up to 700,000 cells with layers on every side, and up to where the
+    2D kernel is the faster one with a periodic axis."""
     from paper_2406_16796_gb300 import axp
 
-    b = W._bcs("pml", "pml")
-    grid = W.GridSpec(n=n, d=(0.05, 0.05, 0.05), dt=0.03, m=1.1, g=0.7, B_ext=(0.0, 0.2, 1.0), axion_bc=b, em_bc=b, pml_cells=6)
+    b = W._bcs(*bc)
+    grid = W.GridSpec(n=n, d=(0.05, 0.05, 0.05), dt=0.03, m=1.1, g=0.7, B_ext=(0.0, 0.2, 1.0), axion_bc=b, em_bc=b,
+                      pml_cells=6 if "pml" in bc else 0)
     st = W.random_state(grid, seed=9, active=TM)
     g, og = axp.Grid(grid), oracle.OracleGrid(grid)
     g.load(st)
@@ -159,3 +167,30 @@ def test_boundary_benchmark_says_what_ran(bc, prec, per_step):
     from paper_2406_16796_gb300 import bccheck
 
     assert bccheck.reflectivity(bc, precision=prec, n=200, t_end=3.0)["launches_per_step"] == per_step
+
+
+@pytest.mark.parametrize("n,bc", [((836, 836, 1), ("periodic", "periodic")), ((1300, 530, 1), ("periodic", "pml")),
+                                  ((4096, 160, 1), ("pml", "periodic")), ((400, 400, 1), ("pml", "pml"))])
+def test_auto_is_not_slower_than_the_named_kernel(n, bc):
+    import time
+
+    from paper_2406_16796_gb300 import axp
+
+    b = W._bcs(*bc)
+    t = []
+    for kernel in (axp.AXP_KERNEL_AUTO, axp.AXP_KERNEL_TM2D):
+        g = axp.Grid(W.GridSpec(n=n, d=(0.05, 0.05, 0.05), dt=0.03, m=1.1, g=0.7, B_ext=(0.0, 0.2, 1.0), axion_bc=b, em_bc=b,
+                                pml_cells=6 if "pml" in bc else 0))
+        g.set_kernel(kernel)
+        g.write("E0z", np.full(g.shape, 1e-3))
+        g.step(10)
+        best = 1e9
+        for _ in range(5):
+            g.synchronize()
+            t0 = time.perf_counter()
+            g.step(20)
+            g.synchronize()
+            best = min(best, time.perf_counter() - t0)
+        t.append(best)
+        g.close()
+    assert t[0] < 1.06 * t[1], t
