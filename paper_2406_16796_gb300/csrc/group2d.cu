@@ -8,7 +8,8 @@
 // kernels_tm2d_x2.cuh): each warp of a resident grid takes tiles for itself, so members of
 // any width and height fill the chip evenly (16 uneven members of the serving stream, 6.5M
 // cells: 172 us per step with tiles of 250 x 64 cells per block, 136 now).
-// Members of odd width run as one-column tiles per block, in a launch of their own.  Whoever
+// Members of odd width run as one-column tiles per block; a group of both kinds runs in one
+// launch whose blocks take odd members' tiles first, then warp tiles.  Whoever
 // finishes the last tile of a member in a launch advances that member's step counter; the
 // last to leave rewinds the queue.  A member's buffer roles alternate with
 // period two, so each member carries the kernel parameters of both parities
@@ -86,12 +87,12 @@ constexpr size_t kGroupStage = tm2d_x2::stage_bytes(kGroupThreads);
 __host__ __device__ inline int group_vx(int64_t nx) { return nx % 2 == 0 ? kVxPair : kVxOne; }
 
 constexpr size_t kOddStage = tm2d::stage_bytes<float>(kGroupThreads);
+constexpr size_t kMixedStage = kOddStage > kGroupStage ? kOddStage : kGroupStage;
 
 // members of odd width: one tile per block at a time
-__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group_odd(GDev D)
+__device__ __forceinline__ void odd_members(const GDev &D, unsigned char *group_dyn)
 {
     __shared__ float rows[2][tm2d::NROWS][tm2d::RS];
-    extern __shared__ __align__(16) unsigned char group_dyn[];
     __shared__ fused::Params<float> sP;
     __shared__ int s_item;
     __shared__ long long s_done;
@@ -137,12 +138,11 @@ __global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group_odd(GDev D)
 
 // members of even width: each warp takes warp tiles for itself.  No block-wide barrier is
 // met inside the loop, and no warp waits for another.
-__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group(GDev D)
+__device__ __forceinline__ void even_members(const GDev &D, unsigned char *group_dyn)
 {
     constexpr int kWarps = kGroupThreads / 32;
     __shared__ __align__(16) float yring[kWarps][tm2d_x2::YR][tm2d_x2::NY + 1];
     __shared__ fused::Params<float> sP[kWarps];
-    extern __shared__ __align__(16) unsigned char group_dyn[];
     const int w = (int)(threadIdx.x / 32), lane = (int)(threadIdx.x % 32);
     constexpr int kWords = sizeof(fused::Params<float>) / sizeof(int);
     static_assert(sizeof(fused::Params<float>) % sizeof(int) == 0, "Params copied as words");
@@ -186,6 +186,26 @@ __global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group(GDev D)
     }
 }
 
+__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group(GDev D)
+{
+    extern __shared__ __align__(16) unsigned char group_dyn[];
+    even_members(D, group_dyn);
+}
+__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group_odd(GDev D)
+{
+    extern __shared__ __align__(16) unsigned char group_dyn[];
+    odd_members(D, group_dyn);
+}
+// Groups of both kinds: two launches one after the other leave the chip idle twice (8 members of
+// 128 x 64 and 8 of 127 x 63: 123 us per step, in one launch 87; 4 of 1024 x 512 and 4 of 1023 x 511: 160, 150;
+// 7 and 1: 191, 131).
+__global__ void __launch_bounds__(kGroupThreads, 2) k_tm2d_group_mixed(GDev D)
+{
+    extern __shared__ __align__(16) unsigned char group_dyn[];
+    odd_members(D, group_dyn);
+    even_members(D, group_dyn);
+}
+
 axp_status cuda_st(cudaError_t e)
 {
     if (e == cudaSuccess) return AXP_OK;
@@ -214,7 +234,7 @@ struct axp_group {
     int32_t chunk;  // y planes per tile
     bool chunk_given;  // by axp_group_set_chunk; else warp tiles take the planes that fill the chip best
     bool dirty;
-    int grid_blocks, odd_blocks;  // resident blocks of the two kernels
+    int grid_blocks, odd_blocks, mixed_blocks;  // resident blocks of the kernels
     int64_t launches;
     bool use_graph;
     cudaGraphExec_t graph;
@@ -239,11 +259,17 @@ int32_t tiles_of(const axp_grid *g, int32_t chunk)
 }
 
 // Planes per warp tile: the fewest waves of resident warps times rows + 6 planes of
-// pipeline, over all members.
+// pipeline, over all members.  Blocks that hold an odd member's tile are left out while they are
+// a quarter or less (7 members of 1024 x 512 and one of 1023 x 511: 169 us per step with them, 131
+// without; 4 and 4, more than half the blocks: 150 with, 180 without).
 int32_t warp_rows(const axp_group *G)
 {
     if (G->chunk_given) return G->chunk;
-    const int64_t slots = (int64_t)G->grid_blocks * (kGroupThreads / 32);
+    int64_t odd = 0;
+    for (const auto &M : G->members)
+        if (M.active && M.g->desc.n[0] % 2 != 0) odd += tiles_of(M.g, G->chunk);
+    const int64_t blocks = odd == 0 ? G->grid_blocks : G->mixed_blocks - (odd <= G->mixed_blocks / 4 ? odd : 0);
+    const int64_t slots = blocks * (kGroupThreads / 32);
     int32_t best = 64;
     double best_cost = 0.0;
     for (int32_t rows = 16; rows <= 512; rows++) {
@@ -306,15 +332,14 @@ axp_status rebuild(axp_group *G)
 cudaError_t enqueue(axp_group *G, int64_t nsteps)
 {
     for (int64_t s = 0; s < nsteps; s++) {
-        if (G->D.nwarp > 0) {
-            const int most = (G->D.nwarp + kGroupThreads / 32 - 1) / (kGroupThreads / 32);
-            k_tm2d_group<<<std::min(G->grid_blocks, most), kGroupThreads, kGroupStage, G->stream>>>(G->D);
-            G->launches++;
-        }
-        if (G->D.nitems > 0) {
-            k_tm2d_group_odd<<<std::min(G->odd_blocks, G->D.nitems), kGroupThreads, kOddStage, G->stream>>>(G->D);
-            G->launches++;
-        }
+        const int64_t most = (G->D.nwarp + kGroupThreads / 32 - 1) / (kGroupThreads / 32), odd = G->D.nitems;
+        if (odd == 0)
+            k_tm2d_group<<<(unsigned)std::min<int64_t>(G->grid_blocks, most), kGroupThreads, kGroupStage, G->stream>>>(G->D);
+        else if (most == 0)
+            k_tm2d_group_odd<<<(unsigned)std::min<int64_t>(G->odd_blocks, odd), kGroupThreads, kOddStage, G->stream>>>(G->D);
+        else
+            k_tm2d_group_mixed<<<(unsigned)std::min<int64_t>(G->mixed_blocks, most + odd), kGroupThreads, kMixedStage, G->stream>>>(G->D);
+        G->launches++;
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
@@ -381,6 +406,11 @@ axp_status axp_group_create(int32_t max_grids, int32_t max_tiles, void *dev_work
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tm2d_group_odd, kGroupThreads, kOddStage);
     G->odd_blocks = sms * std::max(1, occ);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tm2d_group_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMixedStage);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_tm2d_group_mixed, kGroupThreads, kMixedStage);
+    G->mixed_blocks = sms * std::max(1, occ);
     if (e == cudaSuccess) e = cudaMemsetAsync(G->ws, 0, L.total, G->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(G->stream);
     if (e != cudaSuccess) {
@@ -540,7 +570,7 @@ axp_status axp_group_run(axp_group *G, int64_t nsteps)
         }
         G->graph_steps = nsteps;
     }
-    G->launches += nsteps * ((G->D.nwarp > 0) + (G->D.nitems > 0));
+    G->launches += nsteps;
     return cuda_st(cudaGraphLaunch(G->graph, G->stream));
 }
 
